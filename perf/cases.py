@@ -72,9 +72,9 @@ def listed():
         # the multiscale cadence: molecules every 40th field step
         _case("cadence40", (128, 128, 192), 50000, "128/4", 80, geometry="ring", substeps=40, preroll=40),
         # frozen two-level molecules, a field-bound run on a grid larger than L2
-        _case("frozen", (256, 256, 128), 300000, "1/0", 48, geometry="ring", model="bloch"),
+        _case("frozen", (256, 256, 128), 200000, "1/0", 120, geometry="ring", model="bloch"),
         # no molecules: transmission and reflection spectra of the bare structure
-        _case("spectra", (128, 128, 192), 0, "64/1", 96, geometry="ring", planes=2, nfreq=48, fields=True),
+        _case("spectra", (128, 128, 192), 0, "64/1", 240, geometry="ring", planes=2, nfreq=48, fields=True),
         # molecules alone under a prescribed field, transition dipole d(R), absorber inside the packet
         _case("prescribed_dr", (16, 16, 64), 20000, "128/3", 8, drive="prescribed", d_of_r=True, absorber=2.5),
     ]
@@ -101,7 +101,7 @@ def draw(rng):
         n = 1
         while kind == "mixture" and n < 2:
             n = rng.randint(2, 3)
-        top = {"run": (0, 4), "wide": (5, 8), "wider": (9, 16), "parity": (1, 12), "mixed": (1, 8), "mixture": (0, 10)}[kind]
+        top = {"run": (1, 4), "wide": (5, 8), "wider": (9, 16), "parity": (1, 12), "mixed": (1, 8), "mixture": (1, 10)}[kind]
         rs = [64, 128] if kind == "mixed" else [64, 128, 256]
         sp = [(rng.choice(rs), rng.randint(*top)) for _ in range(n)]
         nsim = 1 if rng.random() < 0.7 else rng.randint(2, 5)
@@ -112,15 +112,15 @@ def draw(rng):
                      precision="mixed" if kind == "mixed" else "fp32")
     if kind == "cadence":
         sub = rng.choice([2, 5, 10, 20, 40])
-        sp = [(rng.choice([64, 128]), rng.randint(0, 8))]
+        sp = [(rng.choice([64, 128]), rng.randint(1, 8))]
         return _case(None, grid, mols(sp, 30000), "%d/%d" % sp[0], 2 * sub, geometry=geometry, substeps=sub, preroll=sub)
     if kind == "frozen":
-        return _case(None, grid, span(64, 300000), "1/0", rng.randint(8, 48), geometry=geometry, model="bloch",
+        return _case(None, grid, span(64, 300000), "1/0", rng.randint(16, 120), geometry=geometry, model="bloch",
                      substeps=rng.choice([1, 1, 4]))
     if kind == "spectra":
-        return _case(None, grid, 0, "64/1", rng.randint(16, 96), geometry=geometry, planes=rng.randint(1, 4),
+        return _case(None, grid, 0, "64/1", rng.randint(40, 240), geometry=geometry, planes=rng.randint(1, 4),
                      nfreq=span(1, 32), fields=rng.random() < 0.5)
-    sp = [(rng.choice([64, 128]), rng.randint(0, 4))]
+    sp = [(rng.choice([64, 128]), rng.randint(1, 4))]
     dr = rng.random() < 0.5
     return _case(None, (16, 16, 64), mols(sp, 40000), "%d/%d" % sp[0], steps, drive="prescribed", d_of_r=dr,
                  absorber=rng.choice([8.5, 2.5]))
@@ -267,7 +267,7 @@ def run(state):
         out["P_g"], out["P_e"] = P[:, 0].astype(np.float32), P[:, 1].astype(np.float32)
         out["mu"] = sim.dipoles().astype(np.float32)
         if absorbed is not None:  # a loop over single steps does not look at these
-            out["norm"] = (P.sum(axis=1) + absorbed.sum(axis=1)).astype(np.float32)
+            out["norm"] = (P[:, 0] + P[:, 1] + (absorbed[:, 0] + absorbed[:, 1])).astype(np.float32)
             out["R_e"] = Re.astype(np.float32)
             if case["absorber"] < 8.0:
                 out["absorbed"] = absorbed.astype(np.float32)
