@@ -86,7 +86,10 @@ enum { MS_FIELD_E = 0, MS_FIELD_H = 1 };
  * form. */
 enum { MS_MOL_AUTO = 0, MS_MOL_FUSED = 1, MS_MOL_STREAMING = 2 };
 /* Stored rows of each molecule's state.  MS_STATE_FULL: both surfaces carry
- * every channel (j, m), j <= J.  MS_STATE_PARITY: only (ground, even j) and
+ * every channel (j, m), j <= J; the point-resident kernels and, from J = 5 on,
+ * the static rule's kernels leave the rows that the j = 0 start cannot reach
+ * (zeros before and after every step) unread, and process every row of a state
+ * loaded with any of them populated.  MS_STATE_PARITY: only (ground, even j) and
  * (excited, odd j), the only rows the dynamics populate from the j = 0
  * ground-state start (each coupling changes j by one and swaps the
  * surfaces), which halves the state and the work.  Results are those of the

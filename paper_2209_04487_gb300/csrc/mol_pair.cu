@@ -173,8 +173,8 @@ __global__ void __launch_bounds__(Rs2Dims<J, TILE, PAR>::NT, Rs2Dims<J, TILE, PA
 #pragma unroll
     for (int k = 0; k < D::NBOX; ++k) {
       const bool last = k == D::NBOX - 1 && D::NBOX > 1;
-      tensor2d_g2s(base + D::O_STG + k * D::BOXR * SEG, last ? &maps.s_r : &maps.s, r0, mol * ROWS + k * D::BOXR,
-                   &s_bar[0]);
+      tensor2d_g2s(base + D::O_STG + k * D::BOXR * SEG, last ? &maps.s_r : &maps.s, r0,
+                   mol * sp.mrows + k * D::BOXR, &s_bar[0]);
       tensor2d_g2s(base + D::O_STG + (D::RP + k * D::BOXR) * SEG, last ? &maps.d2_r : &maps.d2, r0,
                    mol * ROWS + k * D::BOXR, &s_bar[0]);
     }
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(Rs2Dims<J, TILE, PAR>::NT, Rs2Dims<J, TILE, PA
     float2 sx[RPW], sy[RPW];  // the series sum S, pair layout
     float2 pg_hi = make_float2(0.f, 0.f), pg_lo = pg_hi, pe_hi = pg_hi, pe_lo = pg_hi;  // populations
     float2 a_g = pg_hi, a_e = pg_hi, aS = pg_hi, aZ = pg_hi, aD = pg_hi, rnd = pg_hi;
-    float2* gs = sp.psi + (long long)lm * ROWS * NR;
+    float2* gs = sp.psi + (long long)lm * sp.mrows * NR;
 
     // R_n = M R_{n-1} from term buffer P, added to S with weight (ka, kb):
     // odd n (P = 0): S += i k R, ka = -k, kb = k; even n (P = 1): S += k R, kb = k

@@ -384,18 +384,9 @@ ms_status build_species(ms_sim* s, int si, const ms_species& d, double dt, const
   sp.jmax = J;
   sp.nrot = nrot;
   sp.nmol = (int)ids.size();
-  sp.par = par ? 1 : 0;
-  if (par) {  // ground rows: channels of even j; excited rows: odd j
-    sp.rows_g = 0;
-    sp.rows = 0;
-    for (int j = 0; j <= J; ++j) {
-      sp.rows += 2 * j + 1;
-      if (j % 2 == 0) sp.rows_g += 2 * j + 1;
-    }
-  } else {
-    sp.rows_g = nrot;
-    sp.rows = 2 * nrot;
-  }
+  sp.par_form = par ? 1 : 0;
+  sp.all_rows = 0;
+  sp.mrows = par ? nrot : 2 * nrot;
   sp.mixed = mixed ? 1 : 0;
   sp.kpl = nullptr;
   const double dR = (d.rmax - d.rmin) / (nr - 1);
@@ -414,6 +405,7 @@ ms_status build_species(ms_sim* s, int si, const ms_species& d, double dt, const
     sp.theta = dmax * dtau;
     MS_TRY(upload(s, (float**)&sp.dipw, w.data(), w.size()));
   }
+  ms::mol_set_rows(sp, ms::mol_reachable_rows(sp));
   std::vector<double> r(nr), Ug(nr), Ue(nr);
   for (int i = 0; i < nr; ++i) {
     r[i] = d.rmin + i * dR;
@@ -474,7 +466,7 @@ ms_status build_species(ms_sim* s, int si, const ms_species& d, double dt, const
     }
     phi0[a] = acc / (double)nr;
   }
-  const size_t per = (size_t)sp.rows * nr;
+  const size_t per = (size_t)sp.mrows * nr;  // row 0 is (ground, j = 0) in either order of the rows
   std::vector<float2> row0(nr);
   for (int a = 0; a < nr; ++a) row0[a] = make_float2((float)phi0[a].real(), (float)phi0[a].imag());
   MS_TRY(zeros(s, &sp.psi, per * ids.size()));
@@ -521,8 +513,49 @@ ms_status build_species(ms_sim* s, int si, const ms_species& d, double dt, const
 // A plan switch to the streaming layout needs the (T - 1)s scratch.
 ms_status ensure_scratch(ms_sim* s, ms::SpeciesDev& sp) {
   if (sp.d2 || sp.nmol == 0) return MS_OK;
-  return zeros(s, &sp.d2, (size_t)sp.nmol * sp.rows * sp.nr);
+  return zeros(s, &sp.d2, (size_t)sp.nmol * sp.mrows * sp.nr);
 }
+
+// Brings a full-form species' rows into the order that its plan's kernels
+// process (on the handle's stream).
+ms_status order_rows(ms_sim* s, ms::SpeciesDev& sp) {
+  if (sp.bloch || sp.par_form) return MS_OK;
+  const bool want = ms::mol_reachable_rows(sp);
+  if (want == (sp.par != 0)) return MS_OK;
+  if (ms::launch_order_rows(sp, want, s->stream) != cudaSuccess) return MS_ECUDA;
+  ms::mol_set_rows(sp, want);
+  s->gdirty = true;
+  return MS_OK;
+}
+
+// While it lives, every full-form species' rows are in channel order, the order
+// of a checkpoint; its end brings back the order that the plans want.
+struct ChannelOrder {
+  ms_sim* s;
+  ms_status st = MS_OK;
+  bool dirty;
+  int par[ms::kMaxSpecies];
+  explicit ChannelOrder(ms_sim* s_) : s(s_), dirty(s_->gdirty) {
+    for (int si = 0; si < s->nspecies; ++si) {
+      ms::SpeciesDev& sp = s->sp[si];
+      par[si] = sp.par;
+      if (sp.bloch || sp.par_form || !sp.par || st != MS_OK) continue;
+      if (ms::launch_order_rows(sp, false, s->stream) != cudaSuccess) st = MS_ECUDA;
+      else ms::mol_set_rows(sp, false);
+    }
+  }
+  ms_status end() {
+    bool same = true;  // the captured steps stand if every species processes the rows that it did
+    for (int si = 0; si < s->nspecies; ++si) {
+      const ms_status e = order_rows(s, s->sp[si]);
+      if (st == MS_OK) st = e;
+      same = same && s->sp[si].par == par[si];
+    }
+    s->gdirty = dirty || !same;
+    return st;
+  }
+  ~ChannelOrder() { end(); }
+};
 
 // Device memory released before returning (the tuner's sandbox).
 struct Scratch {
@@ -557,7 +590,7 @@ ms_status tune_species(ms_sim* s, int si) {
   const int nc = ms::mol_plan_candidates(sp, cand, 32);
   if (nc < 2 || sp.nmol == 0) return MS_OK;
   const int nt = std::min(sp.nmol, 2048);
-  const size_t per = (size_t)sp.rows * sp.nr;
+  const size_t per = (size_t)sp.mrows * sp.nr;
   Scratch sc{s, {}};
   ms::SpeciesDev t = sp;
   ms::MolDev m = s->md;
@@ -644,6 +677,7 @@ ms_status tune_species(ms_sim* s, int si) {
     t.kern = cand[c][1];
     t.ch = cand[c][2];
     t.cps = cand[c][3];
+    MS_TRY(order_rows(s, t));  // the sandbox's own rows
     auto run = [&]() {
       ms::launch_mol_stage1(t, m, g, 1, err, s->stream);
       ms::launch_mol_stage2(t, m, g, 1, err, s->stream);
@@ -675,7 +709,7 @@ ms_status tune_species(ms_sim* s, int si) {
   sp.kern = cand[pick][1];
   sp.ch = cand[pick][2];
   sp.cps = cand[pick][3];
-  return MS_OK;
+  return order_rows(s, sp);
 }
 
 ms_status create_impl(const ms_grid_desc* G, const ms_materials_desc* M, const ms_molecules_desc* D,
@@ -1097,14 +1131,14 @@ static int pipelined_molecules(ms_sim* s, const ms::SpeciesDev* sp, int prescrib
   for (int si = 0; si < s->nspecies; ++si) {
     const ms::SpeciesDev& a = sp[si];
     const int nb = a.path == MS_MOL_STREAMING && !a.bloch ? std::min(s->batches, std::max(a.nmol, 1)) : 1;
-    const size_t per = (size_t)a.rows * a.nr;
+    const size_t per = (size_t)a.mrows * a.nr, per_d2 = (size_t)a.rows * a.nr;
     for (int b = 0; b < nb; ++b) {
       const int lo = (int)((long long)a.nmol * b / nb), hi = (int)((long long)a.nmol * (b + 1) / nb);
       ms::SpeciesDev r = a;
       r.nmol = hi - lo;
       r.mol = a.mol + lo;
       r.psi = a.psi + per * lo;
-      if (a.d2) r.d2 = a.d2 + per * lo;
+      if (a.d2) r.d2 = a.d2 + per_d2 * lo;
       r.fld = a.fld + lo;
       if (a.bloch_y) r.bloch_y = a.bloch_y + 3 * (size_t)lo;
       runs[nrun++] = r;
@@ -1236,7 +1270,7 @@ ms_status ms_step_noalloc(ms_sim* s, int64_t n) {
   for (int si = 0; si < s->nspecies; ++si) {
     const ms::SpeciesDev& sp = s->sp[si];
     if (sp.path != MS_MOL_STREAMING || sp.bloch || sp.nmol == 0) continue;
-    const size_t bytes = (size_t)sp.nmol * sp.rows * sp.nr * sizeof(float2);
+    const size_t bytes = (size_t)sp.nmol * sp.mrows * sp.nr * sizeof(float2);
     if (bytes > kNoAllocScratchBytes || off > kNoAllocScratchBytes - bytes) return MS_EINVAL;
     scratch[si] = s->noalloc_base + off / sizeof(float2);
     off += (bytes + 255) / 256 * 256;
@@ -1534,7 +1568,7 @@ std::vector<Blob> state_blobs(ms_sim* s) {
   for (int si = 0; si < s->nspecies; ++si) {
     const ms::SpeciesDev& sp = s->sp[si];
     if (sp.bloch) b.push_back({sp.bloch_y, (size_t)sp.nmol * 3 * sizeof(double)});
-    else b.push_back({sp.psi, (size_t)sp.nmol * sp.rows * sp.nr * sizeof(float2)});
+    else b.push_back({sp.psi, (size_t)sp.nmol * sp.mrows * sp.nr * sizeof(float2)});
   }
   if (s->nmol > 0) {
     const size_t n = (size_t)s->nmol;
@@ -1567,7 +1601,7 @@ CkHeader make_header(ms_sim* s, uint64_t nblobs) {
   h.aux_len = s->g.aux_len;
   h.ndet = s->g.ndet;
   h.nfreq = s->g.nfreq;
-  for (int si = 0; si < s->nspecies; ++si) h.state_rows[si] = s->sp[si].rows;
+  for (int si = 0; si < s->nspecies; ++si) h.state_rows[si] = s->sp[si].mrows;
   h.mol_substeps = s->nsub;
   h.src_kind = s->src_kind;
   for (int si = 0; si < s->nspecies; ++si) {
@@ -1614,6 +1648,11 @@ ms_status ms_save(ms_sim* s, const char* path) {
   const CkHeader h = make_header(s, blobs.size());
   FILE* f = std::fopen(path, "wb");
   if (!f) return MS_EIO;
+  ChannelOrder order(s);
+  if (order.st != MS_OK || cudaStreamSynchronize(s->stream) != cudaSuccess) {
+    std::fclose(f);
+    return MS_ECUDA;
+  }
   ms_status st = std::fwrite(&h, sizeof(h), 1, f) == 1 ? MS_OK : MS_EIO;
   PinnedPair pin;
   std::vector<char> buf;
@@ -1664,7 +1703,28 @@ ms_status ms_save(ms_sim* s, const char* path) {
     }
   }
   if (std::fclose(f) != 0 && st == MS_OK) st = MS_EIO;
+  const ms_status os = order.end();
+  if (st == MS_OK) st = os;
   return st == MS_OK ? latched(s) : st;
+}
+
+// After a load: whether the loaded states populate rows that the j = 0 start
+// cannot reach (no run of this library does); such species process every row.
+static ms_status find_other_rows(ms_sim* s) {
+  // the flag borrows the first Eq. 8 sum, which every readout computes anew
+  int* d = reinterpret_cast<int*>(s->md.Rnum);
+  for (int si = 0; si < s->nspecies; ++si) {
+    ms::SpeciesDev& sp = s->sp[si];
+    if (sp.bloch || sp.par_form) continue;
+    int flag = 0;
+    if (cudaMemsetAsync(d, 0, sizeof(int), s->stream) != cudaSuccess ||
+        ms::launch_find_other_rows(sp, d, s->stream) != cudaSuccess ||
+        cudaMemcpyAsync(&flag, d, sizeof(int), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
+        cudaStreamSynchronize(s->stream) != cudaSuccess)
+      return MS_ECUDA;
+    sp.all_rows = flag;
+  }
+  return MS_OK;
 }
 
 ms_status ms_load(ms_sim* s, const char* path) {
@@ -1683,6 +1743,12 @@ ms_status ms_load(ms_sim* s, const char* path) {
     a.steps = b.steps = 0;
     if (std::memcmp(&a, &b, sizeof(a)) != 0) st = MS_EINVAL;
   }
+  if (st != MS_OK) {
+    std::fclose(f);
+    return st;
+  }
+  ChannelOrder order(s);
+  if (order.st != MS_OK || cudaStreamSynchronize(s->stream) != cudaSuccess) st = MS_ECUDA;
   PinnedPair pin;
   std::vector<char> buf;
   for (size_t k = 0; st == MS_OK && k < blobs.size(); ++k) {
@@ -1733,6 +1799,9 @@ ms_status ms_load(ms_sim* s, const char* path) {
   }
   std::fclose(f);
   if (cudaStreamSynchronize(s->stream) != cudaSuccess && st == MS_OK) st = MS_ECUDA;  // copies in flight
+  const ms_status fs = find_other_rows(s);
+  const ms_status os = order.end();
+  if (st == MS_OK) st = fs != MS_OK ? fs : os;
   if (st != MS_OK) return st;
   // the step counter, host and device
   const long long step = h.steps;
@@ -1807,7 +1876,7 @@ ms_status ms_set_species_plan_ex(ms_sim* s, int32_t species, const int32_t plan[
   sp.ch = chunk;
   sp.cps = cps;
   s->gdirty = true;
-  return MS_OK;
+  return order_rows(s, sp);
 }
 
 ms_status ms_set_species_plan(ms_sim* s, int32_t species, int32_t path, int32_t kernel, int32_t chunk) {

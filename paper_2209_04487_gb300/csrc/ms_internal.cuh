@@ -100,12 +100,22 @@ struct Grid {
 // One species' device tables (all built on the host in FP64).
 struct SpeciesDev {
   int nr, jmax, nrot;
-  int par;                  // parity-reduced rows: ground even j, excited odd j
-  int rows, rows_g;         // state rows per molecule, of which ground rows
+  // Rows.  The couplings change j by one and swap the surfaces, so from the
+  // j = 0 ground-state start only (ground, even j) and (excited, odd j) are
+  // ever populated.  Stored: every row (MS_STATE_FULL) or those
+  // (MS_STATE_PARITY, par_form).  Processed (par): only those; a full-form
+  // molecule then stores them first, ground before excited, each in channel
+  // order, and its other rows, which hold zeros, behind them.  Kernels that
+  // process every row (par = 0) want full-form molecules in channel order.
+  int par;
+  int rows, rows_g;         // rows processed per molecule, of which ground rows
+  int mrows;                // rows stored per molecule
+  int par_form;             // MS_STATE_PARITY
+  int all_rows;             // a loaded state populates the other rows too: process every row
   int nmol;                 // molecules of this species
   const int* mol;           // their global ids (sorted by species, then by id)
-  float2* psi;              // state [nmol][rows][nr] (ground rows first), s = T^{-1/2} psi
-  float2* d2;               // streaming form: scratch (T - 1) s, same layout
+  float2* psi;              // state [nmol][mrows][nr], s = T^{-1/2} psi
+  float2* d2;               // streaming form: scratch (T - 1) s of the processed rows, [nmol][rows][nr]
   float4* fld;              // streaming form: per molecule (theta E'_z, theta E'_x/2, theta E'_y/2, terms)
   int mixed;                // kinetic pass as the split-FP16 tensor-core GEMM (MS_PREC_MIXED_F16X3)
   const uint16_t* kpl;      // mixed: (K - I) strip as four FP16 planes (Re hi, Re lo, Im hi, Im lo), x 2^kpl_exp
@@ -217,6 +227,14 @@ int launch_bloch_step(const SpeciesDev& sp, const MolDev& md, const Grid& g, int
                       cudaStream_t s);
 void launch_bloch_observe(const SpeciesDev& sp, const MolDev& md, cudaStream_t s);
 bool mol_step_supported(int nr, int nrot, int path);
+// whether the kernels of the species' plan process only the reachable rows
+bool mol_reachable_rows(const SpeciesDev& sp);
+// sets par, rows and rows_g for processing the reachable rows (or every row)
+void mol_set_rows(SpeciesDev& sp, bool reachable);
+// full-form molecules: channel order -> reachable rows first (or back), in place
+cudaError_t launch_order_rows(const SpeciesDev& sp, bool reachable_first, cudaStream_t s);
+// flags, in *flag, a non-zero value in a row that the j = 0 start cannot reach (channel order)
+cudaError_t launch_find_other_rows(const SpeciesDev& sp, int* flag, cudaStream_t s);
 // the driver's tensor-map encoder, which the tiled kernels need, is available
 bool mol_tensor_maps_available();
 // the (layout, kernel, chunk width, CTAs per SM) plans a species can run; returns how many
