@@ -40,42 +40,11 @@
 
 #include "ms_internal.cuh"
 #include "mol_common.cuh"
+#include "mol_fft.cuh"
 
 namespace ms {
 
 namespace {
-
-constexpr int kPad = 0;  // state rows are stored unpadded (one bulk copy per molecule)
-
-template <int NR>
-struct FFTShape;
-template <>
-struct FFTShape<64> {
-  static constexpr int N1 = 8, N2 = 8, THREADS = 256;
-};
-template <>
-struct FFTShape<128> {
-  static constexpr int N1 = 16, N2 = 8, THREADS = 256;
-};
-template <>
-struct FFTShape<256> {
-  static constexpr int N1 = 16, N2 = 16, THREADS = 256;
-};
-
-// cos / sin of t*pi/8, t = 0..7 (exact decimal expansions of the constants)
-__host__ __device__ constexpr double cos_pi8(int t) {
-  return t == 0 ? 1.0
-       : t == 1 ? 0.92387953251128675613
-       : t == 2 ? 0.70710678118654752440
-       : t == 3 ? 0.38268343236508977173
-       : t == 4 ? 0.0
-       : t == 5 ? -0.38268343236508977173
-       : t == 6 ? -0.70710678118654752440
-                : -0.92387953251128675613;
-}
-__host__ __device__ constexpr double sin_pi8(int t) { return t <= 4 ? cos_pi8(4 - t) : cos_pi8(t - 4); }
-__host__ __device__ constexpr float hi_of(double v) { return (float)v; }
-__host__ __device__ constexpr float lo_of(double v) { return (float)(v - (double)(float)v); }
 
 // (x) * (c + i s) with c = ch + cl, s = sh + sl (compensated)
 __device__ __forceinline__ float2 cmul_c(float2 x, float ch, float sh, float cl, float sl) {
@@ -90,154 +59,10 @@ __device__ __forceinline__ float2 cmul_c_add(float2 x, float4 w, float2 a) {
   return make_float2(fmaf(x.x, w.x, fmaf(-x.y, w.y, re_lo)), fmaf(x.x, w.y, fmaf(x.y, w.x, im_lo)));
 }
 
-// multiply by exp(-+ i t pi/8) (forward: minus)
-template <int T, bool INV>
-__device__ __forceinline__ float2 twiddle16(float2 v) {
-  if constexpr (T == 0) {
-    return v;
-  } else if constexpr (T == 4) {
-    return INV ? make_float2(-v.y, v.x) : make_float2(v.y, -v.x);
-  } else {
-    constexpr float c = (float)cos_pi8(T);
-    constexpr float s = INV ? (float)sin_pi8(T) : -(float)sin_pi8(T);
-    return make_float2(fmaf(v.x, c, -v.y * s), fmaf(v.x, s, v.y * c));
-  }
-}
-
-template <int L>
-__device__ constexpr int bitrev(int a) {
-  int r = 0;
-  for (int b = 1, q = L >> 1; b < L; b <<= 1, q >>= 1)
-    if (a & b) r |= q;
-  return r;
-}
-
-// In-register DFT of size L (8 or 16), radix-2 decimation in time.
-template <int L, bool INV, int H, int J>
-__device__ __forceinline__ void dft_stage_j(float2 (&x)[L]) {
-  if constexpr (J < H) {
-    constexpr int T = J * (16 / (2 * H));
-#pragma unroll
-    for (int a = J; a < L; a += 2 * H) {
-      const float2 u = x[a];
-      const float2 v = twiddle16<T, INV>(x[a + H]);
-      x[a] = u + v;
-      x[a + H] = u - v;
-    }
-    dft_stage_j<L, INV, H, J + 1>(x);
-  }
-}
-template <int L, bool INV, int H>
-__device__ __forceinline__ void dft_stages(float2 (&x)[L]) {
-  if constexpr (H < L) {
-    dft_stage_j<L, INV, H, 0>(x);
-    dft_stages<L, INV, 2 * H>(x);
-  }
-}
-template <int L, bool INV>
-__device__ __forceinline__ void dft_reg(float2 (&x)[L]) {
-#pragma unroll
-  for (int a = 0; a < L; ++a) {
-    const int b = bitrev<L>(a);
-    if (b > a) {
-      const float2 t = x[a];
-      x[a] = x[b];
-      x[b] = t;
-    }
-  }
-  dft_stages<L, INV, 1>(x);
-}
-
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// Four-step FFT pass on all `rows` rows (each NR complex, stride NRP) held
-// in shared memory, in place: forward DFT, multiply by kph[k], inverse DFT.
-// With kph = (P_k - 1)/NR it produces (T - 1) x; with kph = P_k/NR it
-// applies T.  n = n1 + N1 n2, k = k2 + N2 k1.  Step A: per n1, an N2-point
-// DFT over n2 and the twiddle exp(-2 pi i n1 k2/NR); step B: per k2, an
-// N1-point DFT over n1.  The intermediate y[n1][k2] lives at n1 + N1 k2,
-// xor-swizzled within each block of N1 so that step B is conflict free.
-// Position of y[n1][k2] of `row` within the row: the xor with (k2 mod N1)
-// spreads step B's N2 threads over distinct banks, the xor with CR for odd
-// rows keeps the two rows that share a half-warp apart.
-template <int N1, int N2>
-__device__ __forceinline__ int swz(int n1, int k2, int row) {
-  constexpr int CR = N1 > N2 ? N2 : (N1 == N2 && N1 == 8 ? 1 : 0);
-  return (n1 ^ (k2 % N1) ^ ((row & 1) * CR)) + N1 * k2;
-}
-
-template <int NR>
-__device__ void kinetic_pass(float2* st, int rows, const float2* kph, const float2* tw) {
-  using S = FFTShape<NR>;
-  constexpr int N1 = S::N1, N2 = S::N2, NT = S::THREADS, NRP = NR + kPad;
-  const int t = threadIdx.x;
-  {  // step A
-    constexpr int per = NT / N1;
-    const int n1 = t % N1, rsub = t / N1;
-    for (int r0 = 0; r0 < rows; r0 += per) {
-      const int row = r0 + rsub;
-      float2 x[N2];
-      if (row < rows) {
-#pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) x[n2] = st[row * NRP + n1 + N1 * n2];
-      }
-      __syncwarp();  // a row's N1 threads sit in one warp
-      if (row < rows) {
-        dft_reg<N2, false>(x);
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2)
-          st[row * NRP + swz<N1, N2>(n1, k2, row)] = cmul(x[k2], tw[k2 * N1 + n1]);
-      }
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-  {  // step B, the phase, inverse step B (in place per thread)
-    constexpr int per = NT / N2;
-    const int k2 = t % N2, rsub = t / N2;
-    for (int r0 = 0; r0 < rows; r0 += per) {
-      const int row = r0 + rsub;
-      if (row < rows) {
-        float2 x[N1];
-#pragma unroll
-        for (int n1 = 0; n1 < N1; ++n1) x[n1] = st[row * NRP + swz<N1, N2>(n1, k2, row)];
-        dft_reg<N1, false>(x);  // x[k1] = X[k2 + N2 k1]
-#pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) x[k1] = cmul(x[k1], kph[k2 + N2 * k1]);
-        dft_reg<N1, true>(x);
-#pragma unroll
-        for (int n1 = 0; n1 < N1; ++n1) st[row * NRP + swz<N1, N2>(n1, k2, row)] = x[n1];
-      }
-    }
-  }
-  __syncthreads();
-  {  // inverse step A
-    constexpr int per = NT / N1;
-    const int n1 = t % N1, rsub = t / N1;
-    for (int r0 = 0; r0 < rows; r0 += per) {
-      const int row = r0 + rsub;
-      float2 x[N2];
-      if (row < rows) {
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) {
-          const float2 w = tw[k2 * N1 + n1];
-          x[k2] = cmul(st[row * NRP + swz<N1, N2>(n1, k2, row)], make_float2(w.x, -w.y));
-        }
-        dft_reg<N2, true>(x);
-      }
-      __syncwarp();
-      if (row < rows) {
-#pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) st[row * NRP + n1 + N1 * n2] = x[n2];
-      }
-      __syncwarp();
-    }
-  }
-  __syncthreads();
 }
 
 // 16-byte asynchronous global -> shared copies (per thread), completed by
@@ -452,7 +277,7 @@ __global__ void __launch_bounds__(FFTShape<NR>::THREADS, FUSED ? 2 : (MAXR <= 4 
       return;
     }
     // ---- kinetic pass: st <- d2 = (T - 1) s
-    kinetic_pass<NR>(st, rows, s_kd, s_tw);
+    kinetic_pass<NR>(st, st, rows, s_kd, s_tw);
   } else {
     __syncthreads();
   }
@@ -687,47 +512,11 @@ cudaError_t launch_wait_timeout_probe(int tries, int* flag, cudaStream_t s) {
 // the coupling series (sigma_x swaps the surfaces) and the dipole only
 // exchange the other surface's vector, through one shared buffer.
 // ----------------------------------------------------------------------------
-template <int I, int N, class F>
-__device__ __forceinline__ void static_for(F&& f) {
-  if constexpr (I < N) {
-    f(std::integral_constant<int, I>());
-    static_for<I + 1, N>(f);
-  }
-}
 constexpr int ch_j(int c) { return c < 1 ? 0 : (c < 4 ? 1 : (c < 9 ? 2 : (c < 16 ? 3 : (c < 25 ? 4 : -1)))); }
 __host__ __device__ constexpr int j_of_c(int c) { return ch_j(c); }
 constexpr int ch_m(int c) { return c - ch_j(c) * ch_j(c) - ch_j(c); }
 // channel of (j, m), or -1 outside the basis of size J
 constexpr int ch_of(int j, int m, int J) { return (j < 0 || j > J || m < -j || m > j) ? -1 : j * j + j + m; }
-
-// ---- angular coefficients as compile-time constants ------------------------
-// square root by Newton's iteration in double precision (x >= 0)
-constexpr double c_sqrt(double x) {
-  if (x <= 0.0) return 0.0;
-  double r = x < 1.0 ? 1.0 : x;
-  for (int i = 0; i < 64; ++i) r = 0.5 * (r + x / r);
-  return r;
-}
-constexpr bool ch_valid(int j, int m) { return j >= 0 && m >= -j && m <= j; }
-// <j+1, m|cos t|j, m>, -<j+1, m+1|sin t e^{i p}|j, m> and <j-1, m+1|sin t e^{i p}|j, m>
-// in the Condon-Shortley phase convention
-constexpr double c_ang_a(int j, int m) {
-  return c_sqrt(((j + 1.0) * (j + 1) - (double)m * m) / ((2.0 * j + 1) * (2.0 * j + 3)));
-}
-constexpr double c_ang_b(int j, int m) {
-  return -c_sqrt((j + m + 1.0) * (j + m + 2) / ((2.0 * j + 1) * (2.0 * j + 3)));
-}
-constexpr double c_ang_c(int j, int m) {
-  return c_sqrt((j - m) * (j - m - 1.0) / ((2.0 * j - 1) * (2.0 * j + 1)));
-}
-// Row (j, m) of Z, S+ = sin t e^{ip} and S- = sin t e^{-ip} on the runs (j + 1, .) and (j - 1, .):
-// Z from (j +- 1, m), S+ from (j +- 1, m - 1), S- from (j +- 1, m + 1).
-constexpr float c_zu(int j, int m) { return (float)c_ang_a(j, m); }
-constexpr float c_zd(int j, int m) { return ch_valid(j - 1, m) ? (float)c_ang_a(j - 1, m) : 0.f; }
-constexpr float c_pu(int j, int m) { return ch_valid(j + 1, m - 1) ? (float)c_ang_c(j + 1, m - 1) : 0.f; }
-constexpr float c_pd(int j, int m) { return ch_valid(j - 1, m - 1) ? (float)c_ang_b(j - 1, m - 1) : 0.f; }
-constexpr float c_mu(int j, int m) { return (float)c_ang_b(j, m); }
-constexpr float c_md(int j, int m) { return j >= 1 ? (float)c_ang_c(j, m) : 0.f; }
 
 // Per molecule of a streaming species: the local field in the molecule frame
 // scaled by theta, (theta E'_z, theta E'_x / 2, theta E'_y / 2), and the
@@ -791,13 +580,12 @@ struct Rows {
   }
 };
 
-// i (theta/n) (M in) for row R of surface SF, M = E'_z Z + (E'_x - i E'_y)/2 S+
+// i (theta/n) (M in) for row R of either surface, M = E'_z Z + (E'_x - i E'_y)/2 S+
 // + (E'_x + i E'_y)/2 S- (the molecule-frame coupling), `in` the other
 // surface's rows; f = (theta E'_z, theta E'_x/2, theta E'_y/2)
-template <int J, bool PAR, int SF, int R, class V>
+template <int J, int R, class V>
 __device__ __forceinline__ float2 coupling_row(const V& in, float fz, float fx, float fy, float cn) {
-  using L = Rows<J, PAR>;
-  constexpr int C = L::chan(SF, R), j = ch_j(C), mm = ch_m(C);
+  constexpr int j = ch_j(R), mm = ch_m(R);
   float2 az = make_float2(0.f, 0.f), ap = az, am = az;
   auto mac = [&](float2& a, float cf, auto ni) {
     constexpr int q = decltype(ni)::value;
@@ -807,16 +595,16 @@ __device__ __forceinline__ float2 coupling_row(const V& in, float fz, float fx, 
     }
   };
   if constexpr (j < J) {
-    mac(az, c_zu(j, mm), std::integral_constant<int, L::row(1 - SF, ch_of(j + 1, mm, J))>());
-    mac(ap, c_pu(j, mm), std::integral_constant<int, L::row(1 - SF, ch_of(j + 1, mm - 1, J))>());
-    mac(am, c_mu(j, mm), std::integral_constant<int, L::row(1 - SF, ch_of(j + 1, mm + 1, J))>());
+    mac(az, c_zu(j, mm), std::integral_constant<int, (ch_of(j + 1, mm, J))>());
+    mac(ap, c_pu(j, mm), std::integral_constant<int, (ch_of(j + 1, mm - 1, J))>());
+    mac(am, c_mu(j, mm), std::integral_constant<int, (ch_of(j + 1, mm + 1, J))>());
   }
   if constexpr (j > 0) {
-    mac(az, c_zd(j, mm), std::integral_constant<int, c_zd(j, mm) != 0.f ? L::row(1 - SF, ch_of(j - 1, mm, J)) : -1>());
+    mac(az, c_zd(j, mm), std::integral_constant<int, c_zd(j, mm) != 0.f ? (ch_of(j - 1, mm, J)) : -1>());
     mac(ap, c_pd(j, mm),
-        std::integral_constant<int, c_pd(j, mm) != 0.f ? L::row(1 - SF, ch_of(j - 1, mm - 1, J)) : -1>());
+        std::integral_constant<int, c_pd(j, mm) != 0.f ? (ch_of(j - 1, mm - 1, J)) : -1>());
     mac(am, c_md(j, mm),
-        std::integral_constant<int, c_md(j, mm) != 0.f ? L::row(1 - SF, ch_of(j - 1, mm + 1, J)) : -1>());
+        std::integral_constant<int, c_md(j, mm) != 0.f ? (ch_of(j - 1, mm + 1, J)) : -1>());
   }
   // a = fz Z-part + fx (S+ + S-) - i fy (S+ - S-)
   const float bx = ap.x + am.x, by = ap.y + am.y, cx = ap.x - am.x, cy = ap.y - am.y;
@@ -865,18 +653,16 @@ __device__ __forceinline__ void dipole_rows(const V& gv, const W& ev, float2& ac
   }
 }
 
-// Point-resident R-space pass (and, FUSED, the kinetic pass): one CTA of 2 N_r
-// threads per molecule, thread = (radial point, surface); PAR: parity-reduced
-// rows.  FUSED (N_r = 128): the state is staged once into D and turned in
-// place into d2 = (T - 1) s by the shared-memory FFT, while a second copy of
-// s (an L2 hit) fills X.  Otherwise d2 comes from the kinetic kernel's
-// scratch.  Every CTA barrier sits in code all threads run; the per-surface
-// work between them is compiled once per surface (row counts differ when
-// PAR).
-template <int J, int NR, bool FUSED, bool PAR, bool DIPR = false>
-__global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? (PAR ? 3 : 2) : 1))
+// Point-resident R-space pass (and, FUSED, the kinetic pass) of states with
+// every row populated (the reachable rows run on whole rotors, mol_rotor.cu):
+// one CTA of 2 N_r threads per molecule, thread = (radial point, surface).
+// FUSED (N_r = 128): the state is staged once into D and turned in place into
+// d2 = (T - 1) s by the shared-memory FFT, while a second copy of s (an L2
+// hit) fills X.  Otherwise d2 comes from the kinetic kernel's scratch.
+template <int J, int NR, bool FUSED, bool DIPR = false>
+__global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? 2 : 1))
     mol_rpoint_kernel(SpeciesDev sp, MolDev md, int* err) {
-  using L = Rows<J, PAR>;
+  using L = Rows<J, false>;
   constexpr int ROWS = L::ROWS, NG = L::NG, NT = 2 * NR, NW = NT / 32;
   constexpr int RMAX = L::NG > L::NE ? L::NG : L::NE;
   constexpr unsigned kStateBytes = (unsigned)ROWS * NR * sizeof(float2);  // one molecule's state
@@ -960,57 +746,42 @@ __global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? (PAR ? 3 :
       mbar_expect_tx(&s_bar[1], kStateBytes);
       bulk_g2s(X, sp.psi + mol0, kStateBytes, &s_bar[1]);
     }
-    kinetic_pass<NR>(D, ROWS, s_kd, s_tw);  // D <- d2 = (T - 1) s
+    kinetic_pass<NR>(D, D, ROWS, s_kd, s_tw);  // D <- d2 = (T - 1) s
     if (!wait_all(1)) return;
   }
-  // per-surface work: both surfaces share one row list in the full layout
-  auto per_surface = [&](auto&& fn) {
-    if constexpr (PAR) {
-      if (sf == 0) fn(std::integral_constant<int, 0>());
-      else fn(std::integral_constant<int, 1>());
-    } else {
-      fn(std::integral_constant<int, 0>());
-    }
-  };
   // ---- eta = V^{1/2} u, u = s + d2, over this thread's own rows of the state
-  auto eta = [&](auto sfc) {
-    constexpr int SF = decltype(sfc)::value;
-    static_for<0, L::N(SF)>([&](auto ri) {
-      constexpr int r = decltype(ri)::value, j = ch_j(L::chan(SF, r));
+  if (nterms > 0)
+    static_for<0, L::NROT>([&](auto ri) {
+      constexpr int r = decltype(ri)::value, j = ch_j(r);
       Xo[r * NR] = cmul(vh[j], Xo[r * NR] + Do[r * NR]);
     });
-  };
-  if (nterms > 0) per_surface(eta);
   __syncthreads();
   // ---- coupling series: S = sum_n (i theta M sigma_x)^n eta / n!
   float2 sacc[RMAX], in[RMAX];
 #pragma unroll
   for (int r = 0; r < RMAX; ++r) sacc[r] = make_float2(0.f, 0.f);
-  auto term = [&](auto sfc, float cn, bool store) {
-    constexpr int SF = decltype(sfc)::value;
-    static_for<0, L::N(SF)>([&](auto ri) {
+  auto term = [&](float cn, bool store) {
+    static_for<0, L::NROT>([&](auto ri) {
       constexpr int r = decltype(ri)::value;
-      const float2 o = coupling_row<J, PAR, SF, r>(in, f.x, f.y, f.z, cn);
+      const float2 o = coupling_row<J, r>(in, f.x, f.y, f.z, cn);
       sacc[r].x += o.x;
       sacc[r].y += o.y;
       if (store) Xo[r * NR] = o;
     });
   };
-  const int n_oth = PAR ? (sf ? L::NG : L::NE) : L::NROT;
   for (int n = 1; n <= nterms; ++n) {
 #pragma unroll
-    for (int r = 0; r < RMAX; ++r)
-      if (r < n_oth) in[r] = Xt[r * NR];
+    for (int r = 0; r < RMAX; ++r) in[r] = Xt[r * NR];
     __syncthreads();  // every thread has its input: the buffer may be overwritten
     const float cn = 1.f / (float)n;
     const bool store = n < nterms;
-    per_surface([&](auto sfc) { term(sfc, cn, store); });
+    term(cn, store);
     if (store) __syncthreads();
   }
   // ---- d1 = (V - 1) u + V^{1/2} S ; mask ; s' = s + (d2 + d1) + cfix s
   float sn2 = 0.f, sn2_lo = 0.f, absd = 0.f, rnd = 0.f;  // |s'|^2 compensated from the first term on
-  auto update = [&](auto sfc) {
-    constexpr int SF = decltype(sfc)::value, NO = L::N(SF);
+  {
+    constexpr int NO = L::NROT;
     // s again (from L2), in two batches each requested in full first; d2 from shared memory
     constexpr int NB = NO > 1 ? (NO + 1) / 2 : 1;
     float2 sb[NB];
@@ -1021,7 +792,7 @@ __global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? (PAR ? 3 :
     };
     fetch(0);
     static_for<0, NO>([&](auto ri) {
-      constexpr int r = decltype(ri)::value, j = ch_j(L::chan(SF, r));
+      constexpr int r = decltype(ri)::value, j = ch_j(r);
       if constexpr (r == NB) fetch(NB);
       const float2 sv = sb[r % NB], dv = Do[r * NR];
       const float2 u = sv + dv;
@@ -1039,8 +810,7 @@ __global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? (PAR ? 3 :
       sacc[r] = s1;  // the new state of this surface, kept for the dipole
       Xo[r * NR] = s1;
     });
-  };
-  per_surface(update);
+  }
   __syncthreads();
   // ---- dipole in the molecule frame: sum over ground rows of conj(g_c) (A e)_c
   // for A = Z, S+, S-; ground rows [0, NH) on the ground-surface threads, the
@@ -1049,11 +819,10 @@ __global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? (PAR ? 3 :
   {
     constexpr int NH = (NG + 1) / 2;
 #pragma unroll
-    for (int r = 0; r < RMAX; ++r)
-      if (r < n_oth) in[r] = Xt[r * NR];
+    for (int r = 0; r < RMAX; ++r) in[r] = Xt[r * NR];
     float2 accP = make_float2(0.f, 0.f), accM = accP, accZ = accP;
-    if (sf == 0) dipole_rows<J, PAR, 0, NH>(sacc, in, accP, accM, accZ);
-    else dipole_rows<J, PAR, NH, NG>(in, sacc, accP, accM, accZ);
+    if (sf == 0) dipole_rows<J, false, 0, NH>(sacc, in, accP, accM, accZ);
+    else dipole_rows<J, false, NH, NG>(in, sacc, accP, accM, accZ);
     dP = accP.x + accM.x;
     dQ = accP.y - accM.y;
     dZ = 2.f * accZ.x;
@@ -1112,11 +881,11 @@ __global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? (PAR ? 3 :
   }
 }
 
-template <int J, int NR, bool FUSED, bool PAR, bool DIPR = false>
-static void launch_rpoint_jnp(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
-  constexpr int ROWS = Rows<J, PAR>::ROWS;
+template <int J, int NR, bool FUSED, bool DIPR = false>
+static void launch_rpoint_jnd(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
+  constexpr int ROWS = Rows<J, false>::ROWS;
   const size_t smem = (size_t)2 * ROWS * NR * sizeof(float2) + (FUSED ? 2 * NR * sizeof(float2) : 0);
-  auto k = mol_rpoint_kernel<J, NR, FUSED, PAR, DIPR>;
+  auto k = mol_rpoint_kernel<J, NR, FUSED, DIPR>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   k<<<sp.nmol, 2 * NR, smem, s>>>(sp, md, err);
@@ -1125,17 +894,19 @@ template <int J, int NR, bool FUSED>
 static void launch_rpoint_jn(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
   if constexpr (NR <= 128) {  // R-dependent dipole: N_r 64 or 128
     if (sp.dipw) {
-      if (sp.par) launch_rpoint_jnp<J, NR, FUSED, true, true>(sp, md, err, s);
-      else launch_rpoint_jnp<J, NR, FUSED, false, true>(sp, md, err, s);
+      launch_rpoint_jnd<J, NR, FUSED, true>(sp, md, err, s);
       return;
     }
   }
-  if (sp.par) launch_rpoint_jnp<J, NR, FUSED, true>(sp, md, err, s);
-  else launch_rpoint_jnp<J, NR, FUSED, false>(sp, md, err, s);
+  launch_rpoint_jnd<J, NR, FUSED>(sp, md, err, s);
 }
 
 template <int NR, bool FUSED = false>
 static void launch_rpoint_n(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
+  if (sp.par) {
+    launch_rotor(sp, md, err, s);
+    return;
+  }
   switch (sp.jmax) {
     case 0: launch_rpoint_jn<0, NR, FUSED>(sp, md, err, s); break;
     case 1: launch_rpoint_jn<1, NR, FUSED>(sp, md, err, s); break;
@@ -1184,7 +955,7 @@ __global__ void __launch_bounds__(FFTShape<NR>::THREADS) mol_dipole_r_kernel(Spe
     if (!ok) mbar_wait_sleep(&s_bar[0], 0);
     return;
   }
-  kinetic_pass<NR>(X, ROWS, s_kh, s_tw);  // psi' = T^{1/2} s'
+  kinetic_pass<NR>(X, X, ROWS, s_kh, s_tw);  // psi' = T^{1/2} s'
   float dP = 0.f, dQ = 0.f, dZ = 0.f;
   if (t < NR) {
     float2 gv[NG], ev[NE > 0 ? NE : 1];  // J = 0, parity-reduced: no excited row
@@ -1307,7 +1078,7 @@ __global__ void __launch_bounds__(FFTShape<NR>::THREADS)
     __syncthreads();
     load_state(st, ge + (long long)b0 * NR, nb, NR, NRP);
     __syncthreads();
-    kinetic_pass<NR>(st, nb, s_kh, s_tw);  // psi = T^{1/2} s
+    kinetic_pass<NR>(st, st, nb, s_kh, s_tw);  // psi = T^{1/2} s
     for (int r = threadIdx.x; r < NR; r += blockDim.x) {
       float a = 0.f;
       for (int row = 0; row < nb; ++row) {
@@ -1401,7 +1172,7 @@ __global__ void __launch_bounds__(FFTShape<NR>::THREADS)
     if (!ok) mbar_wait(&s_bar, 0, kWaitPolls);
     return;
   }
-  kinetic_pass<NR>(st, nrows, s_kd, s_tw);
+  kinetic_pass<NR>(st, st, nrows, s_kd, s_tw);
   const float4* s4 = reinterpret_cast<const float4*>(st);
   float4* d4 = reinterpret_cast<float4*>(sp.d2 + r0 * NR);
   for (int q = t; q < nrows * NR / 2; q += blockDim.x) d4[q] = s4[q];

@@ -7,6 +7,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "ms_internal.cuh"
@@ -76,6 +77,44 @@ constexpr long long kWaitPolls = 1LL << 24;  // far beyond any copy's duration
 
 __device__ __forceinline__ int j_of(int c) { return (int)sqrtf((float)c + 0.5f); }  // c = j^2+j+m
 
+template <int I, int N, class F>
+__device__ __forceinline__ void static_for(F&& f) {
+  if constexpr (I < N) {
+    f(std::integral_constant<int, I>());
+    static_for<I + 1, N>(f);
+  }
+}
+
+// ---- angular coefficients as compile-time constants ------------------------
+// square root by Newton's iteration in double precision (x >= 0)
+constexpr double c_sqrt(double x) {
+  if (x <= 0.0) return 0.0;
+  double r = x < 1.0 ? 1.0 : x;
+  for (int i = 0; i < 64; ++i) r = 0.5 * (r + x / r);
+  return r;
+}
+constexpr bool ch_valid(int j, int m) { return j >= 0 && m >= -j && m <= j; }
+// <j+1, m|cos t|j, m>, -<j+1, m+1|sin t e^{i p}|j, m> and <j-1, m+1|sin t e^{i p}|j, m>
+// in the Condon-Shortley phase convention
+constexpr double c_ang_a(int j, int m) {
+  return c_sqrt(((j + 1.0) * (j + 1) - (double)m * m) / ((2.0 * j + 1) * (2.0 * j + 3)));
+}
+constexpr double c_ang_b(int j, int m) {
+  return -c_sqrt((j + m + 1.0) * (j + m + 2) / ((2.0 * j + 1) * (2.0 * j + 3)));
+}
+constexpr double c_ang_c(int j, int m) {
+  return c_sqrt((j - m) * (j - m - 1.0) / ((2.0 * j - 1) * (2.0 * j + 1)));
+}
+// Row (j, m) of Z, S+ = sin t e^{ip} and S- = sin t e^{-ip} on the runs (j + 1, .) and (j - 1, .):
+// Z from (j +- 1, m), S+ from (j +- 1, m - 1), S- from (j +- 1, m + 1).
+constexpr float c_zu(int j, int m) { return (float)c_ang_a(j, m); }
+constexpr float c_zd(int j, int m) { return ch_valid(j - 1, m) ? (float)c_ang_a(j - 1, m) : 0.f; }
+constexpr float c_pu(int j, int m) { return ch_valid(j + 1, m - 1) ? (float)c_ang_c(j + 1, m - 1) : 0.f; }
+constexpr float c_pd(int j, int m) { return ch_valid(j - 1, m - 1) ? (float)c_ang_b(j - 1, m - 1) : 0.f; }
+constexpr float c_mu(int j, int m) { return (float)c_ang_b(j, m); }
+constexpr float c_md(int j, int m) { return j >= 1 ? (float)c_ang_c(j, m) : 0.f; }
+
+
 
 // compensated FP32 accumulation (TwoSum): hi + lo carries ~48 bits
 __device__ __forceinline__ void acc2(float& hi, float& lo, float x) {
@@ -127,6 +166,35 @@ static cudaError_t upload_triplet_tables_local(const CouplEntry* dip) {
 
 constexpr int kTriGuard = 3;  // zero rows ahead of each term buffer
 
+// ---- packed FP32x2 arithmetic (one instruction; sign changes and equal constants of both parts are free)
+__device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ float2 dup2(float c) { return make_float2(c, c); }
+// round_update on one point held as a (Re, Im) pair, packed: s' = fl(s + D'),
+// D' = D + c s, with the exact residual of that rounding folded into acc
+// (per part; the two parts are added at the end)
+__device__ __forceinline__ float2 round_update2(float2 sv, float2 D, float2 c, float2& acc) {
+  const float2 d = fma2(c, sv, D);
+  const float2 n = add2(sv, d);
+  const float2 b = sub2(n, sv);
+  const float2 e = add2(sub2(sv, sub2(n, b)), sub2(d, b));
+  acc = fma2(n, e, acc);
+  return n;
+}
+// compensated sums of point pairs (TwoSum per part)
+__device__ __forceinline__ void acc2p(float2& hi, float2& lo, float2 x) {
+  const float2 t = add2(hi, x);
+  const float2 z = sub2(t, hi);
+  lo = add2(lo, add2(sub2(hi, sub2(t, z)), sub2(x, z)));
+  hi = t;
+}
+
+
 
 // Wait for phase `parity`, each try suspending up to hint_ns until the phase
 // completes; gives up after `tries` tries (by default about 2 s in all).
@@ -171,6 +239,9 @@ static void launch_persistent(RspaceKernel k, int nt, int bytes, const SpeciesDe
 // parity-reduced species), launched persistently on stream s.
 void launch_rspace_pair(const SpeciesDev& sp, const MolDev& md, int* err, const RspaceMaps& maps, int tile,
                         cudaStream_t s);
+// The molecular step on whole rotors, J <= 4, reachable rows (mol_rotor.cu):
+// the R-space pass of a streaming species or the whole fused step.
+void launch_rotor(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s);
 // uploads the angular tables into mol_pair.cu's copy
 cudaError_t upload_triplet_tables_pair(const CouplEntry* dip);
 // The one-point-a-thread tiled R-space pass (mol_tile.cu) at tile width

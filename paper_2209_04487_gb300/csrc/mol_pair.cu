@@ -96,13 +96,6 @@ struct Rs2Dims {
                 "tensor-copy destinations 128-byte aligned, tables 16-byte aligned");
 };
 
-__device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
-__device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
 // (ax + i ay)(bx + i by) on point pairs
 __device__ __forceinline__ void cmul2(float2 ax, float2 ay, float2 bx, float2 by, float2& rx, float2& ry) {
   rx = fma2(ax, bx, neg2(mul2(ay, by)));
@@ -116,25 +109,6 @@ template <int OFF>
 __device__ __forceinline__ void sts4(unsigned char* base, int off, float4 v) {
   *reinterpret_cast<float4*>(base + off + OFF) = v;
 }
-// round_update on one point held as a (Re, Im) pair, packed: s' = fl(s + D'),
-// D' = D + c s, with the exact residual of that rounding folded into acc
-// (per part; the two parts are added at the end)
-__device__ __forceinline__ float2 round_update2(float2 sv, float2 D, float2 c, float2& acc) {
-  const float2 d = fma2(c, sv, D);
-  const float2 n = add2(sv, d);
-  const float2 b = sub2(n, sv);
-  const float2 e = add2(sub2(sv, sub2(n, b)), sub2(d, b));
-  acc = fma2(n, e, acc);
-  return n;
-}
-// compensated sums of point pairs (TwoSum per part)
-__device__ __forceinline__ void acc2p(float2& hi, float2& lo, float2 x) {
-  const float2 t = add2(hi, x);
-  const float2 z = sub2(t, hi);
-  lo = add2(lo, add2(sub2(hi, sub2(t, z)), sub2(x, z)));
-  hi = t;
-}
-
 // first row of shell j' within its surface (the surface holding j')
 template <bool PAR>
 __device__ __forceinline__ int shell_row(int jp) {

@@ -1,0 +1,308 @@
+// Molecular step on whole rotors (J <= 4, reachable rows): the kernel and its
+// launch.
+//
+// The reachable rows of a molecule are one vector psi_{j m} over all channels
+// (the surface is the parity of j), (J + 1)^2 values at a radial point.  A
+// thread holds all of them at one point in registers, so the coupling
+// E'.R^ = E'_z Z + S+- parts, which joins (j, m) with (j +- 1, m) and (j +- 1,
+// m +- 1), is register arithmetic with compile-time coefficients: no exchange
+// through shared memory and no barrier between the terms of the series.  With
+// a thread per surface and point instead (the kernel that runs states with
+// every row populated), the other surface's rows pass through shared memory
+// for every term and its barriers and the idle half of the larger surface's
+// threads cost a third of the time.
+//
+// The coupling's exponential series S = sum_{n=1..N} (i theta M)^n / n! eta is
+// summed by Horner's rule, S = i theta M y_1, y_n = eta + (i theta / (n + 1)) M
+// y_{n+1}, y_N = eta: each row's S goes straight into the update.  Values are
+// kept as (Re, Im) pairs and multiplied by real coefficients as packed FP32x2
+// products, whose equal constants are immediates.
+//
+// What bounds it: issue slots and instruction fetch (2,900 instructions of
+// straight-line code at J = 4, about 85 a row and point; three CTAs of N_r = 128
+// an SM by registers), then HBM.  Per row and point of the reachable rows: the
+// R-space pass at J = 4, N_r = 64 (375,000 molecules) takes 4.57 ps, 5.3 TB/s,
+// against 7.13 for a thread per surface; the fused step at J = 4, N_r = 128
+// (187,500 molecules) 6.87 against 12.14 ps.
+//
+// FUSED (N_r = 128): the kinetic pass runs in the same kernel.  The state
+// arrives by one bulk copy and stays in shared memory; the FFT turns it into
+// d2 = (T - 1) s beside it.
+#include "mol_fft.cuh"
+
+namespace ms {
+namespace {
+
+template <int J>
+struct RotorDims {
+  static constexpr int NROT = (J + 1) * (J + 1);
+  // first row of shell j among the reachable rows: ground even shells, then excited odd shells
+  static constexpr int shell(int j) {
+    int n = 0;
+    for (int q = 0; q <= J; ++q)
+      if ((q & 1) < (j & 1) || ((q & 1) == (j & 1) && q < j)) n += 2 * q + 1;
+    return n;
+  }
+  static constexpr int row(int j, int m) { return shell(j) + j + m; }
+  // register of (j, m): columns m = -J .. J, each by j
+  static constexpr int at(int j, int m) {
+    int n = 0;
+    for (int q = -J; q < m; ++q) n += J + 1 - (q < 0 ? -q : q);
+    return n + j - (m < 0 ? -m : m);
+  }
+};
+
+// calls fn(j, m) for every channel, columns in order
+template <int J, class F>
+__device__ __forceinline__ void for_channels(F&& fn) {
+  static_for<-J, J + 1>([&](auto mc) {
+    constexpr int m = decltype(mc)::value;
+    static_for<(m < 0 ? -m : m), J + 1>([&](auto jc) { fn(jc, mc); });
+  });
+}
+
+template <int J, int NR, bool FUSED, bool DIPR>
+__global__ void __launch_bounds__(NR, NR <= 64 ? 6 : (NR <= 128 ? 3 : 1))
+    mol_rotor_kernel(SpeciesDev sp, MolDev md, int* err) {
+  using D = RotorDims<J>;
+  constexpr int NROT = D::NROT, NW = NR / 32;
+  constexpr unsigned kStateBytes = (unsigned)NROT * NR * sizeof(float2);
+  extern __shared__ __align__(16) float4 smem4[];
+  float2* Sb = reinterpret_cast<float2*>(smem4);  // fused: [NROT][NR] s
+  float2* Db = Sb + NROT * NR;                    // fused: [NROT][NR] d2
+  float2* s_tw = Db + NROT * NR;                  // fused: [N2][N1] FFT twiddles
+  float2* s_kd = s_tw + NR;                       // fused: [NR] kinetic phase deltas
+  __shared__ __align__(8) unsigned long long s_bar[1];
+  __shared__ float s_red[NW][10];
+  __shared__ float s_fin[8], s_fin_lo[2];
+
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int lm = blockIdx.x, m_ = sp.mol[lm];
+  float2* const gs = sp.psi + (long long)lm * sp.mrows * NR;  // this molecule's state
+  if constexpr (FUSED) {
+    if (t == 0) {
+      mbar_init(&s_bar[0], 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      mbar_expect_tx(&s_bar[0], kStateBytes);
+      bulk_g2s(Sb, gs, kStateBytes, &s_bar[0]);
+    }
+    s_tw[t] = __ldg(&sp.twiddle[t]);
+    s_kd[t] = __ldg(&sp.kdelta[t]);
+  }
+  float4 f = __ldg(&sp.fld[lm]);  // (theta E'_z, theta E'_x/2, theta E'_y/2, terms)
+  if constexpr (DIPR) {           // times d(R) / max|d| at this thread's point
+    const float dw = __ldg(&sp.dipw[t]);
+    f.x *= dw;
+    f.y *= dw;
+    f.z *= dw;
+  }
+  const int nterms = max(__float_as_int(f.w), 1);  // no field: one term of zeros
+  const float mk = sp.maskw[t].x;
+  const float cfix = md.ncorr[m_];  // rounding feedback of the previous step
+  // what the closing threads add to: the previous dipole, the absorbed norm so far
+  const double old = t < 3 ? md.mu[3 * (long long)m_ + t]
+                           : (t == 5 || t == 6 ? md.absorbed[2 * (long long)m_ + (t - 5)] : 0.0);
+  if constexpr (FUSED) {
+    __syncthreads();  // the barrier is initialised
+    const bool ok = mbar_wait_sleep(&s_bar[0], 0);
+    if (!__syncthreads_and(ok)) {
+      if (t == 0) atomicOr(err, kErrTimeout);
+      if (!ok) mbar_wait_sleep(&s_bar[0], 0);
+      return;
+    }
+    kinetic_pass<NR, NR, true>(Db, Sb, NROT, s_kd, s_tw);  // d2 = (T - 1) s
+  }
+  const float2* const ss = (FUSED ? Sb : gs) + t;
+  const float2* const ds = (FUSED ? Db : sp.d2 + (long long)lm * NROT * NR) + t;
+  auto s_at = [&](int row) { return ss[row * NR]; };
+  auto d_at = [&](int row) { return FUSED ? ds[row * NR] : __ldg(ds + row * NR); };
+  // potential phases of shell j on the surface of its parity
+  auto vh_at = [&](auto jc) {
+    constexpr int j = decltype(jc)::value;
+    return __ldg(sp.vhalf + ((j & 1) * (J + 1) + j) * NR + t);
+  };
+  auto vd_at = [&](auto jc) {
+    constexpr int j = decltype(jc)::value;
+    return __ldg(sp.vdelta + ((j & 1) * (J + 1) + j) * NR + t);
+  };
+
+  float2 v[NROT], q[NROT];
+  // base + i (M v) at (j, m); z2, x2, y2 the field's factors
+  auto coupled = [&](auto jc, auto mc, float2 z2, float2 x2, float2 y2, float2 base) -> float2 {
+    constexpr int j = decltype(jc)::value, m = decltype(mc)::value;
+    auto sum2 = [&](auto cf0, auto cf1, auto c2) {  // cf0 (j - 1, c2) + cf1 (j + 1, c2)
+      constexpr int cq = decltype(c2)::value, mq = cq < 0 ? -cq : cq;
+      constexpr bool lo = j - 1 >= mq, hi = j + 1 <= J && j + 1 >= mq;
+      if constexpr (lo && hi)
+        return fma2(dup2(cf0()), v[D::at(lo ? j - 1 : j, lo ? cq : m)], mul2(dup2(cf1()), v[D::at(hi ? j + 1 : j, hi ? cq : m)]));
+      else if constexpr (lo) return mul2(dup2(cf0()), v[D::at(j - 1, cq)]);
+      else if constexpr (hi) return mul2(dup2(cf1()), v[D::at(j + 1, cq)]);
+      else return make_float2(0.f, 0.f);
+    };
+    const float2 az = sum2([] { return c_zd(j, m); }, [] { return c_zu(j, m); }, std::integral_constant<int, m>());
+    const float2 ap = sum2([] { return c_pd(j, m); }, [] { return c_pu(j, m); }, std::integral_constant<int, m - 1>());
+    const float2 am = sum2([] { return c_md(j, m); }, [] { return c_mu(j, m); }, std::integral_constant<int, m + 1>());
+    const float2 r = fma2(z2, az, mul2(x2, add2(ap, am)));
+    const float2 e = fma2(y2, sub2(ap, am), base);
+    return make_float2(e.x - r.y, e.y + r.x);
+  };
+  auto eta = [&](auto jc, auto mc) -> float2 {  // V^{1/2} (s + d2)
+    constexpr int row = D::row(decltype(jc)::value, decltype(mc)::value);
+    return cmul(vh_at(jc), add2(s_at(row), d_at(row)));
+  };
+  for_channels<J>([&](auto jc, auto mc) { v[D::at(decltype(jc)::value, decltype(mc)::value)] = eta(jc, mc); });
+  // ---- y_1 by Horner's rule
+#pragma unroll 1
+  for (int n = nterms; n >= 2; --n) {
+    const float cn = 1.f / (float)n;
+    const float2 z2 = dup2(f.x * cn), x2 = dup2(f.y * cn), y2 = dup2(f.z * cn);
+    if (n == nterms) {
+      for_channels<J>([&](auto jc, auto mc) {
+        constexpr int k = D::at(decltype(jc)::value, decltype(mc)::value);
+        q[k] = coupled(jc, mc, z2, x2, y2, v[k]);
+      });
+    } else {  // three terms and more: eta again
+      for_channels<J>([&](auto jc, auto mc) {
+        q[D::at(decltype(jc)::value, decltype(mc)::value)] = coupled(jc, mc, z2, x2, y2, eta(jc, mc));
+      });
+    }
+#pragma unroll
+    for (int k = 0; k < NROT; ++k) v[k] = q[k];
+  }
+  // ---- S = i theta M y_1, d1 = (V - 1) u + V^{1/2} S, mask, s' = s + (d2 + d1) + cfix s
+  float2 hi = make_float2(0.f, 0.f), lo = hi, rnd = hi;  // populations (ground, excited), compensated
+  float ab[2] = {0.f, 0.f};
+  {
+    const float2 z2 = dup2(f.x), x2 = dup2(f.y), y2 = dup2(f.z), cf = dup2(cfix);
+    const bool masked = mk < 1.f;
+    float2* const go = gs + t;
+    float b2 = 0.f;
+    for_channels<J>([&](auto jc, auto mc) {
+      constexpr int j = decltype(jc)::value, m = decltype(mc)::value, k = D::at(j, m), row = D::row(j, m), sf = j & 1;
+      const float2 S = coupled(jc, mc, z2, x2, y2, make_float2(0.f, 0.f));
+      const float2 s0 = s_at(row), d0 = d_at(row), u = add2(s0, d0), vh = vh_at(jc), vd = vd_at(jc);
+      float2 d1 = make_float2(fmaf(vd.x, u.x, fmaf(-vd.y, u.y, fmaf(vh.x, S.x, -vh.y * S.y))),
+                              fmaf(vd.x, u.y, fmaf(vd.y, u.x, fmaf(vh.x, S.y, vh.y * S.x))));
+      if (masked) {
+        const float2 p = add2(u, d1);
+        d1 = fma2(dup2(mk - 1.f), u, mul2(dup2(mk), d1));
+        ab[sf] += (1.f - mk * mk) * fmaf(p.x, p.x, p.y * p.y);
+      }
+      const float2 sn = round_update2(s0, add2(d0, d1), cf, rnd);
+      __stcs(go + row * NR, sn);
+      q[k] = sn;
+      const float b = fmaf(sn.x, sn.x, sn.y * sn.y);
+      if constexpr (sf == 1) acc2p(hi, lo, make_float2(j > (m < 0 ? -m : m) ? b2 : 0.f, b));  // compensated from the first term on
+      else if constexpr (j == J) acc2p(hi, lo, make_float2(b, 0.f));
+      else b2 = b;
+    });
+  }
+  // ---- dipole: over pairs of rows of one column (Z) and of columns m, m + 1 (S+, S-); each pair joins a
+  // ground and an excited row, and conj(g) e and conj(e) g give the same Re (P + M), Im (P - M)
+  float2 aX = make_float2(0.f, 0.f), aZ = aX;
+  float aY = 0.f;
+  if constexpr (!DIPR) {  // with d(R) the dipole is read from T^{1/2} s' by mol_dipole_r_kernel
+    for_channels<J>([&](auto jc, auto mc) {
+      constexpr int j = decltype(jc)::value, m = decltype(mc)::value, m1 = m + 1 < 0 ? -m - 1 : m + 1;
+      const float2 a = q[D::at(j, m)];
+      if constexpr (j < J) aZ = fma2(dup2(c_zu(j, m)), mul2(a, q[D::at(j + 1, m)]), aZ);
+      constexpr bool up = j + 1 <= J && j + 1 >= m1, dn = j - 1 >= m1;
+      if constexpr (up || dn) {
+        float2 r = make_float2(0.f, 0.f);
+        if constexpr (up) r = mul2(dup2(c_mu(j, m)), q[D::at(up ? j + 1 : j, up ? m + 1 : m)]);
+        if constexpr (up && dn) r = fma2(dup2(c_md(j, m)), q[D::at(dn ? j - 1 : j, dn ? m + 1 : m)], r);
+        else if constexpr (dn) r = mul2(dup2(c_md(j, m)), q[D::at(dn ? j - 1 : j, dn ? m + 1 : m)]);
+        aX = fma2(a, r, aX);
+        aY = fmaf(a.y, r.x, fmaf(-a.x, r.y, aY));
+      }
+    });
+  }
+  // ---- block reduction: populations compensated, the rest plain FP32
+  float r8[8] = {hi.x, hi.y, ab[0], ab[1], aX.x + aX.y, aY, 2.f * (aZ.x + aZ.y), rnd.x + rnd.y};
+  float l2[2] = {lo.x, lo.y};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float h2 = __shfl_xor_sync(0xffffffffu, r8[k], o);
+      const float g2 = __shfl_xor_sync(0xffffffffu, l2[k], o);
+      acc2(r8[k], l2[k], h2);
+      l2[k] += g2;
+    }
+#pragma unroll
+    for (int k = 2; k < 8; ++k) r8[k] += __shfl_xor_sync(0xffffffffu, r8[k], o);
+  }
+  if (lane == 0) {
+#pragma unroll
+    for (int k = 0; k < 7; ++k) s_red[w][k] = r8[k];
+    s_red[w][7] = l2[0];
+    s_red[w][8] = l2[1];
+    s_red[w][9] = r8[7];
+  }
+  __syncthreads();
+  if (t < 8) {
+    float h = 0.f, l = 0.f;
+    for (int ww = 0; ww < NW; ++ww) {
+      acc2(h, l, s_red[ww][t < 7 ? t : 9]);
+      if (t < 2) l += s_red[ww][7 + t];
+    }
+    s_fin[t] = h + l;
+    if (t < 2) s_fin_lo[t] = l - (s_fin[t] - h);
+  }
+  __syncthreads();
+  if (t < 3) {  // lab dipole: mu = O mu', mu' = d dR (Re(S+ + S-), Im(S+ - S-), 2 Re Z)
+    if constexpr (!DIPR) {
+      const float* O = md.rot + 9 * (long long)m_ + 3 * t;
+      const float lab = (float)sp.dipole * sp.dR * (O[0] * s_fin[4] + O[1] * s_fin[5] + O[2] * s_fin[6]);
+      const double nl = (double)lab;
+      md.dmu[3 * (long long)m_ + t] = nl - old;
+      md.mu[3 * (long long)m_ + t] = nl;
+    }
+  } else if (t < 5) {
+    const double P = ((double)s_fin[t - 3] + (double)s_fin_lo[t - 3]) * (double)sp.dR;
+    md.pop[2 * (long long)m_ + (t - 3)] = P;
+    if (!isfinite(P)) atomicOr(err, kErrNonFinite);
+  } else if (t < 7) {
+    md.absorbed[2 * (long long)m_ + (t - 5)] = old + (double)s_fin[t - 3] * (double)sp.dR;
+  } else if (t == 7) {
+    md.ncorr[m_] = rounding_feedback(s_fin[7], s_fin[0] + s_fin[1]);
+  }
+}
+
+template <int J, int NR, bool FUSED, bool DIPR>
+static void launch_rotor_t(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
+  constexpr int bytes = FUSED ? (2 * RotorDims<J>::NROT + 2) * NR * (int)sizeof(float2) : 0;
+  auto k = mol_rotor_kernel<J, NR, FUSED, DIPR>;
+  if (FUSED) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  }
+  k<<<sp.nmol, NR, bytes, s>>>(sp, md, err);
+}
+
+template <int J>
+static void launch_rotor_j(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
+  const bool fused = sp.path == MS_MOL_FUSED;  // N_r = 128
+  if (sp.dipw) {                               // d(R): N_r 64 or 128
+    if (fused) launch_rotor_t<J, 128, true, true>(sp, md, err, s);
+    else if (sp.nr == 128) launch_rotor_t<J, 128, false, true>(sp, md, err, s);
+    else launch_rotor_t<J, 64, false, true>(sp, md, err, s);
+  } else if (fused) launch_rotor_t<J, 128, true, false>(sp, md, err, s);
+  else if (sp.nr == 64) launch_rotor_t<J, 64, false, false>(sp, md, err, s);
+  else if (sp.nr == 128) launch_rotor_t<J, 128, false, false>(sp, md, err, s);
+  else launch_rotor_t<J, 256, false, false>(sp, md, err, s);
+}
+
+}  // namespace
+
+void launch_rotor(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
+  switch (sp.jmax) {
+    case 0: launch_rotor_j<0>(sp, md, err, s); break;
+    case 1: launch_rotor_j<1>(sp, md, err, s); break;
+    case 2: launch_rotor_j<2>(sp, md, err, s); break;
+    case 3: launch_rotor_j<3>(sp, md, err, s); break;
+    case 4: launch_rotor_j<4>(sp, md, err, s); break;
+  }
+}
+
+}  // namespace ms
