@@ -19,10 +19,10 @@
 // products, whose equal constants are immediates.
 //
 // What bounds it: issue slots and instruction fetch (2,900 instructions of
-// straight-line code at J = 4, about 85 a row and point; three CTAs of N_r = 128
-// an SM by registers), then HBM.  Per row and point of the reachable rows: the
-// R-space pass at J = 4, N_r = 64 (375,000 molecules) takes 4.57 ps, 5.3 TB/s,
-// against 7.13 for a thread per surface; the fused step at J = 4, N_r = 128
+// straight-line code at J = 4, about 85 a row and point; twelve warps an SM by
+// registers), then HBM.  Per row and point of the reachable rows: the R-space
+// pass at J = 4, N_r = 64 (375,000 molecules) takes 4.42 ps, 5.4 TB/s, against
+// 7.13 for a thread per surface; the fused step at J = 4, N_r = 128
 // (187,500 molecules) 6.87 against 12.14 ps.
 //
 // FUSED (N_r = 128): the kinetic pass runs in the same kernel.  The state
@@ -61,69 +61,39 @@ __device__ __forceinline__ void for_channels(F&& fn) {
   });
 }
 
-template <int J, int NR, bool FUSED, bool DIPR>
-__global__ void __launch_bounds__(NR, NR <= 64 ? 6 : (NR <= 128 ? 3 : 1))
-    mol_rotor_kernel(SpeciesDev sp, MolDev md, int* err) {
-  using D = RotorDims<J>;
-  constexpr int NROT = D::NROT, NW = NR / 32;
-  constexpr unsigned kStateBytes = (unsigned)NROT * NR * sizeof(float2);
-  extern __shared__ __align__(16) float4 smem4[];
-  float2* Sb = reinterpret_cast<float2*>(smem4);  // fused: [NROT][NR] s
-  float2* Db = Sb + NROT * NR;                    // fused: [NROT][NR] d2
-  float2* s_tw = Db + NROT * NR;                  // fused: [N2][N1] FFT twiddles
-  float2* s_kd = s_tw + NR;                       // fused: [NR] kinetic phase deltas
-  __shared__ __align__(8) unsigned long long s_bar[1];
-  __shared__ float s_red[NW][10];
-  __shared__ float s_fin[8], s_fin_lo[2];
+struct RotorSums {
+  float2 hi, lo;  // populations (ground, excited), compensated
+  float ab[2];    // absorbed norm
+  float2 x, z;    // dipole sums by parts
+  float y;
+  float2 rnd;     // rounding residual products
+};
 
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int lm = blockIdx.x, m_ = sp.mol[lm];
-  float2* const gs = sp.psi + (long long)lm * sp.mrows * NR;  // this molecule's state
-  if constexpr (FUSED) {
-    if (t == 0) {
-      mbar_init(&s_bar[0], 1);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      mbar_expect_tx(&s_bar[0], kStateBytes);
-      bulk_g2s(Sb, gs, kStateBytes, &s_bar[0]);
-    }
-    s_tw[t] = __ldg(&sp.twiddle[t]);
-    s_kd[t] = __ldg(&sp.kdelta[t]);
-  }
-  float4 f = __ldg(&sp.fld[lm]);  // (theta E'_z, theta E'_x/2, theta E'_y/2, terms)
-  if constexpr (DIPR) {           // times d(R) / max|d| at this thread's point
-    const float dw = __ldg(&sp.dipw[t]);
+// The R-space pass at one radial point p of a molecule: gs its state (global,
+// at p), ss and ds where s and d2 are read (at p; FUSED: shared memory).
+template <int J, int NR, bool FUSED, bool DIPR>
+__device__ __forceinline__ void rotor_point(const SpeciesDev& sp, int p, float2* gs, const float2* ss, const float2* ds,
+                                            float4 f, float cfix, RotorSums& a) {
+  using D = RotorDims<J>;
+  constexpr int NROT = D::NROT;
+  if constexpr (DIPR) {  // times d(R) / max|d| at this point
+    const float dw = __ldg(&sp.dipw[p]);
     f.x *= dw;
     f.y *= dw;
     f.z *= dw;
   }
   const int nterms = max(__float_as_int(f.w), 1);  // no field: one term of zeros
-  const float mk = sp.maskw[t].x;
-  const float cfix = md.ncorr[m_];  // rounding feedback of the previous step
-  // what the closing threads add to: the previous dipole, the absorbed norm so far
-  const double old = t < 3 ? md.mu[3 * (long long)m_ + t]
-                           : (t == 5 || t == 6 ? md.absorbed[2 * (long long)m_ + (t - 5)] : 0.0);
-  if constexpr (FUSED) {
-    __syncthreads();  // the barrier is initialised
-    const bool ok = mbar_wait_sleep(&s_bar[0], 0);
-    if (!__syncthreads_and(ok)) {
-      if (t == 0) atomicOr(err, kErrTimeout);
-      if (!ok) mbar_wait_sleep(&s_bar[0], 0);
-      return;
-    }
-    kinetic_pass<NR, NR, true>(Db, Sb, NROT, s_kd, s_tw);  // d2 = (T - 1) s
-  }
-  const float2* const ss = (FUSED ? Sb : gs) + t;
-  const float2* const ds = (FUSED ? Db : sp.d2 + (long long)lm * NROT * NR) + t;
+  const float mk = __ldg(&sp.maskw[p]).x;
   auto s_at = [&](int row) { return ss[row * NR]; };
   auto d_at = [&](int row) { return FUSED ? ds[row * NR] : __ldg(ds + row * NR); };
   // potential phases of shell j on the surface of its parity
   auto vh_at = [&](auto jc) {
     constexpr int j = decltype(jc)::value;
-    return __ldg(sp.vhalf + ((j & 1) * (J + 1) + j) * NR + t);
+    return __ldg(sp.vhalf + ((j & 1) * (J + 1) + j) * NR + p);
   };
   auto vd_at = [&](auto jc) {
     constexpr int j = decltype(jc)::value;
-    return __ldg(sp.vdelta + ((j & 1) * (J + 1) + j) * NR + t);
+    return __ldg(sp.vdelta + ((j & 1) * (J + 1) + j) * NR + p);
   };
 
   float2 v[NROT], q[NROT];
@@ -170,12 +140,9 @@ __global__ void __launch_bounds__(NR, NR <= 64 ? 6 : (NR <= 128 ? 3 : 1))
     for (int k = 0; k < NROT; ++k) v[k] = q[k];
   }
   // ---- S = i theta M y_1, d1 = (V - 1) u + V^{1/2} S, mask, s' = s + (d2 + d1) + cfix s
-  float2 hi = make_float2(0.f, 0.f), lo = hi, rnd = hi;  // populations (ground, excited), compensated
-  float ab[2] = {0.f, 0.f};
   {
     const float2 z2 = dup2(f.x), x2 = dup2(f.y), y2 = dup2(f.z), cf = dup2(cfix);
     const bool masked = mk < 1.f;
-    float2* const go = gs + t;
     float b2 = 0.f;
     for_channels<J>([&](auto jc, auto mc) {
       constexpr int j = decltype(jc)::value, m = decltype(mc)::value, k = D::at(j, m), row = D::row(j, m), sf = j & 1;
@@ -186,111 +153,211 @@ __global__ void __launch_bounds__(NR, NR <= 64 ? 6 : (NR <= 128 ? 3 : 1))
       if (masked) {
         const float2 p = add2(u, d1);
         d1 = fma2(dup2(mk - 1.f), u, mul2(dup2(mk), d1));
-        ab[sf] += (1.f - mk * mk) * fmaf(p.x, p.x, p.y * p.y);
+        a.ab[sf] += (1.f - mk * mk) * fmaf(p.x, p.x, p.y * p.y);
       }
-      const float2 sn = round_update2(s0, add2(d0, d1), cf, rnd);
-      __stcs(go + row * NR, sn);
+      const float2 sn = round_update2(s0, add2(d0, d1), cf, a.rnd);
+      __stcs(gs + row * NR, sn);
       q[k] = sn;
       const float b = fmaf(sn.x, sn.x, sn.y * sn.y);
-      if constexpr (sf == 1) acc2p(hi, lo, make_float2(j > (m < 0 ? -m : m) ? b2 : 0.f, b));  // compensated from the first term on
-      else if constexpr (j == J) acc2p(hi, lo, make_float2(b, 0.f));
+      if constexpr (sf == 1) acc2p(a.hi, a.lo, make_float2(j > (m < 0 ? -m : m) ? b2 : 0.f, b));  // compensated from the first term on
+      else if constexpr (j == J) acc2p(a.hi, a.lo, make_float2(b, 0.f));
       else b2 = b;
     });
   }
   // ---- dipole: over pairs of rows of one column (Z) and of columns m, m + 1 (S+, S-); each pair joins a
   // ground and an excited row, and conj(g) e and conj(e) g give the same Re (P + M), Im (P - M)
-  float2 aX = make_float2(0.f, 0.f), aZ = aX;
-  float aY = 0.f;
   if constexpr (!DIPR) {  // with d(R) the dipole is read from T^{1/2} s' by mol_dipole_r_kernel
     for_channels<J>([&](auto jc, auto mc) {
       constexpr int j = decltype(jc)::value, m = decltype(mc)::value, m1 = m + 1 < 0 ? -m - 1 : m + 1;
-      const float2 a = q[D::at(j, m)];
-      if constexpr (j < J) aZ = fma2(dup2(c_zu(j, m)), mul2(a, q[D::at(j + 1, m)]), aZ);
+      const float2 b = q[D::at(j, m)];
+      if constexpr (j < J) a.z = fma2(dup2(c_zu(j, m)), mul2(b, q[D::at(j + 1, m)]), a.z);
       constexpr bool up = j + 1 <= J && j + 1 >= m1, dn = j - 1 >= m1;
       if constexpr (up || dn) {
         float2 r = make_float2(0.f, 0.f);
         if constexpr (up) r = mul2(dup2(c_mu(j, m)), q[D::at(up ? j + 1 : j, up ? m + 1 : m)]);
         if constexpr (up && dn) r = fma2(dup2(c_md(j, m)), q[D::at(dn ? j - 1 : j, dn ? m + 1 : m)], r);
         else if constexpr (dn) r = mul2(dup2(c_md(j, m)), q[D::at(dn ? j - 1 : j, dn ? m + 1 : m)]);
-        aX = fma2(a, r, aX);
-        aY = fmaf(a.y, r.x, fmaf(-a.x, r.y, aY));
+        a.x = fma2(b, r, a.x);
+        a.y = fmaf(b.y, r.x, fmaf(-b.x, r.y, a.y));
       }
     });
   }
-  // ---- block reduction: populations compensated, the rest plain FP32
-  float r8[8] = {hi.x, hi.y, ab[0], ab[1], aX.x + aX.y, aY, 2.f * (aZ.x + aZ.y), rnd.x + rnd.y};
-  float l2[2] = {lo.x, lo.y};
+}
+
+// A molecule's sums over its lanes, populations compensated, the rest plain
+// FP32: r[0..7] = P_g, P_e, absorbed, Re(S+ + S-), Im(S+ - S-), 2 Re Z, the
+// rounding residuals; l the low parts of the populations.
+__device__ __forceinline__ void rotor_warp_sum(const RotorSums& a, float (&r)[8], float (&l)[2]) {
+  const float v[8] = {a.hi.x, a.hi.y, a.ab[0], a.ab[1], a.x.x + a.x.y, a.y, 2.f * (a.z.x + a.z.y), a.rnd.x + a.rnd.y};
+  l[0] = a.lo.x;
+  l[1] = a.lo.y;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) r[k] = v[k];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const float h2 = __shfl_xor_sync(0xffffffffu, r8[k], o);
-      const float g2 = __shfl_xor_sync(0xffffffffu, l2[k], o);
-      acc2(r8[k], l2[k], h2);
-      l2[k] += g2;
+      const float h2 = __shfl_xor_sync(0xffffffffu, r[k], o);
+      const float g2 = __shfl_xor_sync(0xffffffffu, l[k], o);
+      acc2(r[k], l[k], h2);
+      l[k] += g2;
     }
 #pragma unroll
-    for (int k = 2; k < 8; ++k) r8[k] += __shfl_xor_sync(0xffffffffu, r8[k], o);
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < 7; ++k) s_red[w][k] = r8[k];
-    s_red[w][7] = l2[0];
-    s_red[w][8] = l2[1];
-    s_red[w][9] = r8[7];
-  }
-  __syncthreads();
-  if (t < 8) {
-    float h = 0.f, l = 0.f;
-    for (int ww = 0; ww < NW; ++ww) {
-      acc2(h, l, s_red[ww][t < 7 ? t : 9]);
-      if (t < 2) l += s_red[ww][7 + t];
-    }
-    s_fin[t] = h + l;
-    if (t < 2) s_fin_lo[t] = l - (s_fin[t] - h);
-  }
-  __syncthreads();
-  if (t < 3) {  // lab dipole: mu = O mu', mu' = d dR (Re(S+ + S-), Im(S+ - S-), 2 Re Z)
-    if constexpr (!DIPR) {
-      const float* O = md.rot + 9 * (long long)m_ + 3 * t;
-      const float lab = (float)sp.dipole * sp.dR * (O[0] * s_fin[4] + O[1] * s_fin[5] + O[2] * s_fin[6]);
-      const double nl = (double)lab;
-      md.dmu[3 * (long long)m_ + t] = nl - old;
-      md.mu[3 * (long long)m_ + t] = nl;
-    }
-  } else if (t < 5) {
-    const double P = ((double)s_fin[t - 3] + (double)s_fin_lo[t - 3]) * (double)sp.dR;
-    md.pop[2 * (long long)m_ + (t - 3)] = P;
-    if (!isfinite(P)) atomicOr(err, kErrNonFinite);
-  } else if (t < 7) {
-    md.absorbed[2 * (long long)m_ + (t - 5)] = old + (double)s_fin[t - 3] * (double)sp.dR;
-  } else if (t == 7) {
-    md.ncorr[m_] = rounding_feedback(s_fin[7], s_fin[0] + s_fin[1]);
+    for (int k = 2; k < 8; ++k) r[k] += __shfl_xor_sync(0xffffffffu, r[k], o);
   }
 }
 
-template <int J, int NR, bool FUSED, bool DIPR>
-static void launch_rotor_t(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
-  constexpr int bytes = FUSED ? (2 * RotorDims<J>::NROT + 2) * NR * (int)sizeof(float2) : 0;
-  auto k = mol_rotor_kernel<J, NR, FUSED, DIPR>;
-  if (FUSED) {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+// What the closing threads t < 8 of a molecule hold from before its step.
+__device__ __forceinline__ double rotor_old(const MolDev& md, int m, int t) {
+  return t < 3 ? md.mu[3 * (long long)m + t]
+               : (t == 5 || t == 6 ? md.absorbed[2 * (long long)m + (t - 5)] : 0.0);
+}
+
+// The molecule's outputs from its sums, by threads t < 8.
+template <bool DIPR>
+__device__ __forceinline__ void rotor_close(const SpeciesDev& sp, const MolDev& md, int m, int t, double old,
+                                            const float* fin, const float* fin_lo, int* err) {
+  if (t < 3) {  // lab dipole: mu = O mu', mu' = d dR (Re(S+ + S-), Im(S+ - S-), 2 Re Z)
+    if constexpr (!DIPR) {  // with d(R) the dipole is read from T^{1/2} s' by mol_dipole_r_kernel
+      const float* O = md.rot + 9 * (long long)m + 3 * t;
+      const float lab = (float)sp.dipole * sp.dR * (O[0] * fin[4] + O[1] * fin[5] + O[2] * fin[6]);
+      const double nl = (double)lab;
+      md.dmu[3 * (long long)m + t] = nl - old;
+      md.mu[3 * (long long)m + t] = nl;
+    }
+  } else if (t < 5) {
+    const double P = ((double)fin[t - 3] + (double)fin_lo[t - 3]) * (double)sp.dR;
+    md.pop[2 * (long long)m + (t - 3)] = P;
+    if (!isfinite(P)) atomicOr(err, kErrNonFinite);
+  } else if (t < 7) {
+    md.absorbed[2 * (long long)m + (t - 5)] = old + (double)fin[t - 3] * (double)sp.dR;
+  } else if (t == 7) {
+    md.ncorr[m] = rounding_feedback(fin[7], fin[0] + fin[1]);
   }
+}
+
+// The fused step: one CTA of N_r threads a molecule.
+template <int J, int NR, bool DIPR>
+__global__ void __launch_bounds__(NR, 3) mol_rotor_fused_kernel(SpeciesDev sp, MolDev md, int* err) {
+  constexpr int NROT = RotorDims<J>::NROT, NW = NR / 32;
+  constexpr unsigned kStateBytes = (unsigned)NROT * NR * sizeof(float2);
+  extern __shared__ __align__(16) float4 smem4[];
+  float2* Sb = reinterpret_cast<float2*>(smem4);  // [NROT][NR] s
+  float2* Db = Sb + NROT * NR;                    // [NROT][NR] d2
+  float2* s_tw = Db + NROT * NR;                  // [N2][N1] FFT twiddles
+  float2* s_kd = s_tw + NR;                       // [NR] kinetic phase deltas
+  __shared__ __align__(8) unsigned long long s_bar[1];
+  __shared__ float s_red[NW][10];
+  __shared__ float s_fin[8], s_fin_lo[2];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int lm = blockIdx.x, m = sp.mol[lm];
+  float2* const gs = sp.psi + (long long)lm * sp.mrows * NR;  // this molecule's state
+  if (t == 0) {
+    mbar_init(&s_bar[0], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_expect_tx(&s_bar[0], kStateBytes);
+    bulk_g2s(Sb, gs, kStateBytes, &s_bar[0]);
+  }
+  s_tw[t] = __ldg(&sp.twiddle[t]);
+  s_kd[t] = __ldg(&sp.kdelta[t]);
+  const float4 f = __ldg(&sp.fld[lm]);  // (theta E'_z, theta E'_x/2, theta E'_y/2, terms)
+  const float cfix = md.ncorr[m];       // rounding feedback of the previous step
+  const double old = rotor_old(md, m, t);
+  __syncthreads();  // the barrier is initialised
+  const bool ok = mbar_wait_sleep(&s_bar[0], 0);
+  if (!__syncthreads_and(ok)) {
+    if (t == 0) atomicOr(err, kErrTimeout);
+    if (!ok) mbar_wait_sleep(&s_bar[0], 0);
+    return;
+  }
+  kinetic_pass<NR, NR, true>(Db, Sb, NROT, s_kd, s_tw);  // d2 = (T - 1) s
+  RotorSums a = {};
+  rotor_point<J, NR, true, DIPR>(sp, t, gs + t, Sb + t, Db + t, f, cfix, a);
+  float r[8], l[2];
+  rotor_warp_sum(a, r, l);
+  if (lane == 0) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s_red[w][k] = r[k];
+    s_red[w][8] = l[0];
+    s_red[w][9] = l[1];
+  }
+  __syncthreads();
+  if (t < 8) {
+    float h = 0.f, lo = 0.f;
+    for (int ww = 0; ww < NW; ++ww) {
+      acc2(h, lo, s_red[ww][t]);
+      if (t < 2) lo += s_red[ww][8 + t];
+    }
+    s_fin[t] = h + lo;
+    if (t < 2) s_fin_lo[t] = lo - (s_fin[t] - h);
+  }
+  __syncthreads();
+  rotor_close<DIPR>(sp, md, m, t, old, s_fin, s_fin_lo, err);
+}
+
+// The streaming R-space pass: two warps a molecule, each 32 points at a time, so
+// that the closing sums (a third of the instructions at J = 1) are paid twice a
+// molecule and not once for every 32 points.  Per row and point, against a warp
+// for every 32 points: J = 4, N_r = 256 6.56 -> 4.68 ps, J = 1, N_r = 64 7.91 ->
+// 6.76 ps; one warp a molecule: 5.13 against 4.42 ps at J = 4, N_r = 64.
+template <int J, int NR, bool DIPR>
+__global__ void __launch_bounds__(64, 6) mol_rotor_kernel(SpeciesDev sp, MolDev md, int* err) {
+  constexpr int NROT = RotorDims<J>::NROT;
+  __shared__ float s_red[2][10], s_fin[10];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int lm = blockIdx.x, m = sp.mol[lm];
+  float2* const gs = sp.psi + (long long)lm * sp.mrows * NR + lane;
+  const float2* const ds = sp.d2 + (long long)lm * NROT * NR + lane;
+  const float4 f = __ldg(&sp.fld[lm]);  // (theta E'_z, theta E'_x/2, theta E'_y/2, terms)
+  const float cfix = md.ncorr[m];       // rounding feedback of the previous step
+  const double old = rotor_old(md, m, t);
+  RotorSums a = {};
+#pragma unroll 1
+  for (int p = 32 * w; p < NR; p += 64) rotor_point<J, NR, false, DIPR>(sp, p + lane, gs + p, gs + p, ds + p, f, cfix, a);
+  float r[8], l[2];
+  rotor_warp_sum(a, r, l);
+  if (lane == 0) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s_red[w][k] = r[k];
+    s_red[w][8] = l[0];
+    s_red[w][9] = l[1];
+  }
+  __syncthreads();
+  if (w != 0) return;
+  if (lane < 8) {
+    float h = s_red[0][lane], lo = lane < 2 ? s_red[0][8 + lane] + s_red[1][8 + lane] : 0.f;
+    acc2(h, lo, s_red[1][lane]);
+    s_fin[lane] = h + lo;
+    if (lane < 2) s_fin[8 + lane] = lo - (s_fin[lane] - h);
+  }
+  __syncwarp();
+  rotor_close<DIPR>(sp, md, m, lane, old, s_fin, s_fin + 8, err);
+}
+
+template <int J, int NR, bool DIPR>
+static void launch_rotor_fused(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
+  constexpr int bytes = (2 * RotorDims<J>::NROT + 2) * NR * (int)sizeof(float2);
+  auto k = mol_rotor_fused_kernel<J, NR, DIPR>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   k<<<sp.nmol, NR, bytes, s>>>(sp, md, err);
+}
+template <int J, int NR, bool DIPR>
+static void launch_rotor_streaming(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
+  mol_rotor_kernel<J, NR, DIPR><<<sp.nmol, 64, 0, s>>>(sp, md, err);
 }
 
 template <int J>
 static void launch_rotor_j(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
   const bool fused = sp.path == MS_MOL_FUSED;  // N_r = 128
   if (sp.dipw) {                               // d(R): N_r 64 or 128
-    if (fused) launch_rotor_t<J, 128, true, true>(sp, md, err, s);
-    else if (sp.nr == 128) launch_rotor_t<J, 128, false, true>(sp, md, err, s);
-    else launch_rotor_t<J, 64, false, true>(sp, md, err, s);
-  } else if (fused) launch_rotor_t<J, 128, true, false>(sp, md, err, s);
-  else if (sp.nr == 64) launch_rotor_t<J, 64, false, false>(sp, md, err, s);
-  else if (sp.nr == 128) launch_rotor_t<J, 128, false, false>(sp, md, err, s);
-  else launch_rotor_t<J, 256, false, false>(sp, md, err, s);
+    if (fused) launch_rotor_fused<J, 128, true>(sp, md, err, s);
+    else if (sp.nr == 128) launch_rotor_streaming<J, 128, true>(sp, md, err, s);
+    else launch_rotor_streaming<J, 64, true>(sp, md, err, s);
+  } else if (fused) launch_rotor_fused<J, 128, false>(sp, md, err, s);
+  else if (sp.nr == 64) launch_rotor_streaming<J, 64, false>(sp, md, err, s);
+  else if (sp.nr == 128) launch_rotor_streaming<J, 128, false>(sp, md, err, s);
+  else launch_rotor_streaming<J, 256, false>(sp, md, err, s);
 }
 
 }  // namespace
