@@ -3,10 +3,13 @@
 // polarization current (section "The domain decomposition methodology for
 // FDTD"; coupling section for dP/dt).
 //
-// Both half steps are HBM-bound stencils: a thread marches along z through
-// one (i, j) column, x fastest across the lanes so that a warp touches 128
-// contiguous bytes per component; the z neighbour stays in registers, the x
-// neighbour comes from the adjacent lane, the y neighbour through L1/L2.
+// Both half steps are stencils bound by HBM (grids beyond L2) or by the loads
+// in flight.  A thread marches along z through four neighbouring columns (x to
+// x + 3, 16-byte loads), the lanes running over the plane's quads in storage
+// order; the z neighbour stays in registers, the x neighbour comes from the
+// adjacent lane, the y neighbour through L1/L2.  Rows that are no multiple of
+// four cells take the kernels with one column a thread, which issue about 180
+// instructions for 32 cells of a plane where these issue about 130 for 128.
 #include "ms_internal.cuh"
 
 namespace ms {
@@ -54,24 +57,22 @@ __device__ __forceinline__ long long pml_index(const Grid& g, int s, int k, int 
 // Incident line, H half step (one block per sim).  Node m of the line sits
 // at z = (ks - 2 + m) dx; only nodes inside the numerical light cone of the
 // source (m <= step + 2) can be non-zero, so only those are touched.
-__device__ void aux_h_block(const Grid& g, int s) {
+__device__ void aux_h_block(const Grid& g, int s, int t, int nt) {
   const long long n = *g.step;
   const int lim = (int)min((long long)g.aux_len, n + 4);
   float* E1 = g.auxE + (long long)s * (g.aux_len + 1);
   float* H1 = g.auxH + (long long)s * g.aux_len;
-  const int t = threadIdx.y * kTx + threadIdx.x;
-  for (int m = t; m < lim; m += kTx * kTy) H1[m] -= g.ch * (E1[m + 1] - E1[m]);
+  for (int m = t; m < lim; m += nt) H1[m] -= g.ch * (E1[m + 1] - E1[m]);
 }
 
 // Incident line, E half step, and the new source sample at its node 0.
-__device__ void aux_e_block(const Grid& g, int s) {
+__device__ void aux_e_block(const Grid& g, int s, int t, int nt) {
   const long long n = *g.step;
   const int lim = (int)min((long long)g.aux_len, n + 4);
   float* E1 = g.auxE + (long long)s * (g.aux_len + 1);
   const float* H1 = g.auxH + (long long)s * g.aux_len;
   const float ce = g.ce_vac;
-  const int t = threadIdx.y * kTx + threadIdx.x;
-  for (int m = 1 + t; m < lim; m += kTx * kTy) E1[m] += ce * (0.f - (H1[m] - H1[m - 1]));
+  for (int m = 1 + t; m < lim; m += nt) E1[m] += ce * (0.f - (H1[m] - H1[m - 1]));
   if (t == 0) E1[0] = (float)incident_field(g.src[s], (double)(n + 1) * g.dt);
 }
 
@@ -85,7 +86,7 @@ struct HPlane {
 
 __global__ void __launch_bounds__(kTx * kTy, 6) yee_h_kernel(Grid g, int ntiles) {
   if ((int)blockIdx.x >= ntiles) {
-    aux_h_block(g, (int)blockIdx.x - ntiles);
+    aux_h_block(g, (int)blockIdx.x - ntiles, threadIdx.y * kTx + threadIdx.x, kTx * kTy);
     return;
   }
   const Tile t = tile_of(g, blockIdx.x);
@@ -172,7 +173,7 @@ struct EPlane {
 
 __global__ void __launch_bounds__(kTx * kTy, 5) yee_e_kernel(Grid g, int ntiles) {
   if ((int)blockIdx.x >= ntiles) {
-    aux_e_block(g, (int)blockIdx.x - ntiles);
+    aux_e_block(g, (int)blockIdx.x - ntiles, threadIdx.y * kTx + threadIdx.x, kTx * kTy);
     return;
   }
   const Tile t = tile_of(g, blockIdx.x);
@@ -290,16 +291,276 @@ __global__ void __launch_bounds__(kTx * kTy, 5) yee_e_kernel(Grid g, int ntiles)
   }
 }
 
+// ---- four columns a thread ---------------------------------------------------
+// Phases of a step, H and E half step: 256^3 with a 100 nm film 118 -> 101 us
+// (6.0 TB/s) and 144 -> 137 us; 128 x 128 x 192, whose fields stay in L2, 29 ->
+// 18 us and 31 -> 21 us; 32 x 32 x 64 10.3 -> 6.6 us and 13.4 -> 9.9 us.
+// A thread takes quad q of the plane (row j = q / (nx/4), cells 4 i4 .. 4 i4 + 3)
+// and kz planes.  Quads past the plane load the last one and store nothing.
+constexpr int kQt = 128;  // threads a block
+
+struct Quad {
+  int i, j, s, k0, k1;  // first cell, row, sim, planes
+  bool in, last, first; // in the plane; the row's last, first quad
+};
+
+__device__ __forceinline__ Quad quad_of(const Grid& g, int b, int kz) {
+  const int n4 = g.nx >> 2, np = n4 * g.ny, tq = (np + kQt - 1) / kQt, tz = (g.nz + kz - 1) / kz;
+  Quad t;
+  int q = (b % tq) * kQt + (int)threadIdx.x;
+  b /= tq;
+  t.in = q < np;
+  q = min(q, np - 1);
+  t.j = q / n4;
+  const int i4 = q - t.j * n4;
+  t.i = 4 * i4;
+  t.first = i4 == 0;
+  t.last = i4 == n4 - 1;
+  t.k0 = (b % tz) * kz;
+  t.k1 = min(t.k0 + kz, g.nz);
+  t.s = b / tz;
+  return t;
+}
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ float4 operator-(float4 a, float4 b) {
+  return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
+__device__ __forceinline__ float4 operator+(float4 a, float4 b) {
+  return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+// a x + b y
+__device__ __forceinline__ float4 comb4(float a, float4 x, float b, float4 y) {
+  return make_float4(a * x.x + b * y.x, a * x.y + b * y.y, a * x.z + b * y.z, a * x.w + b * y.w);
+}
+// h - c d
+__device__ __forceinline__ float4 sub_mul4(float4 h, float c, float4 d) {
+  return make_float4(h.x - c * d.x, h.y - c * d.y, h.z - c * d.z, h.w - c * d.w);
+}
+// the quad moved by one cell: (b, c, d, next quad's a) and (previous quad's d, a, b, c)
+__device__ __forceinline__ float4 up_x(float4 v, float edge, bool shuffled) {
+  const float n = __shfl_down_sync(0xffffffffu, v.x, 1);
+  return make_float4(v.y, v.z, v.w, shuffled ? n : edge);
+}
+__device__ __forceinline__ float4 down_x(float4 v, float edge, bool shuffled) {
+  const float n = __shfl_up_sync(0xffffffffu, v.w, 1);
+  return make_float4(shuffled ? n : edge, v.x, v.y, v.z);
+}
+
+// H^{n-1/2} -> H^{n+1/2} (the arithmetic of yee_h_kernel)
+__global__ void __launch_bounds__(kQt) yee_h4_kernel(Grid g, int ntiles, int kz) {
+  if ((int)blockIdx.x >= ntiles) {
+    aux_h_block(g, (int)blockIdx.x - ntiles, threadIdx.x, kQt);
+    return;
+  }
+  const Quad t = quad_of(g, blockIdx.x, kz);
+  const int sxy = g.nx * g.ny;
+  const int dy = t.j + 1 < g.ny ? g.nx : -(g.ny - 1) * g.nx;
+  const int dx = t.last ? 4 - g.nx : 4;                      // to the first cell of the next quad of the row
+  const bool xsh = (threadIdx.x & 31) < 31 && !t.last;       // the next lane holds it
+  const long long sb = (long long)t.s * g.ncell_sim;
+  const float* __restrict__ Ex = g.E[0] + sb;
+  const float* __restrict__ Ey = g.E[1] + sb;
+  const float* __restrict__ Ez = g.E[2] + sb;
+  float* __restrict__ H0 = g.H[0] + sb;
+  float* __restrict__ H1 = g.H[1] + sb;
+  float* __restrict__ H2 = g.H[2] + sb;
+  int c = t.k0 * sxy + t.j * g.nx + t.i;
+  float4 ex = ld4(Ex + c), ey = ld4(Ey + c);
+  for (int k = t.k0; k < t.k1; ++k, c += sxy) {
+    const bool top = k + 1 >= g.nz;
+    const int cz = c + (top ? -(g.nz - 1) * sxy : sxy);
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const bool zero_top = top && !g.periodic_z;
+    const float4 ex_z = zero_top ? z4 : ld4(Ex + cz), ey_z = zero_top ? z4 : ld4(Ey + cz);
+    const float4 ez = ld4(Ez + c), ez_y = ld4(Ez + c + dy), ex_y = ld4(Ex + c + dy);
+    const float4 h0 = ld4(H0 + c), h1 = ld4(H1 + c), h2 = ld4(H2 + c);
+    const float ez_e = xsh ? 0.f : Ez[c + dx], ey_e = xsh ? 0.f : Ey[c + dx];
+    const float4 dEz_dy = ez_y - ez, dEx_dy = ex_y - ex;
+    float4 dEy_dz = ey_z - ey, dEx_dz = ex_z - ex;
+    const float4 dEz_dx = up_x(ez, ez_e, xsh) - ez, dEy_dx = up_x(ey, ey_e, xsh) - ey;
+    if (g.pml > 0 && (k < g.pml || k >= g.nz - g.pml)) {
+      const float4 co = g.cpml[k];  // (bE, aE, bH, aH); psi stored times dx
+      const long long q = pml_index(g, t.s, k, t.j, t.i);
+      const float4 px = comb4(co.z, ld4(g.psiH[0] + q), co.w, dEy_dz);
+      const float4 py = comb4(co.z, ld4(g.psiH[1] + q), co.w, dEx_dz);
+      if (t.in) {
+        st4(g.psiH[0] + q, px);
+        st4(g.psiH[1] + q, py);
+      }
+      dEy_dz = dEy_dz + px;
+      dEx_dz = dEx_dz + py;
+    }
+    if (t.in) {
+      st4(H0 + c, sub_mul4(h0, g.ch, dEz_dy - dEy_dz));
+      float4 n1 = sub_mul4(h1, g.ch, dEx_dz - dEz_dx);
+      if (k == g.ks - 1) {
+        const float a = g.auxE[(long long)t.s * (g.aux_len + 1) + 2];
+        n1 = make_float4(fmaf(g.ch, a, n1.x), fmaf(g.ch, a, n1.y), fmaf(g.ch, a, n1.z), fmaf(g.ch, a, n1.w));
+      }
+      st4(H1 + c, n1);
+      st4(H2 + c, sub_mul4(h2, g.ch, dEy_dx - dEx_dy));
+    }
+    ex = ex_z;
+    ey = ey_z;
+  }
+}
+
+// E^n -> E^{n+1} (the arithmetic of yee_e_kernel)
+__global__ void __launch_bounds__(kQt) yee_e4_kernel(Grid g, int ntiles, int kz) {
+  if ((int)blockIdx.x >= ntiles) {
+    aux_e_block(g, (int)blockIdx.x - ntiles, threadIdx.x, kQt);
+    return;
+  }
+  const Quad t = quad_of(g, blockIdx.x, kz);
+  const int sxy = g.nx * g.ny;
+  const int dy = t.j > 0 ? g.nx : -(g.ny - 1) * g.nx;
+  const int dx = t.first ? g.nx - 1 : -1;                    // to the last cell of the previous quad of the row
+  const bool xsh = (threadIdx.x & 31) > 0 && !t.first;       // the previous lane holds it
+  const long long sb = (long long)t.s * g.ncell_sim;
+  const float* __restrict__ Hx = g.H[0] + sb;
+  const float* __restrict__ Hy = g.H[1] + sb;
+  const float* __restrict__ Hz = g.H[2] + sb;
+  float* const E[3] = {g.E[0] + sb, g.E[1] + sb, g.E[2] + sb};
+  int c = t.k0 * sxy + t.j * g.nx + t.i;
+  float4 hx_m = make_float4(0.f, 0.f, 0.f, 0.f), hy_m = hx_m;  // plane k - 1
+  if (t.k0 > 0 || g.periodic_z) {
+    const int cm = t.k0 > 0 ? c - sxy : c + (g.nz - 1) * sxy;
+    hx_m = ld4(Hx + cm);
+    hy_m = ld4(Hy + cm);
+  }  // else: perfect conductor below the bottom plane
+  for (int k = t.k0; k < t.k1; ++k, c += sxy) {
+    const float4 hx = ld4(Hx + c), hy = ld4(Hy + c), hz = ld4(Hz + c), hz_y = ld4(Hz + c - dy), hx_y = ld4(Hx + c - dy);
+    const float4 e0 = ld4(E[0] + c), e1 = ld4(E[1] + c), e2 = ld4(E[2] + c);
+    const unsigned mats = *reinterpret_cast<const unsigned*>(g.mat + sb + c);
+    const float hz_e = xsh ? 0.f : Hz[c + dx], hy_e = xsh ? 0.f : Hy[c + dx];
+    const float4 dHz_dy = hz - hz_y, dHx_dy = hx - hx_y;
+    float4 dHy_dz = hy - hy_m, dHx_dz = hx - hx_m;
+    const float4 dHz_dx = hz - down_x(hz, hz_e, xsh), dHy_dx = hy - down_x(hy, hy_e, xsh);
+    hx_m = hx;
+    hy_m = hy;
+    if (g.pml > 0 && (k < g.pml || k >= g.nz - g.pml)) {
+      const float4 co = g.cpml[k];
+      const long long q = pml_index(g, t.s, k, t.j, t.i);
+      const float4 px = comb4(co.x, ld4(g.psiE[0] + q), co.y, dHy_dz);
+      const float4 py = comb4(co.x, ld4(g.psiE[1] + q), co.y, dHx_dz);
+      if (t.in) {
+        st4(g.psiE[0] + q, px);
+        st4(g.psiE[1] + q, py);
+      }
+      dHy_dz = dHy_dz + px;
+      dHx_dz = dHx_dz + py;
+    }
+    float4 cx = dHz_dy - dHy_dz;
+    const float4 cy = dHx_dz - dHz_dx, cz = dHy_dx - dHx_dy;
+    if (k == g.ks) {
+      const float a = g.auxH[(long long)t.s * g.aux_len + 1];
+      cx = cx + make_float4(a, a, a, a);
+    }
+    if (!t.in) continue;
+    float ev[3][4] = {{e0.x, e0.y, e0.z, e0.w}, {e1.x, e1.y, e1.z, e1.w}, {e2.x, e2.y, e2.z, e2.w}};
+    const float cv[3][4] = {{cx.x, cx.y, cx.z, cx.w}, {cy.x, cy.y, cy.z, cy.w}, {cz.x, cz.y, cz.z, cz.w}};
+    float jv[3][4] = {};
+    if (k >= g.jk0 && k < g.jk1) {  // the slab that holds metal cells
+      bool any = false;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) any = any || g.mc[(mats >> (8 * a)) & 255u].metal;
+      if (any) {
+        const long long jj = (((long long)t.s * (g.jk1 - g.jk0) + (k - g.jk0)) * g.ny + t.j) * g.nx + t.i;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          const float4 j0 = ld4(g.J[d] + jj);
+          float jo[4] = {j0.x, j0.y, j0.z, j0.w};
+#pragma unroll
+          for (int a = 0; a < 4; ++a) {
+            const MaterialCoef& mc = g.mc[(mats >> (8 * a)) & 255u];
+            if (mc.metal) jv[d][a] = jo[a] = mc.alpha * jo[a] + mc.beta * ev[d][a];
+          }
+          st4(g.J[d] + jj, make_float4(jo[0], jo[1], jo[2], jo[3]));
+        }
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const MaterialCoef& mc = g.mc[(mats >> (8 * a)) & 255u];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) ev[d][a] += mc.ce * cv[d][a] - mc.cj * jv[d][a];
+    }
+    if (k >= g.mk0 && k < g.mk1) {  // the molecular slab
+      const long long sl = (((long long)t.s * (g.mk1 - g.mk0) + (k - g.mk0)) * g.ny + t.j) * g.nx + t.i;
+      const int4 o4 = *reinterpret_cast<const int4*>(g.cell_off + sl);
+      const int off[5] = {o4.x, o4.y, o4.z, o4.w, g.cell_off[sl + 4]};
+      if (off[4] > off[0]) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          if (off[a + 1] == off[a]) continue;
+          double px = 0.0, py = 0.0, pz = 0.0;  // ensemble sum in FP64
+          for (int q = off[a]; q < off[a + 1]; ++q) {
+            const int m = g.cell_mol[q];
+            px += g.dmu[3 * (long long)m + 0];
+            py += g.dmu[3 * (long long)m + 1];
+            pz += g.dmu[3 * (long long)m + 2];
+          }
+          const float cp = g.mc[(mats >> (8 * a)) & 255u].cp;
+          ev[0][a] -= cp * (float)px;
+          ev[1][a] -= cp * (float)py;
+          ev[2][a] -= cp * (float)pz;
+        }
+      }
+    }
+    if (!g.periodic_z && k == 0) {  // tangential E on the bottom conductor
+#pragma unroll
+      for (int a = 0; a < 4; ++a) ev[0][a] = ev[1][a] = 0.f;
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) st4(E[d] + c, make_float4(ev[d][0], ev[d][1], ev[d][2], ev[d][3]));
+  }
+}
+
 __global__ void step_counter_kernel(long long* step) { *step += 1; }
 
+// The quad kernels take rows of whole quads and arrays on 16-byte boundaries
+// (mat: 4, cell_off: 16); an allocator of the caller may place them anywhere.
+static bool quads_ok(const Grid& g) {
+  if (g.nx % 4 != 0) return false;
+  uintptr_t a = 0;
+  for (int c = 0; c < 3; ++c) a |= (uintptr_t)g.E[c] | (uintptr_t)g.H[c] | (uintptr_t)g.J[c];
+  if (g.pml > 0)
+    for (int c = 0; c < 2; ++c) a |= (uintptr_t)g.psiE[c] | (uintptr_t)g.psiH[c];
+  a |= (uintptr_t)g.cell_off | ((uintptr_t)g.mat & 3) << 2;
+  return (a & 15) == 0;
+}
+// Planes a thread: eight where that leaves every SM enough warps (about 64), fewer
+// on small grids, whose half steps are as long as one thread's walk.
+static int quad_planes(const Grid& g) {
+  const long long quads = g.ncell_sim / 4 * g.nsim;
+  const long long kz = quads / (152LL * 64 * 32);
+  return (int)(kz < 1 ? 1 : (kz > 8 ? 8 : kz));
+}
+static int quad_tiles(const Grid& g, int kz) {
+  return ((g.nx / 4 * g.ny + kQt - 1) / kQt) * ((g.nz + kz - 1) / kz) * g.nsim;
+}
 
 void launch_yee_h(const Grid& g, cudaStream_t s) {
+  const int aux = g.ks >= 0 ? g.nsim : 0;
+  if (quads_ok(g)) {
+    const int kz = quad_planes(g), nt = quad_tiles(g, kz);
+    yee_h4_kernel<<<nt + aux, kQt, 0, s>>>(g, nt, kz);
+    return;
+  }
   const int nt = yee_tiles(g);
-  yee_h_kernel<<<nt + (g.ks >= 0 ? g.nsim : 0), dim3(kTx, kTy), 0, s>>>(g, nt);
+  yee_h_kernel<<<nt + aux, dim3(kTx, kTy), 0, s>>>(g, nt);
 }
 void launch_yee_e(const Grid& g, cudaStream_t s) {
+  const int aux = g.ks >= 0 ? g.nsim : 0;
+  if (quads_ok(g)) {
+    const int kz = quad_planes(g), nt = quad_tiles(g, kz);
+    yee_e4_kernel<<<nt + aux, kQt, 0, s>>>(g, nt, kz);
+    return;
+  }
   const int nt = yee_tiles(g);
-  yee_e_kernel<<<nt + (g.ks >= 0 ? g.nsim : 0), dim3(kTx, kTy), 0, s>>>(g, nt);
+  yee_e_kernel<<<nt + aux, dim3(kTx, kTy), 0, s>>>(g, nt);
 }
 // E^n at the cells of listed molecules (the coupled step's gather)
 __global__ void record_fields_kernel(Grid g, const int* cell, const long long* ids, int m, float* out) {
