@@ -84,6 +84,7 @@ struct ms_sim {
   // device address of the library's fixed scratch array (ms_step_noalloc),
   // looked up at create with the handle's device current; null if that failed
   float2* noalloc_base = nullptr;
+  int dft_kept = 0;  // detector samples kept and not yet added; 0 between calls
   std::vector<double> pop_init;  // create only: populations at t = 0, uploaded in one copy
   // phase timing
   bool timing = false;
@@ -1156,7 +1157,9 @@ static int pipelined_molecules(ms_sim* s, const ms::SpeciesDev* sp, int prescrib
   return launched;
 }
 
-static void step_once(ms_sim* s, float2* const* scratch, const FieldRecorder* rec = nullptr) {
+// `last`: the last step of a call (or of a captured cycle), after which every
+// kept detector sample is added.
+static void step_once(ms_sim* s, float2* const* scratch, bool last, const FieldRecorder* rec = nullptr) {
   const bool fdtd = s->drive == MS_DRIVE_FDTD;
   // sub-stepping: the molecules advance (by nsub dt) on every nsub-th step only,
   // and only those steps' E updates take the molecular dipole change
@@ -1196,8 +1199,13 @@ static void step_once(ms_sim* s, float2* const* scratch, const FieldRecorder* re
     ms::launch_yee_e(ge, s->stream);  // with the incident lines' E half step
     ++launched;
     if (s->g.ndet > 0) {
-      ms::launch_dft(s->g, s->stream);
+      ms::launch_dft_keep(s->g, s->dft_kept++, s->stream);
       ++launched;
+      if (s->dft_kept == ms::kDftBatch || last) {
+        ms::launch_dft_add(s->g, s->dft_kept, s->stream);
+        s->dft_kept = 0;
+        ++launched;
+      }
     }
   }
   if (s->timing) mark(s);  // the phases end here; the counter runs between steps
@@ -1210,15 +1218,22 @@ static void step_once(ms_sim* s, float2* const* scratch, const FieldRecorder* re
   }
 }
 
+// Steps of a captured cycle: whole molecular cycles, at least 8 steps, or a batch
+// of detector samples.
+static int cycle_steps(const ms_sim* s) {
+  const int least = s->g.ndet > 0 ? ms::kDftBatch : 8;
+  return s->nsub * std::max(1, (least + s->nsub - 1) / s->nsub);
+}
+
 // Capture the launches of s->gsteps steps from phase 0 into a graph.  The
 // host step count is restored: capturing runs nothing.
 static ms_status capture_cycle(ms_sim* s) {
   if (s->gexec) cudaGraphExecDestroy(s->gexec);
   s->gexec = nullptr;
-  s->gsteps = s->nsub * std::max(1, (8 + s->nsub - 1) / s->nsub);
+  s->gsteps = cycle_steps(s);
   const int64_t saved = s->steps;
   if (cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return MS_ECUDA;
-  for (int q = 0; q < s->gsteps; ++q) step_once(s, nullptr);
+  for (int q = 0; q < s->gsteps; ++q) step_once(s, nullptr, q == s->gsteps - 1);
   s->steps = saved;
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(s->stream, &g);
@@ -1243,11 +1258,11 @@ ms_status ms_step(ms_sim* s, int64_t n) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess) return MS_ECUDA;
   if (s->graphs && !s->timing && cs == cudaStreamCaptureStatusNone) {
+    const int L = cycle_steps(s);
     while (n > 0 && s->steps % s->nsub != 0) {  // to the start of a molecular cycle
-      step_once(s, nullptr);
+      step_once(s, nullptr, n == 1 || (s->steps + 1) % s->nsub == 0);
       --n;
     }
-    const int L = s->nsub * std::max(1, (8 + s->nsub - 1) / s->nsub);
     if (n >= L) {
       if (!s->gexec || s->gdirty || s->gsteps != L) MS_TRY(capture_cycle(s));
       for (; n >= L; n -= L) {
@@ -1256,7 +1271,7 @@ ms_status ms_step(ms_sim* s, int64_t n) {
       }
     }
   }
-  for (int64_t q = 0; q < n; ++q) step_once(s, nullptr);
+  for (int64_t q = 0; q < n; ++q) step_once(s, nullptr, q == n - 1);
   return cudaGetLastError() == cudaSuccess ? MS_OK : MS_ECUDA;
 }
 
@@ -1276,7 +1291,7 @@ ms_status ms_step_noalloc(ms_sim* s, int64_t n) {
     off += (bytes + 255) / 256 * 256;
   }
   if (!s->noalloc_base) return MS_ECUDA;
-  for (int64_t q = 0; q < n; ++q) step_once(s, scratch);
+  for (int64_t q = 0; q < n; ++q) step_once(s, scratch, q == n - 1);
   return cudaGetLastError() == cudaSuccess ? MS_OK : MS_ECUDA;
 }
 
@@ -1442,7 +1457,7 @@ ms_status ms_record_local_fields(ms_sim* s, const int64_t* mol_ids, int64_t m, f
   if (st == MS_OK) {
     FieldRecorder rec{static_cast<const long long*>(d_ids), (int)m, static_cast<float*>(d_out)};
     for (int64_t q = 0; q < nsteps; ++q) {
-      step_once(s, nullptr, &rec);
+      step_once(s, nullptr, q == nsteps - 1, &rec);
       rec.out += (size_t)m * 3;
     }
     if (cudaGetLastError() != cudaSuccess ||
@@ -1471,14 +1486,20 @@ ms_status ms_set_detectors(ms_sim* s, const int32_t* planes_z, int32_t nplanes, 
   int* dk = nullptr;
   double* dw = nullptr;
   double2* acc = nullptr;
+  float* ring = nullptr;
+  long long* ring_n = nullptr;
   std::vector<int> k(planes_z, planes_z + nplanes);
   std::vector<double> w(omega, omega + nfreq);
   MS_TRY(upload(s, &dk, k.data(), k.size()));
   MS_TRY(upload(s, &dw, w.data(), w.size()));
   MS_TRY(zeros(s, &acc, (size_t)s->g.nsim * nplanes * nfreq * 4 * s->g.nx * s->g.ny));
+  MS_TRY(zeros(s, &ring, (size_t)ms::kDftBatch * s->g.nsim * nplanes * 6 * s->g.nx * s->g.ny));
+  MS_TRY(zeros(s, &ring_n, ms::kDftBatch));
   s->g.det_k = dk;
   s->g.omega = dw;
   s->g.dft = acc;
+  s->g.dft_ring = ring;
+  s->g.dft_n = ring_n;
   s->g.ndet = nplanes;
   s->g.nfreq = nfreq;
   return cudaStreamSynchronize(s->stream) == cudaSuccess ? MS_OK : MS_ECUDA;

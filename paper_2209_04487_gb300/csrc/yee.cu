@@ -578,50 +578,87 @@ void launch_record_fields(const Grid& g, const int* cell, const long long* ids, 
 // Spectral detection: after the E update of step n (E^{n+1}, H^{n+1/2}),
 // every cell of every detector plane adds dt F e^{i omega t} for each
 // frequency: Ex, Ey of the plane at t_{n+1}; Hx, Hy averaged over the planes
-// z = k - 1/2 and k + 1/2 (indices k - 1 and k) at t_{n+1/2}.  FP64.  A block
-// covers 256 cells of one plane and kDftF frequencies.
-constexpr int kDftF = 8;
-__global__ void dft_kernel(Grid g, int nfc) {
-  __shared__ double2 ph[2][kDftF];  // E and H phases of this block's frequencies, times dt
-  const long long n = *g.step;
+// z = k - 1/2 and k + 1/2 (indices k - 1 and k) at t_{n+1/2}, into FP64
+// accumulators.  Reading and writing those every step took 48 us a step (two
+// planes of 128 x 128 cells, 48 frequencies: 201 MB); the FP64 products alone
+// need 22 us (two a clock and SM).  So a step only keeps its samples, and one
+// launch adds up to kDftBatch kept steps, in their order: every accumulator is
+// read and written once a batch and takes the same sums as step by step.
+__global__ void dft_keep_kernel(Grid g, int slot) {
+  const long long plane = (long long)g.ny * g.nx, q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (q == 0 && blockIdx.y == 0 && blockIdx.z == 0) g.dft_n[slot] = *g.step;
+  if (q >= plane) return;
+  const long long ck = blockIdx.z * g.ncell_sim + (long long)g.det_k[blockIdx.y] * plane + q, cm = ck - plane;
+  float* o = g.dft_ring + (((long long)slot * g.nsim + blockIdx.z) * g.ndet + blockIdx.y) * 6 * plane + q;
+  o[0] = g.E[0][ck];
+  o[plane] = g.E[1][ck];
+  o[2 * plane] = g.H[0][cm];
+  o[3 * plane] = g.H[0][ck];
+  o[4 * plane] = g.H[1][cm];
+  o[5 * plane] = g.H[1][ck];
+}
+
+constexpr int kDftF = 8;  // frequencies a block
+
+// A block: 256 cells of one plane, kDftF frequencies, every component, `count` kept steps.
+__global__ void __launch_bounds__(256) dft_add_kernel(Grid g, int nfc, int count) {
+  __shared__ double2 ph[2][kDftF][kDftBatch];  // dt e^{i omega t} at the E and at the H times
   const int d = blockIdx.y / nfc, f0 = (blockIdx.y % nfc) * kDftF, sim = blockIdx.z;
   const int nf = min(kDftF, g.nfreq - f0);
-  if (threadIdx.x < nf) {
-    double s1, c1, s2, c2;
-    const double w = g.omega[f0 + threadIdx.x];
-    sincos(w * (double)(n + 1) * g.dt, &s1, &c1);
-    sincos(w * ((double)n + 0.5) * g.dt, &s2, &c2);
-    ph[0][threadIdx.x] = make_double2(c1 * g.dt, s1 * g.dt);
-    ph[1][threadIdx.x] = make_double2(c2 * g.dt, s2 * g.dt);
+  for (int q = threadIdx.x; q < 2 * nf * count; q += blockDim.x) {
+    const int b = q % count, f = (q / count) % nf, h = q / (count * nf);
+    const long long n = g.dft_n[b];
+    double sn, cs;
+    sincos(g.omega[f0 + f] * (h ? (double)n + 0.5 : (double)(n + 1)) * g.dt, &sn, &cs);
+    ph[h][f][b] = make_double2(cs * g.dt, sn * g.dt);
   }
   __syncthreads();
   const long long plane = (long long)g.ny * g.nx;
   const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (q >= plane) return;
-  const int k = g.det_k[d];
-  const long long base = sim * g.ncell_sim;
-  const long long ck = base + (long long)k * plane + q, cm = ck - plane;
-  const double v[4] = {g.E[0][ck], g.E[1][ck], 0.5 * ((double)g.H[0][cm] + (double)g.H[0][ck]),
-                       0.5 * ((double)g.H[1][cm] + (double)g.H[1][ck])};
+  const float* ring = g.dft_ring + ((long long)sim * g.ndet + d) * 6 * plane + q;
+  const long long slot = (long long)g.nsim * g.ndet * 6 * plane;
   double2* acc = g.dft + (((long long)sim * g.ndet + d) * g.nfreq + f0) * 4 * plane + q;
-  for (int f = 0; f < nf; ++f) {
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    double v[kDftBatch];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const double2 w = ph[c < 2 ? 0 : 1][f];
-      double2* a = acc + ((long long)f * 4 + c) * plane;
-      double2 x = *a;
-      x.x = fma(v[c], w.x, x.x);
-      x.y = fma(v[c], w.y, x.y);
-      *a = x;
+    for (int b = 0; b < kDftBatch; ++b) {
+      v[b] = 0.0;
+      if (b < count)
+        v[b] = c < 2 ? (double)ring[b * slot + c * plane]
+                     : 0.5 * ((double)ring[b * slot + (2 * c - 2) * plane] + (double)ring[b * slot + (2 * c - 1) * plane]);
+    }
+#pragma unroll 1
+    for (int f = 0; f < nf; f += 2) {  // two frequencies at a time: four independent chains
+      const bool two = f + 1 < nf;
+      const double2 *w0 = ph[c < 2 ? 0 : 1][f], *w1 = ph[c < 2 ? 0 : 1][two ? f + 1 : f];
+      double2 *a0 = acc + ((long long)f * 4 + c) * plane, *a1 = a0 + (two ? 4 * plane : 0);
+      double2 x = *a0, y = *a1;
+#pragma unroll
+      for (int b = 0; b < kDftBatch; ++b) {
+        if (b >= count) break;
+        x.x = fma(v[b], w0[b].x, x.x);
+        x.y = fma(v[b], w0[b].y, x.y);
+        if (two) {
+          y.x = fma(v[b], w1[b].x, y.x);
+          y.y = fma(v[b], w1[b].y, y.y);
+        }
+      }
+      *a0 = x;
+      if (two) *a1 = y;
     }
   }
 }
-void launch_dft(const Grid& g, cudaStream_t s) {
-  if (g.ndet <= 0) return;
+void launch_dft_keep(const Grid& g, int slot, cudaStream_t s) {
+  const long long plane = (long long)g.ny * g.nx;
+  dft_keep_kernel<<<dim3((unsigned)((plane + 255) / 256), (unsigned)g.ndet, (unsigned)g.nsim), 256, 0, s>>>(g, slot);
+}
+void launch_dft_add(const Grid& g, int count, cudaStream_t s) {
   const long long plane = (long long)g.ny * g.nx;
   const int nfc = (g.nfreq + kDftF - 1) / kDftF;
   const dim3 grid((unsigned)((plane + 255) / 256), (unsigned)(g.ndet * nfc), (unsigned)g.nsim);
-  dft_kernel<<<grid, 256, 0, s>>>(g, nfc);
+  dft_add_kernel<<<grid, 256, 0, s>>>(g, nfc, count);
 }
 void launch_step_counter(long long* step, cudaStream_t s) {
   step_counter_kernel<<<1, 1, 0, s>>>(step);

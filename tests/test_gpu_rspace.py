@@ -50,3 +50,29 @@ def _check(B, nr, jmax, path, E0, state_form=0, nsteps=24, nmol=3):
                                           (64, 4, 2), (128, 4, 1), (128, 4, 2), (256, 4, 2)])
 def test_whole_rotor_kernel(B, nr, jmax, path, E0):
     _check(B, nr, jmax, path, E0)
+
+
+@pytest.mark.parametrize("nfreq,calls", [(1, (1, 15, 16, 17, 3)), (9, (33, 1, 40)), (8, (7,) * 6)])
+def test_detector_batches_do_not_depend_on_the_calls(B, nfreq, calls):
+    """Detector samples are added up to 16 steps at a time within a call, in
+    their order: any division of a run into calls gives the accumulators of
+    single steps, bit for bit."""
+    def geo(nx, ny, nz):
+        m = np.zeros((nz, ny, nx), np.uint8)
+        m[24:28, 2:, 3:-4] = W.configs.MAT_SILVER
+        return m
+    n = sum(calls)
+    wl = W.custom("dft", 20, 18, 48, nsim=2, src_k=14, pulses=[[1e9, 1.5, 1e-15, 1e-16]] * 2, geometry=geo,
+                  n_per_sim=0, nsteps=n)
+    planes, om = [12, 40, 25], np.linspace(1.0, 3.0, nfreq) / 6.582119569e-16
+    got = []
+    for steps in ((1,) * n, calls):
+        sim = B.Simulation(wl, step_graphs=B.MS_GRAPHS_AUTO)
+        sim.set_detectors(planes, om)
+        for k in steps:
+            sim.step(k)
+        got.append(np.array([[[sim.dft(p, s, c, f) for f in range(nfreq)] for c in range(4) for s in range(2)]
+                             for p in range(3)]))
+        sim.close()
+    assert (np.abs(got[0]).max(axis=(0, 2, 3, 4)) > 0).all()   # every component of both simulations
+    assert np.array_equal(got[0], got[1])
