@@ -101,27 +101,6 @@ cudaError_t upload_coupling_tables(const CouplEntry* rot, const CouplEntry* dip)
   return cudaMemcpyToSymbol(c_dip, dip, sizeof(CouplEntry) * kMaxRot * kMaxCoupl);
 }
 
-// Terms N of the coupling series exp(iA) ~ sum_{n <= N} (iA)^n / n!, for a
-// Hermitian A with |A| <= x (x = theta |E'|).  Truncated after N terms the
-// step changes the norm by up to 2 x^(N+1)/(N+1)! when N is odd; when N is
-// even the first omitted term (iA)^(N+1) is odd in A and has no real part,
-// so the norm changes only by up to 2 x^(N+2)/(N+1)!, while the amplitude
-// the omitted terms carry, relative to the first-order term, is x^N/(N+1)!.
-// N is the smallest count with a norm change below 1e-11 per step (1e-7 over
-// 10^4 steps) and, for even N, an amplitude error below 1e-6.  24 flags a
-// field out of range.
-__device__ __forceinline__ int coupling_terms(float x) {
-  if (!(x > 0.f)) return 0;
-  float t = x;  // x^N / N!
-  for (int N = 1; N < 24; ++N) {
-    const float t1 = t * x / (float)(N + 1);  // x^(N+1) / (N+1)!
-    const bool done = (N & 1) ? 2.f * t1 < 1e-11f : (2.f * t1 * x < 1e-11f && t1 < 1e-6f * x);
-    if (done) return N;
-    t = t1;
-  }
-  return 24;
-}
-
 // Local field at molecule m in its own frame (a.u.): fld = (E_perp, E'_z), the
 // phases e^{i m' phi_E} (ph[m' + J], m' = -J..J) of the frame turned about z
 // so that E'_y = 0, and the number of coupling-series terms (coupling_terms).
@@ -518,26 +497,13 @@ constexpr int ch_m(int c) { return c - ch_j(c) * ch_j(c) - ch_j(c); }
 // channel of (j, m), or -1 outside the basis of size J
 constexpr int ch_of(int j, int m, int J) { return (j < 0 || j > J || m < -j || m > j) ? -1 : j * j + j + m; }
 
-// Per molecule of a streaming species: the local field in the molecule frame
-// scaled by theta, (theta E'_z, theta E'_x / 2, theta E'_y / 2), and the
-// number of coupling-series terms (coupling_terms).
+// The records on their own, where no FFT kernel makes them: for the mixed kinetic
+// pass and the fused form (a thread of the fused kernel that makes its molecule's
+// record waits for three dependent loads, and its CTA with it: 9.99 against 9.30
+// ms for eight steps of 50,000 molecules).
 __global__ void mol_field_kernel(SpeciesDev sp, MolDev md, Grid g, int prescribed, int* err) {
   const int lm = blockIdx.x * blockDim.x + threadIdx.x;
-  if (lm >= sp.nmol) return;
-  const int m = sp.mol[lm];
-  float E[3];
-  lab_field(md, g, prescribed, m, E, err);
-  const float* O = md.rot + 9 * (long long)m;  // molecule -> lab, row-major
-  const float inv_fau = 1.0f / 5.14220674763e11f;
-  float Ep[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) Ep[i] = (O[i] * E[0] + O[3 + i] * E[1] + O[6 + i] * E[2]) * inv_fau;
-  const float th = (float)sp.theta;
-  const float x = th * sqrtf(Ep[0] * Ep[0] + Ep[1] * Ep[1] + Ep[2] * Ep[2]);
-  if (!isfinite(x)) atomicOr(err, kErrNonFinite);  // a non-finite local field
-  const int nt = coupling_terms(x);
-  if (nt >= 24 || x > 4.f) atomicOr(err, kErrCouplingSeries);
-  sp.fld[lm] = make_float4(th * Ep[2], 0.5f * th * Ep[0], 0.5f * th * Ep[1], __int_as_float(nt));
+  if (lm < sp.nmol) sp.fld[lm] = field_record(sp, md, g, prescribed, sp.mol[lm], err);
 }
 
 // Row layout of a molecule's state.  Full: both surfaces carry every channel
@@ -1127,20 +1093,27 @@ cudaError_t launch_broadcast_row(float2* psi, const float2* row, int nr, size_t 
 }
 
 // ----------------------------------------------------------------------------
-// streaming form, first pass: d2 = (T - 1) s for blocks of rows (rows of all
+// streaming form, first pass: the molecules' field records, by the first nfld
+// blocks (a launch of their own took 4 us a step), and d2 = (T - 1) s for blocks of rows (rows of all
 // molecules of a species are independent here); one bulk copy per block, or one
 // per molecule that the block touches where the molecules store more rows than
 // are processed
 // ----------------------------------------------------------------------------
 template <int NR>
 __global__ void __launch_bounds__(FFTShape<NR>::THREADS)
-    mol_kinetic_kernel(SpeciesDev sp, long long rows_total, int RB, int* err) {
+    mol_kinetic_kernel(SpeciesDev sp, MolDev md, Grid g, int prescribed, int nfld, long long rows_total, int RB,
+                       int* err) {
+  if ((int)blockIdx.x < nfld) {
+    const int lm = blockIdx.x * FFTShape<NR>::THREADS + threadIdx.x;
+    if (lm < sp.nmol) sp.fld[lm] = field_record(sp, md, g, prescribed, sp.mol[lm], err);
+    return;
+  }
   extern __shared__ float4 smem4[];
   float2* s_tw = reinterpret_cast<float2*>(smem4);
   float2* s_kd = s_tw + NR;
   float2* st = s_kd + NR;
   __shared__ __align__(8) unsigned long long s_bar;
-  const long long r0 = blockIdx.x * (long long)RB;
+  const long long r0 = ((int)blockIdx.x - nfld) * (long long)RB;
   const int nrows = (int)min((long long)RB, rows_total - r0);
   const int t = threadIdx.x;
   if (t == 0) {
@@ -1747,8 +1720,10 @@ static int launch_stage1_t(const SpeciesDev& sp, const MolDev& md, const Grid& g
     mol_field_kernel<<<(sp.nmol + 127) / 128, 128, 0, s>>>(sp, md, g, prescribed, err);
     return 1;
   }
+  // the per-molecule frame-field records those kernels read
+  const bool records = use_point(sp) || use_tile(sp) || use_pair(sp);
   int n = 0;
-  if (use_point(sp) || use_tile(sp) || use_pair(sp)) {  // the per-molecule frame-field records those kernels read
+  if (records && sp.mixed) {
     mol_field_kernel<<<(sp.nmol + 127) / 128, 128, 0, s>>>(sp, md, g, prescribed, err);
     ++n;
   }
@@ -1769,8 +1744,10 @@ static int launch_stage1_t(const SpeciesDev& sp, const MolDev& md, const Grid& g
   const int RB = kinetic_rows(NR);
   const size_t ksmem = 2 * (size_t)NR * sizeof(float2) + (size_t)RB * NR * sizeof(float2);
   cudaFuncSetAttribute(mol_kinetic_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ksmem);
-  mol_kinetic_kernel<NR><<<(unsigned)((rows_total + RB - 1) / RB), FFTShape<NR>::THREADS, ksmem, s>>>(
-      sp, rows_total, RB, err);
+  constexpr int NT = FFTShape<NR>::THREADS;
+  const int nfld = records ? (sp.nmol + NT - 1) / NT : 0;
+  mol_kinetic_kernel<NR><<<(unsigned)(nfld + (rows_total + RB - 1) / RB), NT, ksmem, s>>>(
+      sp, md, g, prescribed, nfld, rows_total, RB, err);
   return n + 1;
 }
 

@@ -196,6 +196,47 @@ __device__ __forceinline__ void acc2p(float2& hi, float2& lo, float2 x) {
 
 
 
+// Terms N of the coupling series exp(iA) ~ sum_{n <= N} (iA)^n / n!, for a
+// Hermitian A with |A| <= x (x = theta |E'|).  Truncated after N terms the
+// step changes the norm by up to 2 x^(N+1)/(N+1)! when N is odd; when N is
+// even the first omitted term (iA)^(N+1) is odd in A and has no real part,
+// so the norm changes only by up to 2 x^(N+2)/(N+1)!, while the amplitude
+// the omitted terms carry, relative to the first-order term, is x^N/(N+1)!.
+// N is the smallest count with a norm change below 1e-11 per step (1e-7 over
+// 10^4 steps) and, for even N, an amplitude error below 1e-6.  24 flags a
+// field out of range.
+__device__ __forceinline__ int coupling_terms(float x) {
+  if (!(x > 0.f)) return 0;
+  float t = x;  // x^N / N!
+  for (int N = 1; N < 24; ++N) {
+    const float t1 = t * x / (float)(N + 1);  // x^(N+1) / (N+1)!
+    const bool done = (N & 1) ? 2.f * t1 < 1e-11f : (2.f * t1 * x < 1e-11f && t1 < 1e-6f * x);
+    if (done) return N;
+    t = t1;
+  }
+  return 24;
+}
+
+// A molecule's field record: the local field in the molecule frame scaled by
+// theta, (theta E'_z, theta E'_x / 2, theta E'_y / 2), and the number of
+// coupling-series terms (coupling_terms).
+__device__ __forceinline__ float4 field_record(const SpeciesDev& sp, const MolDev& md, const Grid& g, int prescribed,
+                                               int m, int* err) {
+  float E[3];
+  lab_field(md, g, prescribed, m, E, err);
+  const float* O = md.rot + 9 * (long long)m;  // molecule -> lab, row-major
+  const float inv_fau = 1.0f / 5.14220674763e11f;
+  float Ep[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) Ep[i] = (O[i] * E[0] + O[3 + i] * E[1] + O[6 + i] * E[2]) * inv_fau;
+  const float th = (float)sp.theta;
+  const float x = th * sqrtf(Ep[0] * Ep[0] + Ep[1] * Ep[1] + Ep[2] * Ep[2]);
+  if (!isfinite(x)) atomicOr(err, kErrNonFinite);  // a non-finite local field
+  const int nt = coupling_terms(x);
+  if (nt >= 24 || x > 4.f) atomicOr(err, kErrCouplingSeries);
+  return make_float4(th * Ep[2], 0.5f * th * Ep[0], 0.5f * th * Ep[1], __int_as_float(nt));
+}
+
 // Wait for phase `parity`, each try suspending up to hint_ns until the phase
 // completes; gives up after `tries` tries (by default about 2 s in all).
 __device__ __forceinline__ bool mbar_wait_sleep(unsigned long long* bar, unsigned parity, int tries = 2000,

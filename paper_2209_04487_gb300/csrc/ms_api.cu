@@ -80,7 +80,9 @@ struct ms_sim {
   ms::MolDev md{};
   ms::SpeciesDev sp[ms::kMaxSpecies]{};
   int* d_err = nullptr;
-  long long* d_step = nullptr;
+  long long* d_step = nullptr;  // the step counter's two slots
+  int slot = 0;                 // the one that holds the current step
+  int gslot = 0;                // the one the captured cycle starts from
   // device address of the library's fixed scratch array (ms_step_noalloc),
   // looked up at create with the handle's device current; null if that failed
   float2* noalloc_base = nullptr;
@@ -736,8 +738,8 @@ ms_status create_impl(const ms_grid_desc* G, const ms_materials_desc* M, const m
   g.ce_vac = (float)(dt / (kEps0 * dx));
   g.periodic_z = G->bc_z == MS_BC_PERIODIC;
   g.dt = dt;
-  MS_TRY(zeros(s, &g.step, 1));
-  s->d_step = g.step;
+  MS_TRY(zeros(s, &s->d_step, 2));
+  g.step = g.step_next = s->d_step;  // a step's launches take them from s->slot
   MS_TRY(zeros(s, &s->d_err, 1));
   MS_TRY(upload_angular_tables());
   // materials
@@ -1165,6 +1167,8 @@ static void step_once(ms_sim* s, float2* const* scratch, bool last, const FieldR
   // and only those steps' E updates take the molecular dipole change
   const bool molecular = s->steps % s->nsub == 0;
   int launched = 0;
+  s->g.step = s->d_step + s->slot;
+  s->g.step_next = s->d_step + (s->slot ^ 1);
   if (s->timing) mark(s);
   if (fdtd) {
     ms::launch_yee_h(s->g, s->stream);  // with the incident lines' H half step
@@ -1208,9 +1212,12 @@ static void step_once(ms_sim* s, float2* const* scratch, bool last, const FieldR
       }
     }
   }
-  if (s->timing) mark(s);  // the phases end here; the counter runs between steps
-  ms::launch_step_counter(s->d_step, s->stream);
-  ++launched;
+  if (s->timing) mark(s);  // the phases end here; a counter of its own (no E half step) runs between steps
+  if (!fdtd) {
+    ms::launch_step_counter(s->g.step, s->g.step_next, 1, s->stream);
+    ++launched;
+  }
+  s->slot ^= 1;
   ++s->steps;
   if (s->timing) {
     s->timed_steps++;
@@ -1218,11 +1225,20 @@ static void step_once(ms_sim* s, float2* const* scratch, bool last, const FieldR
   }
 }
 
+// A call that the caller captures ends on the counter slot it began with, so that
+// its graph can be replayed.
+static void keep_slot(ms_sim* s, int slot) {
+  if (s->slot == slot) return;
+  ms::launch_step_counter(s->d_step + s->slot, s->d_step + slot, 0, s->stream);
+  s->slot = slot;
+}
+
 // Steps of a captured cycle: whole molecular cycles, at least 8 steps, or a batch
 // of detector samples.
 static int cycle_steps(const ms_sim* s) {
   const int least = s->g.ndet > 0 ? ms::kDftBatch : 8;
-  return s->nsub * std::max(1, (least + s->nsub - 1) / s->nsub);
+  const int L = s->nsub * std::max(1, (least + s->nsub - 1) / s->nsub);
+  return L % 2 ? 2 * L : L;  // even: a cycle ends on the counter slot it began with
 }
 
 // Capture the launches of s->gsteps steps from phase 0 into a graph.  The
@@ -1232,6 +1248,7 @@ static ms_status capture_cycle(ms_sim* s) {
   s->gexec = nullptr;
   s->gsteps = cycle_steps(s);
   const int64_t saved = s->steps;
+  s->gslot = s->slot;
   if (cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return MS_ECUDA;
   for (int q = 0; q < s->gsteps; ++q) step_once(s, nullptr, q == s->gsteps - 1);
   s->steps = saved;
@@ -1257,6 +1274,7 @@ ms_status ms_step(ms_sim* s, int64_t n) {
   if (s->drive == MS_DRIVE_PRESCRIBED && s->nmol > 0 && s->steps + n > s->nwave) return MS_EINVAL;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess) return MS_ECUDA;
+  const int slot0 = s->slot;
   if (s->graphs && !s->timing && cs == cudaStreamCaptureStatusNone) {
     const int L = cycle_steps(s);
     while (n > 0 && s->steps % s->nsub != 0) {  // to the start of a molecular cycle
@@ -1265,6 +1283,7 @@ ms_status ms_step(ms_sim* s, int64_t n) {
     }
     if (n >= L) {
       if (!s->gexec || s->gdirty || s->gsteps != L) MS_TRY(capture_cycle(s));
+      keep_slot(s, s->gslot);  // the captured cycle starts from this one
       for (; n >= L; n -= L) {
         if (cudaGraphLaunch(s->gexec, s->stream) != cudaSuccess) return MS_ECUDA;
         s->steps += L;
@@ -1272,6 +1291,7 @@ ms_status ms_step(ms_sim* s, int64_t n) {
     }
   }
   for (int64_t q = 0; q < n; ++q) step_once(s, nullptr, q == n - 1);
+  if (cs != cudaStreamCaptureStatusNone) keep_slot(s, slot0);
   return cudaGetLastError() == cudaSuccess ? MS_OK : MS_ECUDA;
 }
 
@@ -1291,7 +1311,11 @@ ms_status ms_step_noalloc(ms_sim* s, int64_t n) {
     off += (bytes + 255) / 256 * 256;
   }
   if (!s->noalloc_base) return MS_ECUDA;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess) return MS_ECUDA;
+  const int slot0 = s->slot;
   for (int64_t q = 0; q < n; ++q) step_once(s, scratch, q == n - 1);
+  if (cs != cudaStreamCaptureStatusNone) keep_slot(s, slot0);
   return cudaGetLastError() == cudaSuccess ? MS_OK : MS_ECUDA;
 }
 
@@ -1826,7 +1850,7 @@ ms_status ms_load(ms_sim* s, const char* path) {
   if (st != MS_OK) return st;
   // the step counter, host and device
   const long long step = h.steps;
-  if (cudaMemcpy(s->g.step, &step, sizeof(step), cudaMemcpyHostToDevice) != cudaSuccess) return MS_ECUDA;
+  if (cudaMemcpy(s->d_step + s->slot, &step, sizeof(step), cudaMemcpyHostToDevice) != cudaSuccess) return MS_ECUDA;
   s->steps = h.steps;
   return latched(s);
 }

@@ -89,7 +89,11 @@ struct Grid {
   const int* cell_off;   // [nsim*(mk1-mk0)*ny*nx + 1]
   const int* cell_mol;   // molecule ids sorted by cell
   const double* dmu;     // [nmol][3] lab dipole change of the last step (a.u.)
-  long long* step;       // device step counter
+  // Device step counter, two slots used in turn: a step's kernels read `step`
+  // and its E half step writes the next index to `step_next` (a launch of its
+  // own for that took 2 us a step), so no kernel reads a slot being written.
+  long long* step;
+  long long* step_next;
   // spectral detection: running DFTs on z-planes, dt sum_n F(t_n) e^{i omega t_n}
   int ndet, nfreq;
   const int* det_k;      // [ndet] plane indices
@@ -252,7 +256,7 @@ cudaError_t launch_wait_timeout_probe(int tries, int* flag, cudaStream_t s);
 bool mol_mixed_supported(int nr);
 int mixed_strip_rows(int nr);
 int mixed_plane_offset(int row, int k, int nr);
-void launch_step_counter(long long* step, cudaStream_t s);
+void launch_step_counter(const long long* from, long long* to, int add, cudaStream_t s);
 // spectral detection: keep this step's samples in slot `slot`; add the first `count` kept steps
 void launch_dft_keep(const Grid& g, int slot, cudaStream_t s);
 void launch_dft_add(const Grid& g, int count, cudaStream_t s);

@@ -54,26 +54,33 @@ __device__ __forceinline__ long long pml_index(const Grid& g, int s, int k, int 
   return (((long long)(s * 2 + slab) * g.pml + kk) * g.ny + j) * g.nx + i;
 }
 
-// Incident line, H half step (one block per sim).  Node m of the line sits
-// at z = (ks - 2 + m) dx; only nodes inside the numerical light cone of the
-// source (m <= step + 2) can be non-zero, so only those are touched.
-__device__ void aux_h_block(const Grid& g, int s, int t, int nt) {
+// Incident line.  Node m of the line sits at z = (ks - 2 + m) dx; only nodes
+// inside the numerical light cone of the source (m <= step + 2) can be
+// non-zero, so only those are touched.  kAuxBlocks blocks per sim share them:
+// with one, a long run waits for its line (at 30,000 steps of the 32 x 32 x 64
+// workload a step took 48 us, 21 us of them for the line).
+constexpr int kAuxBlocks = 32;
+
+// H half step by block b of a sim's, nt threads each
+__device__ void aux_h_block(const Grid& g, int b, int t, int nt) {
+  const int s = b / kAuxBlocks;
   const long long n = *g.step;
   const int lim = (int)min((long long)g.aux_len, n + 4);
   float* E1 = g.auxE + (long long)s * (g.aux_len + 1);
   float* H1 = g.auxH + (long long)s * g.aux_len;
-  for (int m = t; m < lim; m += nt) H1[m] -= g.ch * (E1[m + 1] - E1[m]);
+  for (int m = (b % kAuxBlocks) * nt + t; m < lim; m += kAuxBlocks * nt) H1[m] -= g.ch * (E1[m + 1] - E1[m]);
 }
 
-// Incident line, E half step, and the new source sample at its node 0.
-__device__ void aux_e_block(const Grid& g, int s, int t, int nt) {
+// E half step, and the new source sample at node 0.
+__device__ void aux_e_block(const Grid& g, int b, int t, int nt) {
+  const int s = b / kAuxBlocks;
   const long long n = *g.step;
   const int lim = (int)min((long long)g.aux_len, n + 4);
   float* E1 = g.auxE + (long long)s * (g.aux_len + 1);
   const float* H1 = g.auxH + (long long)s * g.aux_len;
   const float ce = g.ce_vac;
-  for (int m = 1 + t; m < lim; m += nt) E1[m] += ce * (0.f - (H1[m] - H1[m - 1]));
-  if (t == 0) E1[0] = (float)incident_field(g.src[s], (double)(n + 1) * g.dt);
+  for (int m = 1 + (b % kAuxBlocks) * nt + t; m < lim; m += kAuxBlocks * nt) E1[m] += ce * (0.f - (H1[m] - H1[m - 1]));
+  if (b % kAuxBlocks == 0 && t == 0) E1[0] = (float)incident_field(g.src[s], (double)(n + 1) * g.dt);
 }
 
 // H^{n-1/2} -> H^{n+1/2}.  Blocks past the tiles step the incident lines
@@ -176,6 +183,7 @@ __global__ void __launch_bounds__(kTx * kTy, 5) yee_e_kernel(Grid g, int ntiles)
     aux_e_block(g, (int)blockIdx.x - ntiles, threadIdx.y * kTx + threadIdx.x, kTx * kTy);
     return;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *g.step_next = *g.step + 1;
   const Tile t = tile_of(g, blockIdx.x);
   const int i = t.in ? t.i : 0, j = t.in ? t.j : 0;
   const int sxy = g.nx * g.ny;                               // offsets within one sim (< 2^31 cells)
@@ -413,6 +421,7 @@ __global__ void __launch_bounds__(kQt) yee_e4_kernel(Grid g, int ntiles, int kz)
     aux_e_block(g, (int)blockIdx.x - ntiles, threadIdx.x, kQt);
     return;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *g.step_next = *g.step + 1;
   const Quad t = quad_of(g, blockIdx.x, kz);
   const int sxy = g.nx * g.ny;
   const int dy = t.j > 0 ? g.nx : -(g.ny - 1) * g.nx;
@@ -518,7 +527,9 @@ __global__ void __launch_bounds__(kQt) yee_e4_kernel(Grid g, int ntiles, int kz)
   }
 }
 
-__global__ void step_counter_kernel(long long* step) { *step += 1; }
+// to = from + add: the step counter of a step without an E half step (add = 1),
+// or its value in the other slot (add = 0)
+__global__ void step_counter_kernel(const long long* from, long long* to, int add) { *to = *from + add; }
 
 // The quad kernels take rows of whole quads and arrays on 16-byte boundaries
 // (mat: 4, cell_off: 16); an allocator of the caller may place them anywhere.
@@ -543,7 +554,7 @@ static int quad_tiles(const Grid& g, int kz) {
 }
 
 void launch_yee_h(const Grid& g, cudaStream_t s) {
-  const int aux = g.ks >= 0 ? g.nsim : 0;
+  const int aux = g.ks >= 0 ? g.nsim * kAuxBlocks : 0;
   if (quads_ok(g)) {
     const int kz = quad_planes(g), nt = quad_tiles(g, kz);
     yee_h4_kernel<<<nt + aux, kQt, 0, s>>>(g, nt, kz);
@@ -553,7 +564,7 @@ void launch_yee_h(const Grid& g, cudaStream_t s) {
   yee_h_kernel<<<nt + aux, dim3(kTx, kTy), 0, s>>>(g, nt);
 }
 void launch_yee_e(const Grid& g, cudaStream_t s) {
-  const int aux = g.ks >= 0 ? g.nsim : 0;
+  const int aux = g.ks >= 0 ? g.nsim * kAuxBlocks : 0;
   if (quads_ok(g)) {
     const int kz = quad_planes(g), nt = quad_tiles(g, kz);
     yee_e4_kernel<<<nt + aux, kQt, 0, s>>>(g, nt, kz);
@@ -660,8 +671,8 @@ void launch_dft_add(const Grid& g, int count, cudaStream_t s) {
   const dim3 grid((unsigned)((plane + 255) / 256), (unsigned)(g.ndet * nfc), (unsigned)g.nsim);
   dft_add_kernel<<<grid, 256, 0, s>>>(g, nfc, count);
 }
-void launch_step_counter(long long* step, cudaStream_t s) {
-  step_counter_kernel<<<1, 1, 0, s>>>(step);
+void launch_step_counter(const long long* from, long long* to, int add, cudaStream_t s) {
+  step_counter_kernel<<<1, 1, 0, s>>>(from, to, add);
 }
 
 }  // namespace ms

@@ -76,3 +76,33 @@ def test_detector_batches_do_not_depend_on_the_calls(B, nfreq, calls):
         sim.close()
     assert (np.abs(got[0]).max(axis=(0, 2, 3, 4)) > 0).all()   # every component of both simulations
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("captured", [1, 2, 3])
+def test_steps_captured_by_the_caller_replay(B, captured):
+    """A caller's own graph of a few steps, replayed: the step counter's two
+    slots end each replay where it began, so the replays, and steps after
+    them, are those of plain stepping bit for bit."""
+    import torch
+    wl = W.custom("captured", 20, 12, 48, src_k=14, pulses=[[1e10, 1.5, 1e-15, 2e-16]], layer=(20, 24), n_per_sim=40,
+                  species=[W.species_config0(jmax=1), W.Species(nr=128, jmax=3)], fractions=[0.5, 0.5], seed=3,
+                  nsteps=60)
+    def out(sim):
+        r = sim.populations(), sim.dipoles(), sim.fields(B.MS_FIELD_E), sim.fields(B.MS_FIELD_H)
+        sim.close()
+        return r
+    a = B.Simulation(wl, step_graphs=B.MS_GRAPHS_OFF)
+    a.step(5 + 4 * captured + 16)
+    b = B.Simulation(wl)
+    b.step(5)
+    b.populations()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=b.stream):
+        b.step(captured)
+    with torch.cuda.stream(b.stream):
+        for _ in range(4):
+            g.replay()
+    b.stream.synchronize()
+    b.step(16)
+    for x, y in zip(out(a), out(b)):
+        assert np.array_equal(x, y)
