@@ -59,12 +59,6 @@ __device__ __forceinline__ float2 cmul_c_add(float2 x, float4 w, float2 a) {
   return make_float2(fmaf(x.x, w.x, fmaf(-x.y, w.y, re_lo)), fmaf(x.x, w.y, fmaf(x.y, w.x, im_lo)));
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // 16-byte asynchronous global -> shared copies (per thread), completed by
 // cp.async.wait_group.
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -72,17 +66,6 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-__device__ __forceinline__ void load_state(float2* st, const float2* g, int rows, int NR, int NRP) {
-  const float4* g4 = reinterpret_cast<const float4*>(g);
-  const int per_row = NR / 2;
-  const int total = rows * per_row;
-  for (int q = threadIdx.x; q < total; q += blockDim.x) {
-    const int row = q / per_row, col = q - row * per_row;
-    reinterpret_cast<float4*>(st + row * NRP)[col] = g4[q];
-  }
-}
-
 
 }  // namespace
 
@@ -1021,56 +1004,94 @@ static int pair_tile(const SpeciesDev& sp) {
 // ----------------------------------------------------------------------------
 namespace ms {
 
+// A CTA takes `mpb` molecules whose excited rows fill an FFT block (one where a
+// molecule has more, in blocks of RB rows).  Each row's sums of |psi|^2 and
+// r |psi|^2 are taken from the transform's registers, compensated, over the N1
+// lanes that share the row, and summed in FP64 per molecule.  With a molecule a
+// CTA and psi brought back to shared memory 50,000 molecules at J = 4 (ten
+// excited rows) took 1.27 ms.
+template <int NR>
+constexpr int kObserveRows = 8192 / NR;  // rows of a block at most: 64 KB
+
 template <int NR>
 __global__ void __launch_bounds__(FFTShape<NR>::THREADS)
-    mol_observe_kernel(SpeciesDev sp, MolDev md, int RB) {
-  constexpr int NRP = NR + kPad;
+    mol_observe_kernel(SpeciesDev sp, MolDev md, int RB, int mpb, int* err) {
+  constexpr int N1 = FFTShape<NR>::N1, N2 = FFTShape<NR>::N2;
   extern __shared__ float4 smem4[];
   float2* s_tw = reinterpret_cast<float2*>(smem4);
   float2* s_kh = s_tw + NR;
   float2* st = s_kh + NR;
-  __shared__ double s_red[8][2];
-  const int lm = blockIdx.x;
-  const int m = sp.mol[lm];
-  for (int q = threadIdx.x; q < NR; q += blockDim.x) {
+  __shared__ __align__(8) unsigned long long s_bar;
+  __shared__ double s_row[kObserveRows<NR>][2];
+  const int t = threadIdx.x;
+  const int ne = sp.rows - sp.rows_g;  // excited rows
+  const int l0 = blockIdx.x * mpb, nm = min(mpb, sp.nmol - l0);
+  if (t == 0) {
+    mbar_init(&s_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int q = t; q < NR; q += blockDim.x) {
     s_tw[q] = __ldg(&sp.twiddle[q]);
     s_kh[q] = __ldg(&sp.khalf[q]);
   }
-  const int ne = sp.rows - sp.rows_g;  // excited rows
-  const float2* ge = sp.psi + ((long long)lm * sp.mrows + sp.rows_g) * NR;
   double num = 0.0, den = 0.0;
-  for (int b0 = 0; b0 < ne; b0 += RB) {  // blocks of RB rows
-    const int nb = min(RB, ne - b0);
-    __syncthreads();
-    load_state(st, ge + (long long)b0 * NR, nb, NR, NRP);
-    __syncthreads();
-    kinetic_pass<NR>(st, st, nb, s_kh, s_tw);  // psi = T^{1/2} s
-    for (int r = threadIdx.x; r < NR; r += blockDim.x) {
-      float a = 0.f;
-      for (int row = 0; row < nb; ++row) {
-        const float2 v = st[row * NRP + r];
-        a = fmaf(v.x, v.x, fmaf(v.y, v.y, a));
+  unsigned phase = 0;
+  for (int b0 = 0; b0 < ne; b0 += RB) {  // one pass unless a molecule has more than RB rows (mpb = 1)
+    const int nb = mpb > 1 ? nm * ne : min(RB, ne - b0);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the last pass's rows before the copy over them
+    __syncthreads();  // the barrier is initialised; the rows and sums of the last pass are read
+    if (t == 0) {
+      mbar_expect_tx(&s_bar, (unsigned)(nb * NR * sizeof(float2)));
+      const int per = mpb > 1 ? ne : nb;
+      for (int k = 0; k * per < nb; ++k)
+        bulk_g2s(st + k * per * NR, sp.psi + ((long long)(l0 + k) * sp.mrows + sp.rows_g + b0) * NR,
+                 (unsigned)(per * NR * sizeof(float2)), &s_bar);
+    }
+    const bool ok = mbar_wait_sleep(&s_bar, phase);
+    if (!__syncthreads_and(ok)) {
+      if (t == 0) atomicOr(err, kErrTimeout);
+      if (!ok) mbar_wait_sleep(&s_bar, phase);
+      return;
+    }
+    phase ^= 1;
+    kinetic_pass<NR, FFTShape<NR>::THREADS, false>(st, st, nb, s_kh, s_tw, [&](int row, int n1, float2(&x)[N2]) {
+      float dh = 0.f, dl = 0.f, nh = 0.f, nl = 0.f;  // psi = T^{1/2} s
+      if (row < nb) {
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) {
+          const float a = fmaf(x[n2].x, x[n2].x, x[n2].y * x[n2].y), r = __ldg(&sp.r[n1 + N1 * n2]);
+          const float p = a * r;
+          acc2(dh, dl, a);
+          acc2(nh, nl, p);
+          nl += fmaf(a, r, -p);
+        }
       }
-      den += (double)a;
-      num += (double)a * (double)__ldg(&sp.r[r]);
-    }
+#pragma unroll
+      for (int o = N1 / 2; o > 0; o >>= 1) {
+        const float dh2 = __shfl_xor_sync(0xffffffffu, dh, o), dl2 = __shfl_xor_sync(0xffffffffu, dl, o);
+        const float nh2 = __shfl_xor_sync(0xffffffffu, nh, o), nl2 = __shfl_xor_sync(0xffffffffu, nl, o);
+        acc2(dh, dl, dh2);
+        acc2(nh, nl, nh2);
+        dl += dl2;
+        nl += nl2;
+      }
+      if (row < nb && n1 == 0) {
+        s_row[row][0] = (double)nh + (double)nl;
+        s_row[row][1] = (double)dh + (double)dl;
+      }
+    });
+    const int per = mpb > 1 ? ne : nb;  // kinetic_pass ends on a barrier
+    if (t < (mpb > 1 ? nm : 1))
+      for (int k = 0; k < per; ++k) {
+        num += s_row[t * per + k][0];
+        den += s_row[t * per + k][1];
+      }
+    if (mpb > 1) break;
   }
-  num = warp_sum(num);
-  den = warp_sum(den);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    s_red[wid][0] = num;
-    s_red[wid][1] = den;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) {
-      a += s_red[ww][0];
-      b += s_red[ww][1];
-    }
-    md.Rnum[m] = a * sp.dR;
-    md.Rden[m] = b * sp.dR;
+  if (t < nm) {
+    const int m = sp.mol[l0 + t];
+    md.Rnum[m] = num * sp.dR;
+    md.Rden[m] = den * sp.dR;
   }
 }
 
@@ -1823,23 +1844,26 @@ int launch_mol_stage2(const SpeciesDev& sp, const MolDev& md, const Grid& g, int
 }
 
 template <int NR>
-static void launch_observe_t(const SpeciesDev& sp, const MolDev& md, cudaStream_t s) {
-  const int RB = min(sp.nrot, 4096 / NR);
+static void launch_observe_t(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
+  // as many molecules as fill half a block, or one whose rows go in even blocks
+  const int ne = std::max(1, sp.rows - sp.rows_g), most = kObserveRows<NR>;
+  const int mpb = std::max(1, most / 2 / ne);
+  const int passes = (ne + most - 1) / most, RB = mpb > 1 ? mpb * ne : (ne + passes - 1) / passes;
   const size_t smem = 2 * (size_t)NR * sizeof(float2) + mol_state_smem(NR, RB);
   cudaFuncSetAttribute(mol_observe_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  mol_observe_kernel<NR><<<sp.nmol, FFTShape<NR>::THREADS, smem, s>>>(sp, md, RB);
+  mol_observe_kernel<NR><<<(sp.nmol + mpb - 1) / mpb, FFTShape<NR>::THREADS, smem, s>>>(sp, md, RB, mpb, err);
 }
 
-void launch_mol_observe(const SpeciesDev& sp, const MolDev& md, cudaStream_t s) {
+void launch_mol_observe(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
   if (sp.nmol == 0) return;
   if (sp.bloch) {
     launch_bloch_observe(sp, md, s);
     return;
   }
   switch (sp.nr) {
-    case 64: launch_observe_t<64>(sp, md, s); break;
-    case 128: launch_observe_t<128>(sp, md, s); break;
-    case 256: launch_observe_t<256>(sp, md, s); break;
+    case 64: launch_observe_t<64>(sp, md, err, s); break;
+    case 128: launch_observe_t<128>(sp, md, err, s); break;
+    case 256: launch_observe_t<256>(sp, md, err, s); break;
   }
 }
 

@@ -115,8 +115,13 @@ __device__ __forceinline__ int swz(int n1, int k2, int row) {
 }
 
 // The rows are read from `in` (st itself for the transform in place) by NT threads.
-template <int NR, int NT = FFTShape<NR>::THREADS, bool PACK = false>
-__device__ __forceinline__ void kinetic_pass(float2* st, const float2* in, int rows, const float2* kph, const float2* tw) {
+// The result goes back to st, or, with `take`, to take(row, n1, x): x[n2] at
+// point n1 + N1 n2, called for every row by the N1 neighbouring lanes n1, and
+// by whole warps together (rows past the end too, with row >= rows).
+struct KeepRows {};
+template <int NR, int NT = FFTShape<NR>::THREADS, bool PACK = false, class Take = KeepRows>
+__device__ __forceinline__ void kinetic_pass(float2* st, const float2* in, int rows, const float2* kph, const float2* tw,
+                                             Take take = Take()) {
   using S = FFTShape<NR>;
   constexpr int N1 = S::N1, N2 = S::N2, NRP = NR + kPad;
   const int t = threadIdx.x;
@@ -175,7 +180,9 @@ __device__ __forceinline__ void kinetic_pass(float2* st, const float2* in, int r
         dft_reg<N2, true, PACK>(x);
       }
       __syncwarp();
-      if (row < rows) {
+      if constexpr (!std::is_same_v<Take, KeepRows>) {
+        take(row, n1, x);
+      } else if (row < rows) {
 #pragma unroll
         for (int n2 = 0; n2 < N2; ++n2) st[row * NRP + n1 + N1 * n2] = x[n2];
       }

@@ -1410,7 +1410,7 @@ ms_status ms_read_dissociation(ms_sim* s, int64_t first, int64_t count, double* 
   if (!s || first < 0 || count < 0 || first + count > s->nmol) return MS_EINVAL;
   MS_TRY(read_pairs(s, s->md.absorbed, first, count, ag, ae));
   if (Rnum || Rden) {
-    for (int si = 0; si < s->nspecies; ++si) ms::launch_mol_observe(s->sp[si], s->md, s->stream);
+    for (int si = 0; si < s->nspecies; ++si) ms::launch_mol_observe(s->sp[si], s->md, s->d_err, s->stream);
     if (cudaGetLastError() != cudaSuccess) return MS_ECUDA;
     MS_TRY(read_range(s, s->md.Rnum, 1, first, count, Rnum));
     MS_TRY(read_range(s, s->md.Rden, 1, first, count, Rden));

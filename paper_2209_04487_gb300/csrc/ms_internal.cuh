@@ -229,7 +229,7 @@ int launch_mol_stage1(const SpeciesDev& sp, const MolDev& md, const Grid& g, int
                       cudaStream_t s);
 int launch_mol_stage2(const SpeciesDev& sp, const MolDev& md, const Grid& g, int prescribed, int* err,
                       cudaStream_t s);
-void launch_mol_observe(const SpeciesDev& sp, const MolDev& md, cudaStream_t s);
+void launch_mol_observe(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s);
 // launchers (bloch.cu): the frozen two-level step and its Eq. 8 readout
 int launch_bloch_step(const SpeciesDev& sp, const MolDev& md, const Grid& g, int prescribed, int* err,
                       cudaStream_t s);

@@ -52,6 +52,13 @@ def test_whole_rotor_kernel(B, nr, jmax, path, E0):
     _check(B, nr, jmax, path, E0)
 
 
+@pytest.mark.parametrize("nr,jmax,nmol", [(64, 1, 45), (128, 3, 14), (128, 4, 7), (256, 4, 3), (256, 9, 2)])
+def test_dissociation_readout_blocks(B, nr, jmax, nmol):
+    """The readout's blocks: several molecules each with a remainder, one
+    each, and a molecule over two passes."""
+    _check(B, nr, jmax, 2, 6e10, nmol=nmol)
+
+
 @pytest.mark.parametrize("nfreq,calls", [(1, (1, 15, 16, 17, 3)), (9, (33, 1, 40)), (8, (7,) * 6)])
 def test_detector_batches_do_not_depend_on_the_calls(B, nfreq, calls):
     """Detector samples are added up to 16 steps at a time within a call, in
