@@ -975,24 +975,29 @@ static bool rspace_ok(int nr, int jmax);
 // The tiled kernel runs a streaming species' R-space pass where the point-
 // resident one does not and it applies, unless the plan names another kernel.
 static bool pair_ok(int nr, int jmax) { return (nr == 64 || nr == 128 || nr == 256) && jmax <= 16; }
+// The column kernel runs the reachable rows of a streaming species from J = 5
+// to 8 (below, a thread holds the whole rotor; above, half a side's columns no
+// longer fit a thread's registers).
+static bool use_col(const SpeciesDev& sp) {
+  return sp.path == MS_MOL_STREAMING && sp.par && sp.jmax >= 5 && sp.jmax <= 8;
+}
 // The two-points-a-thread tiled kernel runs a streaming species' R-space pass
-// where the plan names it, and by the static rule from J = 5 on (for the
-// parity-reduced state it is the only kernel from J = 5 on).
+// where the plan names it, and by the static rule from J = 5 on (from J = 9 on
+// for the reachable rows).
 static bool use_pair(const SpeciesDev& sp) {
   if (sp.path != MS_MOL_STREAMING || sp.dipw || !pair_ok(sp.nr, sp.jmax)) return false;
-  if (sp.par) return sp.jmax >= 5;
+  if (sp.par) return sp.jmax >= 9;
   return sp.kern == MS_KERN_PAIR || (sp.kern == MS_KERN_DEFAULT && sp.jmax >= 5);
 }
 static bool use_tile(const SpeciesDev& sp) {
-  if (sp.path != MS_MOL_STREAMING || use_point(sp) || use_pair(sp) || !rspace_ok(sp.nr, sp.jmax)) return false;
+  if (sp.path != MS_MOL_STREAMING || use_point(sp) || use_col(sp) || use_pair(sp) || !rspace_ok(sp.nr, sp.jmax))
+    return false;
   return sp.kern == MS_KERN_DEFAULT || sp.kern == MS_KERN_TILE;
 }
 // its tile width: 8 points from J = 9 on; else the plan's, or 8 points from
-// J = 5 on (the nanohole pass 113.7 against 118.3 ms at 16) and 32 below;
-// parity-reduced rows: 16 points to J = 8 (at 8 a CTA would hold two warps)
+// J = 5 on (the nanohole pass 113.7 against 118.3 ms at 16) and 32 below
 static int pair_tile(const SpeciesDev& sp) {
   if (sp.jmax >= 9) return 8;
-  if (sp.par) return 16;
   if (sp.ch == 8 || sp.ch == 16 || sp.ch == 32) return sp.ch;
   return sp.jmax >= 5 ? 8 : 32;
 }
@@ -1375,7 +1380,8 @@ bool mol_reachable_rows(const SpeciesDev& sp) {
   if (sp.par_form) return true;
   if (sp.all_rows) return false;
   return use_point(sp) ||
-         (sp.path == MS_MOL_STREAMING && sp.kern == MS_KERN_DEFAULT && sp.jmax >= 5 && mol_tensor_maps_available());
+         (sp.path == MS_MOL_STREAMING && sp.kern == MS_KERN_DEFAULT && sp.jmax >= 5 &&
+          (sp.jmax <= 8 || mol_tensor_maps_available()));
 }
 
 void mol_set_rows(SpeciesDev& sp, bool reachable) {
@@ -1742,7 +1748,7 @@ static int launch_stage1_t(const SpeciesDev& sp, const MolDev& md, const Grid& g
     return 1;
   }
   // the per-molecule frame-field records those kernels read
-  const bool records = use_point(sp) || use_tile(sp) || use_pair(sp);
+  const bool records = use_point(sp) || use_col(sp) || use_tile(sp) || use_pair(sp);
   int n = 0;
   if (records && sp.mixed) {
     mol_field_kernel<<<(sp.nmol + 127) / 128, 128, 0, s>>>(sp, md, g, prescribed, err);
@@ -1799,13 +1805,17 @@ static int launch_stage2_t(const SpeciesDev& sp, const MolDev& md, const Grid& g
     }
     return 1;
   }
+  if (use_col(sp)) {
+    launch_rspace_col(sp, md, err, s);
+    return 1;
+  }
   RspaceMaps maps;
   if (use_pair(sp)) {
     if (rspace_maps(sp, pair_tile(sp), true, &maps)) {
       launch_rspace_pair(sp, md, err, maps, pair_tile(sp), s);
       return 1;
     }
-    if (sp.par) {  // no other kernel takes the parity-reduced state beyond J = 4: report it
+    if (sp.par) {  // no other kernel takes the reachable rows beyond J = 8: report it
       flag_error_kernel<<<1, 1, 0, s>>>(err, kErrLaunch);
       return 1;
     }

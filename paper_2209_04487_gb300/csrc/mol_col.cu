@@ -1,0 +1,377 @@
+// R-space pass on columns of the rotor (J = 5..8, streaming layout, reachable
+// rows): the kernel and its launch.
+//
+// The reachable rows of a molecule are one vector psi_{j m} over all channels
+// (the surface is the parity of j), and the coupling E'.R^ is E'_z Z within a
+// column of fixed m plus S+- between neighbouring columns.  For the coupling a
+// thread holds whole columns at one radial point in registers: the Z
+// neighbours are its own, the S+- neighbours too except at the edges of its
+// columns, and the coefficients are immediates of packed FP32x2 products.  A
+// thread a row instead reads six neighbours of every row from shared memory,
+// whose pipe then bounds the pass.
+//
+// Four warps take a molecule, 32 radial points at a time (lane = point).  Warps
+// 0 and 1 hold the columns m = 0 .. K - 1 and K .. J, warps 2 and 3 the
+// mirrored ones, -m: with mu = -m the coupling has the same form with the sign
+// of E'_x flipped, so they run the same code.  Column 0 belongs to warp 0 and
+// is read by warp 2.  The vector itself stands in shared memory (one array Y,
+// rewritten term by term between barriers).
+//
+// Everything that is not the coupling (eta before it, the update after it) runs
+// row by row in loops over Y, shared out evenly over the warps: only about 30
+// instructions a row are unrolled.  With every phase unrolled (100 KB of code
+// at J = 8) the pass waited for instructions: 8.8 ps a row and point; with the
+// rows' loads one at a time for those loads: 12.5 ps.  What is left of that
+// wait bounds it (a thread per row: 8.0 ps; now 7.3, 6.4, 6.1 and 6.8 at
+// J = 5, 6, 7, 8; 3.5 ps is HBM's).
+//
+// The coupling's exponential series S = sum_{n=1..N} (i theta M)^n / n! eta is
+// summed by Horner's rule, S = i theta M y_1, y_n = eta + (i theta / (n + 1)) M
+// y_{n+1}, y_N = eta.
+#include "mol_common.cuh"
+
+namespace ms {
+namespace {
+
+template <int J>
+struct ColDims {
+  static constexpr int len(int m) { return m > J ? 0 : J - m + 1; }  // rows of column m
+  static constexpr int rows(int a, int b) {                          // rows of columns [a, b)
+    int n = 0;
+    for (int m = a; m < b; ++m) n += len(m);
+    return n;
+  }
+  // columns 0 .. K - 1 on the low warps: the split with the smallest larger share
+  static constexpr int split() {
+    int best = 2;
+    for (int k = 3; k <= J; ++k) {
+      const int a = rows(0, k), b = rows(k, J + 1), c = rows(0, best), d = rows(best, J + 1);
+      if ((a > b ? a : b) < (c > d ? c : d)) best = k;
+    }
+    return best;
+  }
+  static constexpr int K = split();
+  static constexpr int NROT = (J + 1) * (J + 1);
+  // first row of shell j among the reachable rows: ground even shells, then excited odd shells
+  static constexpr int shell(int j) {
+    int n = 0;
+    for (int q = 0; q <= J; ++q)
+      if ((q & 1) < (j & 1) || ((q & 1) == (j & 1) && q < j)) n += 2 * q + 1;
+    return n;
+  }
+  static constexpr int NG = shell(1);  // ground rows
+  // rows whose loads a warp keeps in flight outside the coupling: few passes over a warp's rows of a surface (4 and
+  // 6, 7 and 6, 7 and 9, 12 and 9) with few idle places; six throughout took 6.97 ps at J = 6, 7.44 at J = 7
+  static constexpr int BATCH = J == 5 ? 6 : (J == 6 ? 7 : (J == 7 ? 9 : 6));
+};
+
+constexpr int kColThreads = 128;
+
+// warps arrive here from different code, so the barrier is named
+__device__ __forceinline__ void col_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kColThreads) : "memory"); }
+
+// One warp's columns: LOW 0 .. K - 1 (0 is only read when mirrored), else K .. J.
+template <int J, bool LOW>
+struct ColWarp {
+  using D = ColDims<J>;
+  static constexpr int C0 = LOW ? 0 : D::K, C1 = LOW ? D::K : J + 1, N = D::rows(C0, C1);
+  static constexpr int ix(int c, int j) { return D::rows(C0, c) + j - c; }
+  static constexpr int at(int j) { return D::shell(j) + j; }  // row (j, 0)
+
+  // calls fn(c, j) for the rows of this warp's columns; OWN: those it stores
+  template <bool OWN, class F>
+  static __device__ __forceinline__ void each(bool mir, F&& fn) {
+    static_for<C0, C1>([&](auto cc) {
+      constexpr int c = decltype(cc)::value;
+      if (OWN && LOW && c == 0 && mir) return;
+      static_for<c, J + 1>([&](auto jc) { fn(cc, jc); });
+    });
+  }
+
+  // Y <- S of the series on Y = eta (at this lane); row(j, c) of Y at Y + 32 (at(j) + sg c)
+  template <class Eta>
+  static __device__ __forceinline__ void series(float2* Y, bool mir, int nterms, float fz, float fx, float fy, Eta&& eta) {
+    const int sg = mir ? -32 : 32;  // from one column to the next
+    float2 v[N], w[N];
+    auto load = [&]() {
+      each<false>(mir, [&](auto cc, auto jc) {
+        constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+        v[ix(c, j)] = (Y + sg * c)[32 * at(j)];
+      });
+    };
+    auto store = [&]() {  // between barriers: every neighbour is read, then everything is written
+      col_sync();
+      each<true>(mir, [&](auto cc, auto jc) {
+        constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+        (Y + sg * c)[32 * at(j)] = w[ix(c, j)];
+      });
+      col_sync();
+    };
+    auto get = [&](auto cc, auto jc) -> float2 {
+      constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+      if constexpr (c >= C0 && c < C1) return v[ix(c, j)];
+      else return (Y + sg * c)[32 * at(j)];
+    };
+    // base + i (M v) at row (c, j); z2, x2, y2 the field's factors
+    auto coupled = [&](auto cc, auto jc, float2 z2, float2 x2, float2 y2, float2 base) -> float2 {
+      constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+      auto sum2 = [&](auto cf0, auto cf1, auto c2) {  // cf0 (c2, j - 1) + cf1 (c2, j + 1)
+        constexpr int cq = decltype(c2)::value, mq = cq < 0 ? -cq : cq;
+        constexpr bool lo = j - 1 >= mq, hi = j + 1 <= J && j + 1 >= mq;
+        using std::integral_constant;
+        if constexpr (lo && hi)
+          return fma2(dup2(cf0()), get(c2, integral_constant<int, j - 1>()),
+                      mul2(dup2(cf1()), get(c2, integral_constant<int, j + 1>())));
+        else if constexpr (lo) return mul2(dup2(cf0()), get(c2, integral_constant<int, j - 1>()));
+        else if constexpr (hi) return mul2(dup2(cf1()), get(c2, integral_constant<int, j + 1>()));
+        else return make_float2(0.f, 0.f);
+      };
+      const float2 az = sum2([] { return c_zd(j, c); }, [] { return c_zu(j, c); }, std::integral_constant<int, c>());
+      const float2 ap = sum2([] { return c_pd(j, c); }, [] { return c_pu(j, c); }, std::integral_constant<int, c - 1>());
+      const float2 am = sum2([] { return c_md(j, c); }, [] { return c_mu(j, c); }, std::integral_constant<int, c + 1>());
+      const float2 t = fma2(z2, az, mul2(x2, add2(ap, am)));
+      const float2 e = fma2(y2, sub2(ap, am), base);
+      return make_float2(e.x - t.y, e.y + t.x);
+    };
+    load();
+#pragma unroll 1
+    for (int n = nterms; n >= 2; --n) {
+      const float cn = 1.f / (float)n;
+      const float2 z2 = dup2(fz * cn), x2 = dup2(fx * cn), y2 = dup2(fy * cn);
+      if (n == nterms) {
+        each<true>(mir, [&](auto cc, auto jc) {
+          constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+          w[ix(c, j)] = coupled(cc, jc, z2, x2, y2, v[ix(c, j)]);
+        });
+      } else {  // three terms and more: eta again
+        each<true>(mir, [&](auto cc, auto jc) {
+          constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+          w[ix(c, j)] = coupled(cc, jc, z2, x2, y2, eta(j, at(j) + (mir ? -c : c)));
+        });
+      }
+      store();
+      load();
+    }
+    const float2 z2 = dup2(fz), x2 = dup2(fx), y2 = dup2(fy);
+    each<true>(mir, [&](auto cc, auto jc) {
+      constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+      w[ix(c, j)] = coupled(cc, jc, z2, x2, y2, make_float2(0.f, 0.f));
+    });
+    store();
+  }
+
+  // Dipole sums of Y = s': over pairs of rows of one column (Z) and of columns c, c + 1 (S+, S-); each pair
+  // joins a ground and an excited row, and conj(g) e and conj(e) g give the same Re (P + M), Im (P - M)
+  static __device__ __forceinline__ void dipole(const float2* Y, bool mir, float2& ax, float& ay, float2& az) {
+    const int sg = mir ? -32 : 32;
+    float2 v[N];
+    each<false>(mir, [&](auto cc, auto jc) {
+      constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+      v[ix(c, j)] = (Y + sg * c)[32 * at(j)];
+    });
+    each<true>(mir, [&](auto cc, auto jc) {
+      constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+      if constexpr (j < J) az = fma2(dup2(c_zu(j, c)), mul2(v[ix(c, j)], v[ix(c, j + 1)]), az);
+    });
+    each<false>(mir, [&](auto cc, auto jc) {
+      constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+      if constexpr (c < J) {
+        auto up = [&](auto j2) -> float2 {
+          constexpr int jq = decltype(j2)::value;
+          if constexpr (c + 1 < C1) return v[ix(c + 1, jq)];
+          else return (Y + sg * (c + 1))[32 * at(jq)];
+        };
+        constexpr bool hi = j + 1 <= J, lo = j - 1 >= c + 1;
+        float2 t = make_float2(0.f, 0.f);
+        if constexpr (hi) t = mul2(dup2(c_mu(j, c)), up(std::integral_constant<int, j + 1>()));
+        if constexpr (lo && hi) t = fma2(dup2(c_md(j, c)), up(std::integral_constant<int, j - 1>()), t);
+        else if constexpr (lo) t = mul2(dup2(c_md(j, c)), up(std::integral_constant<int, j - 1>()));
+        if constexpr (hi || lo) {
+          const float2 q = v[ix(c, j)];
+          ax = fma2(q, t, ax);
+          ay = fmaf(q.y, t.x, fmaf(-q.x, t.y, ay));
+        }
+      }
+    });
+  }
+};
+
+template <int J>
+__global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesDev sp, MolDev md, int* err) {
+  using D = ColDims<J>;
+  constexpr int NROT = D::NROT, NG = D::NG;
+  __shared__ float2 Ys[NROT][32];
+  __shared__ int s_vt[NROT + 3];  // row -> its shell's row of the phase table (and three past the end)
+  __shared__ float s_red[4][10];
+  __shared__ float s_fin[8], s_fin_lo[2];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int lm = blockIdx.x, m = sp.mol[lm], NR = sp.nr;
+  const float4 f = __ldg(&sp.fld[lm]);  // (theta E'_z, theta E'_x/2, theta E'_y/2, terms)
+  const float cfix = md.ncorr[m];       // rounding feedback of the previous step
+  const float2 cf = dup2(cfix);
+  // what the closing threads add to: the previous dipole, the absorbed norm so far
+  const double old = t < 3 ? md.mu[3 * (long long)m + t]
+                           : (t == 5 || t == 6 ? md.absorbed[2 * (long long)m + (t - 5)] : 0.0);
+  for (int q = t; q < NROT + 3; q += kColThreads) {
+    int j = q >= NG, r = q - (j ? NG : 0);
+    while (r >= 2 * j + 1 && j + 2 <= J) {
+      r -= 2 * j + 1;
+      j += 2;
+    }
+    s_vt[q] = j * NR;
+  }
+  const int nterms = max(__float_as_int(f.w), 1);  // no field: one term of zeros
+  const bool mir = (w & 2) != 0;
+  const float fx = mir ? -f.y : f.y;
+  float2* const Y = &Ys[0][lane];
+  float2 hi = make_float2(0.f, 0.f), lo = hi, ax = hi, az = hi, rnd = hi;  // hi, lo: populations (ground, excited)
+  float ab[2] = {0.f, 0.f}, ay = 0.f;
+
+#pragma unroll 1
+  for (int r0 = 0; r0 < NR; r0 += 32) {
+    float2* const s = sp.psi + (long long)lm * sp.mrows * NR + r0 + lane;
+    const float2* const d = sp.d2 + (long long)lm * NROT * NR + r0 + lane;
+    const float4* const vt = sp.vcol + r0 + lane;
+    const float2 mk = __ldg(&sp.maskw[r0 + lane]);
+    __syncthreads();  // the table is built; the last points' dipole has read Y
+    // ---- eta = V^{1/2} (s + d2): rows w, w + 4, .., D::BATCH at a time, their loads in flight together
+#pragma unroll 1
+    for (int q0 = w; q0 < NROT; q0 += 4 * D::BATCH) {
+      float2 s0[D::BATCH], d0[D::BATCH], p[D::BATCH];
+#pragma unroll
+      for (int i = 0; i < D::BATCH; ++i) {
+        const int q = min(q0 + 4 * i, NROT - 1);
+        s0[i] = s[q * NR];
+        d0[i] = __ldg(d + q * NR);
+        p[i] = __ldg(reinterpret_cast<const float2*>(vt + s_vt[q]));
+      }
+#pragma unroll
+      for (int i = 0; i < D::BATCH; ++i)
+        if (q0 + 4 * i < NROT) Y[32 * (q0 + 4 * i)] = cmul(p[i], add2(s0[i], d0[i]));
+    }
+    if (r0 + 32 < NR) {  // the next points' lines towards L2
+      for (int q = t; q < 4 * NROT; q += kColThreads) {
+        const float2* b = (q & 1 ? d : s) - lane + 32 + (q >> 2) * NR + (q & 2) * 8;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(b));
+      }
+    }
+    __syncthreads();
+    // ---- Y <- S
+    auto eta = [&](int j, int row) {
+      return cmul(__ldg(reinterpret_cast<const float2*>(vt + j * NR)), add2(s[row * NR], __ldg(d + row * NR)));
+    };
+    if (w & 1) ColWarp<J, false>::series(Y, mir, nterms, f.x, fx, f.z, eta);
+    else ColWarp<J, true>::series(Y, mir, nterms, f.x, fx, f.z, eta);
+    // ---- d1 = (V - 1) u + V^{1/2} S, mask, s' = s + (d2 + d1) + cfix s; a surface at a time
+    const bool masked = mk.x < 1.f;
+#pragma unroll
+    for (int sf = 0; sf < 2; ++sf) {
+      const int q1 = sf ? NROT : NG;
+      float2 h2 = make_float2(sf ? hi.y : hi.x, 0.f), l2 = make_float2(sf ? lo.y : lo.x, 0.f);
+#pragma unroll 1
+      for (int q0 = (sf ? NG : 0) + w; q0 < q1; q0 += 4 * D::BATCH) {
+        float2 s0[D::BATCH], d0[D::BATCH];
+        float4 p[D::BATCH];
+#pragma unroll
+        for (int i = 0; i < D::BATCH; ++i) {
+          const int q = min(q0 + 4 * i, q1 - 1);
+          s0[i] = s[q * NR];
+          d0[i] = __ldg(d + q * NR);
+          p[i] = __ldg(vt + s_vt[q]);
+        }
+        float b2 = 0.f;
+#pragma unroll
+        for (int i = 0; i < D::BATCH; ++i) {
+          const int q = q0 + 4 * i;
+          float b = 0.f;
+          if (q < q1) {
+            const float2 S = Y[32 * q], u = add2(s0[i], d0[i]);
+            float2 d1 = make_float2(fmaf(p[i].z, u.x, fmaf(-p[i].w, u.y, fmaf(p[i].x, S.x, -p[i].y * S.y))),
+                                    fmaf(p[i].z, u.y, fmaf(p[i].w, u.x, fmaf(p[i].x, S.y, p[i].y * S.x))));
+            if (masked) {
+              const float2 z = add2(u, d1);
+              d1 = fma2(dup2(mk.x - 1.f), u, mul2(dup2(mk.x), d1));
+              ab[sf] += mk.y * fmaf(z.x, z.x, z.y * z.y);
+            }
+            const float2 sn = round_update2(s0[i], add2(d0[i], d1), cf, rnd);
+            __stcs(s + q * NR, sn);
+            Y[32 * q] = sn;
+            b = fmaf(sn.x, sn.x, sn.y * sn.y);
+          }
+          if (i & 1) acc2p(h2, l2, make_float2(b2, b));  // compensated from the first term on
+          else if (i == D::BATCH - 1) acc2p(h2, l2, make_float2(b, 0.f));
+          else b2 = b;
+        }
+      }
+      float h = h2.x, l = l2.x + l2.y;
+      acc2(h, l, h2.y);
+      if (sf) hi.y = h, lo.y = l;
+      else hi.x = h, lo.x = l;
+    }
+    __syncthreads();
+    if (w & 1) ColWarp<J, false>::dipole(Y, mir, ax, ay, az);
+    else ColWarp<J, true>::dipole(Y, mir, ax, ay, az);
+  }
+  // ---- block reduction: populations compensated, the rest plain FP32; mirrored columns count E'_x reversed
+  const float dx = ax.x + ax.y;
+  float v[8] = {hi.x, hi.y, ab[0], ab[1], mir ? -dx : dx, ay, 2.f * (az.x + az.y), rnd.x + rnd.y};
+  float l2[2] = {lo.x, lo.y};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float h2 = __shfl_xor_sync(0xffffffffu, v[k], o);
+      const float g2 = __shfl_xor_sync(0xffffffffu, l2[k], o);
+      acc2(v[k], l2[k], h2);
+      l2[k] += g2;
+    }
+#pragma unroll
+    for (int k = 2; k < 8; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+  }
+  if (lane == 0) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s_red[w][k] = v[k];
+    s_red[w][8] = l2[0];
+    s_red[w][9] = l2[1];
+  }
+  __syncthreads();
+  if (t < 8) {
+    float h = 0.f, l = 0.f;
+#pragma unroll
+    for (int ww = 0; ww < 4; ++ww) {
+      acc2(h, l, s_red[ww][t]);
+      if (t < 2) l += s_red[ww][8 + t];
+    }
+    s_fin[t] = h + l;
+    if (t < 2) s_fin_lo[t] = l - (s_fin[t] - h);
+  }
+  __syncthreads();
+  if (t < 3) {  // lab dipole: mu = O mu', mu' = d dR (Re(S+ + S-), Im(S+ - S-), 2 Re Z)
+    const float* O = md.rot + 9 * (long long)m + 3 * t;
+    const float lab = (float)sp.dipole * sp.dR * (O[0] * s_fin[4] + O[1] * s_fin[5] + O[2] * s_fin[6]);
+    const double nl = (double)lab;
+    md.dmu[3 * (long long)m + t] = nl - old;
+    md.mu[3 * (long long)m + t] = nl;
+  } else if (t < 5) {
+    const double P = ((double)s_fin[t - 3] + (double)s_fin_lo[t - 3]) * (double)sp.dR;
+    md.pop[2 * (long long)m + (t - 3)] = P;
+    if (!isfinite(P)) atomicOr(err, kErrNonFinite);
+  } else if (t < 7) {
+    md.absorbed[2 * (long long)m + (t - 5)] = old + (double)s_fin[t - 3] * (double)sp.dR;
+  } else if (t == 7) {
+    md.ncorr[m] = rounding_feedback(s_fin[7], s_fin[0] + s_fin[1]);
+  }
+}
+
+}  // namespace
+
+void launch_rspace_col(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s) {
+  switch (sp.jmax) {
+    case 5: mol_rspace_col_kernel<5><<<sp.nmol, kColThreads, 0, s>>>(sp, md, err); break;
+    case 6: mol_rspace_col_kernel<6><<<sp.nmol, kColThreads, 0, s>>>(sp, md, err); break;
+    case 7: mol_rspace_col_kernel<7><<<sp.nmol, kColThreads, 0, s>>>(sp, md, err); break;
+    case 8: mol_rspace_col_kernel<8><<<sp.nmol, kColThreads, 0, s>>>(sp, md, err); break;
+  }
+}
+
+}  // namespace ms

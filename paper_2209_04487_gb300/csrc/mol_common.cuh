@@ -283,6 +283,8 @@ void launch_rspace_pair(const SpeciesDev& sp, const MolDev& md, int* err, const 
 // The molecular step on whole rotors, J <= 4, reachable rows (mol_rotor.cu):
 // the R-space pass of a streaming species or the whole fused step.
 void launch_rotor(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s);
+// The R-space pass on columns of the rotor, J = 5..8, reachable rows (mol_col.cu).
+void launch_rspace_col(const SpeciesDev& sp, const MolDev& md, int* err, cudaStream_t s);
 // uploads the angular tables into mol_pair.cu's copy
 cudaError_t upload_triplet_tables_pair(const CouplEntry* dip);
 // The one-point-a-thread tiled R-space pass (mol_tile.cu) at tile width

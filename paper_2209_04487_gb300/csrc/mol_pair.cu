@@ -496,9 +496,7 @@ __global__ void __launch_bounds__(Rs2Dims<J, TILE, PAR>::NT, Rs2Dims<J, TILE, PA
 template <int J, int TILE>
 static void launch_pair_jt(const SpeciesDev& sp, const MolDev& md, int* err, const RspaceMaps& maps,
                            cudaStream_t s) {
-  // the parity-reduced kernels exist from J = 5 on at the rule's tile width
-  constexpr bool kPar = J >= 5 && TILE == (J >= 9 ? 8 : 16);
-  if constexpr (kPar) {
+  if constexpr (J >= 9) {  // the reachable rows (below J = 9: mol_col.cu, mol_rotor.cu)
     if (sp.par) {
       using P = Rs2Dims<J, TILE, true>;
       launch_persistent(mol_rspace_pair_kernel<J, TILE, true>, P::NT, P::BYTES, sp, md, err, maps, s);

@@ -505,6 +505,16 @@ ms_status build_species(ms_sim* s, int si, const ms_species& d, double dt, const
     MS_TRY(upload(s, (float2**)&sp.vhalf_pp, vhp.data(), vhp.size()));
     MS_TRY(upload(s, (float2**)&sp.maskw_pp, mwp.data(), mwp.size()));
   }
+  sp.vcol = nullptr;
+  if (J >= 5 && J <= 8) {  // the column kernel's table: shell j on the surface of its parity
+    std::vector<float4> vc((size_t)(J + 1) * nr);
+    for (int j = 0; j <= J; ++j)
+      for (int i = 0; i < nr; ++i) {
+        const size_t q = ((size_t)(j & 1) * (J + 1) + j) * nr + i;
+        vc[(size_t)j * nr + i] = make_float4(vhalf[q].x, vhalf[q].y, vdelta[q].x, vdelta[q].y);
+      }
+    MS_TRY(upload(s, (float4**)&sp.vcol, vc.data(), vc.size()));
+  }
   MS_TRY(upload(s, (float**)&sp.r, rf.data(), rf.size()));
   MS_TRY(upload(s, (int**)&sp.mol, ids.data(), ids.size()));
   // populations at t = 0

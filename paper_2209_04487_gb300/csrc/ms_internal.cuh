@@ -145,6 +145,8 @@ struct SpeciesDev {
   const float2* vdelta_pp;
   const float2* vhalf_pp;
   const float2* maskw_pp;
+  // reachable rows: (e^{-i V dtau/2}, e^{-i V dtau} - 1) of shell j on the surface of its parity, [jmax+1][nr]
+  const float4* vcol;
   const float* r;           // [nr]
   double theta;             // d * dtau (d(R): its largest |d| times dtau)
   double dipole;            // d (e a0) (d(R): its largest |d|)

@@ -52,6 +52,12 @@ def test_whole_rotor_kernel(B, nr, jmax, path, E0):
     _check(B, nr, jmax, path, E0)
 
 
+@pytest.mark.parametrize("E0", [0.0, 1e6, 1e9, 6e10])
+@pytest.mark.parametrize("nr,jmax,form", [(64, 5, 0), (128, 6, 1), (64, 7, 1), (256, 8, 0), (128, 8, 1)])
+def test_column_kernel(B, nr, jmax, form, E0):
+    _check(B, nr, jmax, 2, E0, state_form=form)
+
+
 @pytest.mark.parametrize("nr,jmax,nmol", [(64, 1, 45), (128, 3, 14), (128, 4, 7), (256, 4, 3), (256, 9, 2)])
 def test_dissociation_readout_blocks(B, nr, jmax, nmol):
     """The readout's blocks: several molecules each with a remainder, one
