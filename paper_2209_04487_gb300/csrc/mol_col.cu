@@ -22,8 +22,7 @@
 // instructions a row are unrolled.  With every phase unrolled (100 KB of code
 // at J = 8) the pass waited for instructions: 8.8 ps a row and point; with the
 // rows' loads one at a time for those loads: 12.5 ps.  What is left of that
-// wait bounds it (a thread per row: 8.0 ps; now 7.3, 6.4, 6.1 and 6.8 at
-// J = 5, 6, 7, 8; 3.5 ps is HBM's).
+// wait bounds it (a thread per row: 8.0 ps; now 6.1 to 6.5; 3.5 ps is HBM's).
 //
 // The coupling's exponential series S = sum_{n=1..N} (i theta M)^n / n! eta is
 // summed by Horner's rule, S = i theta M y_1, y_n = eta + (i theta / (n + 1)) M
@@ -60,9 +59,11 @@ struct ColDims {
     return n;
   }
   static constexpr int NG = shell(1);  // ground rows
-  // rows whose loads a warp keeps in flight outside the coupling: few passes over a warp's rows of a surface (4 and
-  // 6, 7 and 6, 7 and 9, 12 and 9) with few idle places; six throughout took 6.97 ps at J = 6, 7.44 at J = 7
-  static constexpr int BATCH = J == 5 ? 6 : (J == 6 ? 7 : (J == 7 ? 9 : 6));
+  // rows whose loads a warp keeps in flight before the coupling, and after it for the ground and the excited rows:
+  // few passes over a warp's rows (at J = 8: 21, 12 and 9) with few idle places.  Six throughout took 7.29, 6.97,
+  // 7.43 and 6.84 ps a row and point at J = 5, 6, 7 and 8; these 6.34, 6.37, 6.13 and 6.51.
+  static constexpr int EB = J == 8 ? 11 : (J == 6 ? 7 : 9);
+  static constexpr int GB = J == 5 ? 4 : (J == 6 ? 7 : (J == 7 ? 9 : 6)), XB = J == 5 ? 6 : (J == 6 ? 7 : 9);
 };
 
 constexpr int kColThreads = 128;
@@ -234,19 +235,19 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
     const float4* const vt = sp.vcol + r0 + lane;
     const float2 mk = __ldg(&sp.maskw[r0 + lane]);
     __syncthreads();  // the table is built; the last points' dipole has read Y
-    // ---- eta = V^{1/2} (s + d2): rows w, w + 4, .., D::BATCH at a time, their loads in flight together
+    // ---- eta = V^{1/2} (s + d2): rows w, w + 4, .., D::EB at a time, their loads in flight together
 #pragma unroll 1
-    for (int q0 = w; q0 < NROT; q0 += 4 * D::BATCH) {
-      float2 s0[D::BATCH], d0[D::BATCH], p[D::BATCH];
+    for (int q0 = w; q0 < NROT; q0 += 4 * D::EB) {
+      float2 s0[D::EB], d0[D::EB], p[D::EB];
 #pragma unroll
-      for (int i = 0; i < D::BATCH; ++i) {
+      for (int i = 0; i < D::EB; ++i) {
         const int q = min(q0 + 4 * i, NROT - 1);
         s0[i] = s[q * NR];
         d0[i] = __ldg(d + q * NR);
         p[i] = __ldg(reinterpret_cast<const float2*>(vt + s_vt[q]));
       }
 #pragma unroll
-      for (int i = 0; i < D::BATCH; ++i)
+      for (int i = 0; i < D::EB; ++i)
         if (q0 + 4 * i < NROT) Y[32 * (q0 + 4 * i)] = cmul(p[i], add2(s0[i], d0[i]));
     }
     if (r0 + 32 < NR) {  // the next points' lines towards L2
@@ -264,16 +265,15 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
     else ColWarp<J, true>::series(Y, mir, nterms, f.x, fx, f.z, eta);
     // ---- d1 = (V - 1) u + V^{1/2} S, mask, s' = s + (d2 + d1) + cfix s; a surface at a time
     const bool masked = mk.x < 1.f;
-#pragma unroll
-    for (int sf = 0; sf < 2; ++sf) {
-      const int q1 = sf ? NROT : NG;
+    static_for<0, 2>([&](auto sfc) {
+      constexpr int sf = decltype(sfc)::value, q1 = sf ? NROT : NG, UB = sf ? D::XB : D::GB;
       float2 h2 = make_float2(sf ? hi.y : hi.x, 0.f), l2 = make_float2(sf ? lo.y : lo.x, 0.f);
 #pragma unroll 1
-      for (int q0 = (sf ? NG : 0) + w; q0 < q1; q0 += 4 * D::BATCH) {
-        float2 s0[D::BATCH], d0[D::BATCH];
-        float4 p[D::BATCH];
+      for (int q0 = (sf ? NG : 0) + w; q0 < q1; q0 += 4 * UB) {
+        float2 s0[UB], d0[UB];
+        float4 p[UB];
 #pragma unroll
-        for (int i = 0; i < D::BATCH; ++i) {
+        for (int i = 0; i < UB; ++i) {
           const int q = min(q0 + 4 * i, q1 - 1);
           s0[i] = s[q * NR];
           d0[i] = __ldg(d + q * NR);
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
         }
         float b2 = 0.f;
 #pragma unroll
-        for (int i = 0; i < D::BATCH; ++i) {
+        for (int i = 0; i < UB; ++i) {
           const int q = q0 + 4 * i;
           float b = 0.f;
           if (q < q1) {
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
             b = fmaf(sn.x, sn.x, sn.y * sn.y);
           }
           if (i & 1) acc2p(h2, l2, make_float2(b2, b));  // compensated from the first term on
-          else if (i == D::BATCH - 1) acc2p(h2, l2, make_float2(b, 0.f));
+          else if (i == UB - 1) acc2p(h2, l2, make_float2(b, 0.f));
           else b2 = b;
         }
       }
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
       acc2(h, l, h2.y);
       if (sf) hi.y = h, lo.y = l;
       else hi.x = h, lo.x = l;
-    }
+    });
     __syncthreads();
     if (w & 1) ColWarp<J, false>::dipole(Y, mir, ax, ay, az);
     else ColWarp<J, true>::dipole(Y, mir, ax, ay, az);
