@@ -86,6 +86,7 @@ struct ms_sim {
   // device address of the library's fixed scratch array (ms_step_noalloc),
   // looked up at create with the handle's device current; null if that failed
   float2* noalloc_base = nullptr;
+  double* flux = nullptr;  // ms_read_flux: [nsim][nfreq]
   int dft_kept = 0;  // detector samples kept and not yet added; 0 between calls
   std::vector<double> pop_init;  // create only: populations at t = 0, uploaded in one copy
   // phase timing
@@ -1522,6 +1523,7 @@ ms_status ms_set_detectors(ms_sim* s, const int32_t* planes_z, int32_t nplanes, 
   double2* acc = nullptr;
   float* ring = nullptr;
   long long* ring_n = nullptr;
+  double* flux = nullptr;
   std::vector<int> k(planes_z, planes_z + nplanes);
   std::vector<double> w(omega, omega + nfreq);
   MS_TRY(upload(s, &dk, k.data(), k.size()));
@@ -1529,11 +1531,13 @@ ms_status ms_set_detectors(ms_sim* s, const int32_t* planes_z, int32_t nplanes, 
   MS_TRY(zeros(s, &acc, (size_t)s->g.nsim * nplanes * nfreq * 4 * s->g.nx * s->g.ny));
   MS_TRY(zeros(s, &ring, (size_t)ms::kDftBatch * s->g.nsim * nplanes * 6 * s->g.nx * s->g.ny));
   MS_TRY(zeros(s, &ring_n, ms::kDftBatch));
+  MS_TRY(zeros(s, &flux, (size_t)s->g.nsim * nfreq));
   s->g.det_k = dk;
   s->g.omega = dw;
   s->g.dft = acc;
   s->g.dft_ring = ring;
   s->g.dft_n = ring_n;
+  s->flux = flux;
   s->g.ndet = nplanes;
   s->g.nfreq = nfreq;
   return cudaStreamSynchronize(s->stream) == cudaSuccess ? MS_OK : MS_ECUDA;
@@ -1554,23 +1558,11 @@ ms_status ms_read_dft(ms_sim* s, int32_t plane, int32_t sim_index, int32_t compo
 
 ms_status ms_read_flux(ms_sim* s, int32_t plane, double* flux) {
   if (!s || !flux || plane < 0 || plane >= s->g.ndet) return MS_EINVAL;
-  const size_t cells = (size_t)s->g.nx * s->g.ny, nf = (size_t)s->g.nfreq;
-  std::vector<double2> a(4 * cells);
-  const double dx2 = s->dx * s->dx;
-  for (int sim = 0; sim < s->g.nsim; ++sim)
-    for (size_t f = 0; f < nf; ++f) {
-      const double2* src = s->g.dft + ((((size_t)sim * s->g.ndet + plane) * nf + f) * 4) * cells;
-      if (cudaMemcpyAsync(a.data(), src, 4 * cells * sizeof(double2), cudaMemcpyDeviceToHost, s->stream) !=
-              cudaSuccess ||
-          cudaStreamSynchronize(s->stream) != cudaSuccess)
-        return MS_ECUDA;
-      double acc = 0.0;  // Re (Ex conj(Hy) - Ey conj(Hx))
-      for (size_t q = 0; q < cells; ++q) {
-        const double2 ex = a[q], ey = a[cells + q], hx = a[2 * cells + q], hy = a[3 * cells + q];
-        acc += (ex.x * hy.x + ex.y * hy.y) - (ey.x * hx.x + ey.y * hx.y);
-      }
-      flux[(size_t)sim * nf + f] = acc * dx2;
-    }
+  ms::launch_flux(s->g, plane, s->dx * s->dx, s->flux, s->stream);
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaMemcpyAsync(flux, s->flux, (size_t)s->g.nsim * s->g.nfreq * sizeof(double), cudaMemcpyDeviceToHost,
+                      s->stream) != cudaSuccess)
+    return MS_ECUDA;
   return latched(s);
 }
 

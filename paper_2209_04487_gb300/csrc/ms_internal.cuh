@@ -262,6 +262,8 @@ void launch_step_counter(const long long* from, long long* to, int add, cudaStre
 // spectral detection: keep this step's samples in slot `slot`; add the first `count` kept steps
 void launch_dft_keep(const Grid& g, int slot, cudaStream_t s);
 void launch_dft_add(const Grid& g, int count, cudaStream_t s);
+// Poynting flux spectra of one plane: out[nsim][nfreq]
+void launch_flux(const Grid& g, int plane, double dx2, double* out, cudaStream_t s);
 // E^n at the cells of the listed molecules: out[k][3] for k < m
 void launch_record_fields(const Grid& g, const int* cell, const long long* ids, int m, float* out,
                           cudaStream_t s);

@@ -661,6 +661,34 @@ __global__ void __launch_bounds__(256) dft_add_kernel(Grid g, int nfc, int count
     }
   }
 }
+
+// Poynting flux through detector plane `plane`, one block per (frequency, sim): the cells' Re (Ex conj(Hy) - Ey
+// conj(Hx)) in FP64, summed over a thread's cells, then over the block.  Bound by the accumulators' 64 B a cell.
+// Copying the accumulators to the host and summing them there took 2.6 ms a plane for 48 frequencies of 128 x 128.
+__global__ void __launch_bounds__(512) flux_kernel(Grid g, int plane, double dx2, double* out) {
+  __shared__ double part[16];
+  const long long cells = (long long)g.ny * g.nx;
+  const int f = blockIdx.x, sim = blockIdx.y, t = threadIdx.x;
+  const double2* a = g.dft + (((long long)sim * g.ndet + plane) * g.nfreq + f) * 4 * cells;
+  double acc = 0.0;
+  for (long long q = t; q < cells; q += blockDim.x) {
+    const double2 ex = a[q], ey = a[cells + q], hx = a[2 * cells + q], hy = a[3 * cells + q];
+    acc += (ex.x * hy.x + ex.y * hy.y) - (ey.x * hx.x + ey.y * hx.y);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((t & 31) == 0) part[t >> 5] = acc;
+  __syncthreads();
+  if (t == 0) {
+    double v = 0.0;
+    for (int w = 0; w < 16; ++w) v += part[w];
+    out[(long long)sim * g.nfreq + f] = v * dx2;
+  }
+}
+
+void launch_flux(const Grid& g, int plane, double dx2, double* out, cudaStream_t s) {
+  flux_kernel<<<dim3((unsigned)g.nfreq, (unsigned)g.nsim), 512, 0, s>>>(g, plane, dx2, out);
+}
 void launch_dft_keep(const Grid& g, int slot, cudaStream_t s) {
   const long long plane = (long long)g.ny * g.nx;
   dft_keep_kernel<<<dim3((unsigned)((plane + 255) / 256), (unsigned)g.ndet, (unsigned)g.nsim), 256, 0, s>>>(g, slot);

@@ -91,6 +91,29 @@ def test_detector_batches_do_not_depend_on_the_calls(B, nfreq, calls):
     assert np.array_equal(got[0], got[1])
 
 
+@pytest.mark.parametrize("nx,ny,nsim,nfreq", [(8, 8, 1, 1), (16, 32, 2, 3), (19, 27, 3, 2), (150, 130, 1, 2)])
+def test_flux_is_the_sum_over_the_accumulators(B, nx, ny, nsim, nfreq):
+    """Flux spectra against FP64 sums of the accumulators that are read back: planes below, of and above a block's
+    threads.  A term has three roundings; a sum adds at most one per cell of a thread, five over a warp and 16."""
+    wl = W.custom("flux", nx, ny, 48, nsim=nsim, src_k=14, pulses=[[1e9, 1.5, 1e-15, 1e-16]] * nsim, n_per_sim=0,
+                  nsteps=40)
+    sim = B.Simulation(wl)
+    sim.set_detectors([40, 25], np.linspace(1.0, 3.0, nfreq) / 6.582119569e-16)
+    sim.step(40)
+    tol = (3 + -(-nx * ny // 512) + 5 + 16 + 2) * 2.0 ** -53
+    for d in range(2):
+        got = sim.flux(d)
+        for s in range(nsim):
+            for f in range(nfreq):
+                ex, ey, hx, hy = (sim.dft(d, s, c, f) for c in range(4))
+                a, b = ex * np.conj(hy), ey * np.conj(hx)
+                size = (np.abs(ex.real * hy.real) + np.abs(ex.imag * hy.imag) + np.abs(ey.real * hx.real)
+                        + np.abs(ey.imag * hx.imag)).sum()
+                want = np.sum((a - b).real.astype(np.longdouble))
+                assert size > 0 and abs(got[s, f] / wl.dx ** 2 - want) <= 1.5 * tol * size
+    sim.close()
+
+
 @pytest.mark.parametrize("captured", [1, 2, 3])
 def test_steps_captured_by_the_caller_replay(B, captured):
     """A caller's own graph of a few steps, replayed: the step counter's two
