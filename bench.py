@@ -486,8 +486,13 @@ def main():
     per_step = lambda k: phases[k] / max(nsteps, 1)    # ms per step of one timed phase
     peak, peak_src = _peaks()
     nm = [int((wl.species_id == i).sum()) for i in range(len(wl.species))]
-    rows_of = (lambda sp: sp.nrot) if a.state == "parity" else (lambda sp: 2 * sp.nrot)
-    states = [8 * s.nr * rows_of(s) for s in wl.species]   # FP32 state of one molecule (bytes)
+    # rows a molecular step reads and writes: the static rule's kernels process the rows that the j = 0 start can
+    # populate (half of the full state; the others are zeros), a plan that names a kernel every row
+    def rows_of(sp, plan):
+        rule = plan[1] in (B.MS_KERN_DEFAULT, B.MS_KERN_POINT)
+        reach = rule and ((sp.jmax <= 4 and sp.nr == 128) if plan[0] == B.MS_MOL_FUSED else True)
+        return sp.nrot if a.state == "parity" or reach else 2 * sp.nrot
+    states = [8 * s.nr * rows_of(s, p) for s, p in zip(wl.species, main_form["plans"])]   # bytes of one molecule
     st_bytes = sum(b * n for b, n in zip(states, nm))
     one = len(wl.species) == 1
     sp = wl.species[0]
@@ -495,22 +500,25 @@ def main():
         # dominant kernel: the fused molecular step (stage 2), one launch per step;
         # the state read and written once
         rs_bytes = 2 * st_bytes + STATE_RECORDS * wl.n_molecules
-        kernel = f"mol_rpoint_kernel<{sp.jmax},{sp.nr},fused>" if one else "fused molecular steps"
-        note = "algorithmic bytes of the fused molecular step: the state read and written once, 168 B of records"
+        kernel = f"mol_rotor_fused_kernel<{sp.jmax}>" if one else "fused molecular steps"
+        note = ("algorithmic bytes of the fused molecular step: the rows that can be populated read and written once, "
+                "168 B of records")
         roof_kin = None
-        traffic_key = "mol_rpoint_kernel_fused"
+        traffic_key = "mol_rotor_fused_kernel"
     else:
         # dominant kernel: the R-space pass (stage 2); in the streaming form it reads
         # s and d2 and writes s'
         rs_bytes = 3 * st_bytes + STATE_RECORDS * wl.n_molecules
         if one and sp.jmax <= 4:
-            kernel, traffic_key = f"mol_rpoint_kernel<{sp.jmax},{sp.nr}>", "mol_rpoint_kernel"
+            kernel, traffic_key = f"mol_rotor_kernel<{sp.jmax},{sp.nr}>", "mol_rotor_kernel"
+        elif one and main_form["plans"][0][1] == B.MS_KERN_DEFAULT and 5 <= sp.jmax <= 8:
+            kernel, traffic_key = f"mol_rspace_col_kernel<{sp.jmax}>", "mol_rspace_col_kernel"
         elif one and main_form["plans"][0][1] in (B.MS_KERN_PAIR, B.MS_KERN_DEFAULT) and sp.jmax >= 5:
-            # the pair kernel's rule: 8-point tiles, 16 for the parity-reduced rows to J = 8
-            tile = 8 if sp.jmax >= 9 else (main_form["plans"][0][2] or (16 if a.state == "parity" else 8))
+            # the pair kernel's rule: 8-point tiles; over the rows that can be populated from J = 9 on by the rule
+            tile = 8 if sp.jmax >= 9 else (main_form["plans"][0][2] or 8)
             kernel, traffic_key = f"mol_rspace_pair_kernel<{sp.jmax},{tile}>", "mol_rspace_pair_kernel"
-            if a.state == "parity":
-                kernel, traffic_key = f"mol_rspace_pair_kernel<{sp.jmax},{tile},parity>", "mol_rspace_pair_kernel_parity"
+            if rows_of(sp, main_form["plans"][0]) == sp.nrot:
+                kernel, traffic_key = f"mol_rspace_pair_kernel<{sp.jmax},{tile},reachable>", "mol_rspace_pair_kernel_rows"
         elif one and sp.jmax <= 8:
             tile = main_form["plans"][0][2] or (16 if sp.jmax >= 5 else 32)   # the tiled kernel's rule
             kernel, traffic_key = f"mol_rspace_kernel<{sp.jmax},{tile}>", "mol_rspace_kernel"
@@ -538,7 +546,7 @@ def main():
     roof_step = {"bound": "hbm", "achieved": step_bytes / (per_step(1) / 1e3) / 1e9, "peak": peak,
                  "unit": "GB/s", "frac": step_bytes / (per_step(1) / 1e3) / 1e9 / peak,
                  "bytes_per_step": step_bytes, "ms_per_step": per_step(1),
-                 "note": "molecular step (all its kernels) vs one read and one write of the FP32 state"}
+                 "note": "molecular step (all its kernels) vs one read and one write of the FP32 rows that it processes"}
     roof_fdtd = fdtd_roofline(wl, per_step(0), per_step(2), peak)
 
     e2e = None

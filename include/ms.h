@@ -94,9 +94,8 @@ enum { MS_MOL_AUTO = 0, MS_MOL_FUSED = 1, MS_MOL_STREAMING = 2 };
  * ground-state start (each coupling changes j by one and swaps the
  * surfaces), which halves the state and the work.  Results are those of the
  * full state.  Up to J = 4 the point-resident kernels run them (the fused
- * layout only at N_r = 128); from J = 5 on the two-points-a-thread tiled
- * kernel in the streaming layout with the FP32 kinetic pass (MS_EUNSUPPORTED
- * otherwise).  Their plan follows this rule (ms_set_species_plan accepts no
+ * layout only at N_r = 128); from J = 5 on the static rule's kernels in the
+ * streaming layout with the FP32 kinetic pass (MS_EUNSUPPORTED otherwise).  Their plan follows this rule (ms_set_species_plan accepts no
  * other). */
 enum { MS_STATE_FULL = 0, MS_STATE_PARITY = 1 };
 /* Step replay.  MS_GRAPHS_AUTO: ms_step captures the launches of whole
@@ -107,8 +106,9 @@ enum { MS_STATE_FULL = 0, MS_STATE_PARITY = 1 };
  * same results bit for bit. */
 enum { MS_GRAPHS_AUTO = 0, MS_GRAPHS_OFF = 1 };
 /* A species' plan: its layout (MS_MOL_FUSED or MS_MOL_STREAMING) and the
- * kernel of its R-space pass.  MS_KERN_POINT: one CTA of 2 N_r threads per
- * molecule, thread = (radial point, surface) (J <= 4; fused at N_r 128).
+ * kernel of its R-space pass.  MS_KERN_POINT: every row that can be populated
+ * held by one thread per radial point (all the rows where a loaded state
+ * populates others; J <= 4; fused at N_r 128).
  * MS_KERN_TILE: persistent CTAs that each walk a share of the molecules, one
  * molecule at a time over tiles of `chunk` radial points of all rows, staged
  * by tensor copies (streaming; chunk 32 or 16 for J <= 8, 8 for J 9..16;
@@ -116,12 +116,14 @@ enum { MS_GRAPHS_AUTO = 0, MS_GRAPHS_OFF = 1 };
  * radial points (4, 8, 16 or 32) of all rows (any J).  MS_KERN_PAIR: the
  * tiled kernel's schedule with two neighbouring radial points per thread and
  * packed FP32x2 arithmetic (streaming; chunk 32 or 16 for J <= 4, 16 or 8
- * for J 5..8, 8 for J 9..16; chunk 0: 8 from J = 5 on, else 32; the
- * parity-reduced state: 16 for J 5..8).  MS_KERN_DEFAULT: the
- * static rule (the first that applies of point for J <= 4, pair from J = 5
- * on in the streaming layout, tile, chunk at the widest fitting chunk).
- * Parity-reduced and d(R) species run
- * the point-resident kernel only.  Every plan computes the same step; their
+ * for J 5..8, 8 for J 9..16; chunk 0: 8 from J = 5 on, else 32).
+ * MS_KERN_DEFAULT: the static rule.  J <= 4: point.  J 5..8 in the streaming
+ * layout: the rotor's columns held by a thread per radial point, over the rows
+ * that can be populated; J 9..16: pair over those rows.  Where a loaded state
+ * populates others, and otherwise: the first that applies of pair from J = 5
+ * on in the streaming layout, tile, chunk at the widest fitting chunk.
+ * Parity-reduced species follow the rule; d(R) species run the point-resident
+ * kernel only.  Every plan computes the same step; their
  * results differ by FP32 rounding.
  * Autotuning (ms_options.autotune = MS_TUNE_MEASURE): ms_create times every
  * plan a species can run on a sandbox copy of up to 2,048 of its molecules

@@ -46,19 +46,6 @@ namespace ms {
 
 namespace {
 
-// (x) * (c + i s) with c = ch + cl, s = sh + sl (compensated)
-__device__ __forceinline__ float2 cmul_c(float2 x, float ch, float sh, float cl, float sl) {
-  const float re_lo = fmaf(x.x, cl, -x.y * sl);
-  const float im_lo = fmaf(x.x, sl, x.y * cl);
-  return make_float2(fmaf(x.x, ch, fmaf(-x.y, sh, re_lo)), fmaf(x.x, sh, fmaf(x.y, ch, im_lo)));
-}
-// same, plus an addend folded into the last rounding
-__device__ __forceinline__ float2 cmul_c_add(float2 x, float4 w, float2 a) {
-  const float re_lo = fmaf(x.x, w.z, fmaf(-x.y, w.w, a.x));
-  const float im_lo = fmaf(x.x, w.w, fmaf(x.y, w.z, a.y));
-  return make_float2(fmaf(x.x, w.x, fmaf(-x.y, w.y, re_lo)), fmaf(x.x, w.y, fmaf(x.y, w.x, im_lo)));
-}
-
 // 16-byte asynchronous global -> shared copies (per thread), completed by
 // cp.async.wait_group.
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -976,8 +963,9 @@ static bool rspace_ok(int nr, int jmax);
 // resident one does not and it applies, unless the plan names another kernel.
 static bool pair_ok(int nr, int jmax) { return (nr == 64 || nr == 128 || nr == 256) && jmax <= 16; }
 // The column kernel runs the reachable rows of a streaming species from J = 5
-// to 8 (below, a thread holds the whole rotor; above, half a side's columns no
-// longer fit a thread's registers).
+// to 8: 6.1 to 6.5 ps a row and point at N_r = 128, 6.4 at 256 and 6.9 at 64,
+// against 8.0 for the two-points-a-thread kernel.  Below, a thread holds the
+// whole rotor; above, half a side's columns no longer fit a thread's registers.
 static bool use_col(const SpeciesDev& sp) {
   return sp.path == MS_MOL_STREAMING && sp.par && sp.jmax >= 5 && sp.jmax <= 8;
 }
@@ -1179,8 +1167,6 @@ __global__ void __launch_bounds__(FFTShape<NR>::THREADS)
 
 size_t mol_state_smem(int nr, int rows) { return (size_t)rows * (nr + kPad) * sizeof(float2); }
 
-static int threads_for(int nr) { return nr == 256 ? 256 : 128; }
-
 static size_t step_smem(int nr, int nrot, int ch, bool fused) {
   const int rows = 2 * nrot;
   const int jm = (int)std::lround(std::sqrt((double)nrot)) - 1;
@@ -1374,8 +1360,8 @@ bool mol_tensor_maps_available() { return tensor_map_encoder() != nullptr; }
 // on the reachable rows alone: half of a full-form state's bytes and work (its
 // other rows are zeros before and after every step).  Plans that name another
 // kernel process every row.  A step over every row against one over the
-// reachable ones: 22.0 and 11.3 ms with 100,000 molecules at J = 8, N_r = 128
-// (streaming), 2.70 and 1.97 ms with 50,000 at J = 4, N_r = 128 (fused).
+// reachable ones: 22.0 and 9.9 ms with 100,000 molecules at J = 8, N_r = 128
+// (streaming), 2.70 and 1.16 ms with 50,000 at J = 4, N_r = 128 (fused).
 bool mol_reachable_rows(const SpeciesDev& sp) {
   if (sp.par_form) return true;
   if (sp.all_rows) return false;

@@ -48,11 +48,6 @@ cplx expm1i(double a) {
 
 float2 f2(cplx z) { return make_float2((float)z.real(), (float)z.imag()); }
 
-float4 hilo(cplx z) {
-  const float ch = (float)z.real(), sh = (float)z.imag();
-  return make_float4(ch, sh, (float)(z.real() - (double)ch), (float)(z.imag() - (double)sh));
-}
-
 struct Alloc {
   void* (*fn)(size_t, void*) = nullptr;
   void (*fr)(void*, void*) = nullptr;
