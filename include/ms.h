@@ -95,8 +95,8 @@ enum { MS_MOL_AUTO = 0, MS_MOL_FUSED = 1, MS_MOL_STREAMING = 2 };
  * surfaces), which halves the state and the work.  Results are those of the
  * full state.  Up to J = 4 the point-resident kernels run them (the fused
  * layout only at N_r = 128); from J = 5 on the static rule's kernels in the
- * streaming layout with the FP32 kinetic pass (MS_EUNSUPPORTED otherwise).  Their plan follows this rule (ms_set_species_plan accepts no
- * other). */
+ * streaming layout with the FP32 kinetic pass (MS_EUNSUPPORTED otherwise).
+ * Their plan follows this rule (ms_set_species_plan accepts no other). */
 enum { MS_STATE_FULL = 0, MS_STATE_PARITY = 1 };
 /* Step replay.  MS_GRAPHS_AUTO: ms_step captures the launches of whole
  * molecular cycles (at least 8 field steps, a multiple of mol_substeps) once
@@ -264,7 +264,11 @@ ms_status ms_create(const ms_grid_desc* grid, const ms_materials_desc* materials
  * E update (the paper's leap-frog with the molecular current).  With
  * MS_GRAPHS_AUTO the launches of whole cycles replay from a CUDA graph
  * captured on first use (and again after ms_set_prescribed_field,
- * ms_set_replay_field or ms_set_detectors change what the kernels read). */
+ * ms_set_replay_field or ms_set_detectors change what the kernels read).
+ * Steps that the caller captures into a graph of its own replay from whatever
+ * step the handle has reached, also between other calls; capture them again
+ * after ms_set_species_plan, or after ms_load of a state that populates rows
+ * the j = 0 start cannot reach: both can change the order of the stored rows. */
 ms_status ms_step(ms_sim* sim, int64_t n);
 
 /* Allocation-free stepping.  The paper has no counterpart: this is a library

@@ -84,6 +84,7 @@ struct ms_sim {
   long long* d_step = nullptr;  // the step counter's two slots
   int slot = 0;                 // the one that holds the current step
   int gslot = 0;                // the one the captured cycle starts from
+  int home = -1;                // the one every call ends on once the caller has captured steps; -1 before
   // device address of the library's fixed scratch array (ms_step_noalloc),
   // looked up at create with the handle's device current; null if that failed
   float2* noalloc_base = nullptr;
@@ -1258,12 +1259,18 @@ static void step_once(ms_sim* s, float2* const* scratch, bool last, const FieldR
   }
 }
 
-// A call that the caller captures ends on the counter slot it began with, so that
-// its graph can be replayed.
 static void keep_slot(ms_sim* s, int slot) {
   if (s->slot == slot) return;
   ms::launch_step_counter(s->d_step + s->slot, s->d_step + slot, 0, s->stream);
   s->slot = slot;
+}
+
+// The end of a call's steps.  A call that the caller captures ends on the counter
+// slot it began with, and so does every call after it: the caller's graph can be
+// replayed, by itself and between other calls.
+static void end_steps(ms_sim* s, int begin, bool captured) {
+  if (captured && s->home < 0) s->home = begin;
+  if (s->home >= 0) keep_slot(s, s->home);
 }
 
 // Steps of a captured cycle: whole molecular cycles, at least 8 steps, or a batch
@@ -1324,7 +1331,7 @@ ms_status ms_step(ms_sim* s, int64_t n) {
     }
   }
   for (int64_t q = 0; q < n; ++q) step_once(s, nullptr, q == n - 1);
-  if (cs != cudaStreamCaptureStatusNone) keep_slot(s, slot0);
+  end_steps(s, slot0, cs != cudaStreamCaptureStatusNone);
   return cudaGetLastError() == cudaSuccess ? MS_OK : MS_ECUDA;
 }
 
@@ -1348,7 +1355,7 @@ ms_status ms_step_noalloc(ms_sim* s, int64_t n) {
   if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess) return MS_ECUDA;
   const int slot0 = s->slot;
   for (int64_t q = 0; q < n; ++q) step_once(s, scratch, q == n - 1);
-  if (cs != cudaStreamCaptureStatusNone) keep_slot(s, slot0);
+  end_steps(s, slot0, cs != cudaStreamCaptureStatusNone);
   return cudaGetLastError() == cudaSuccess ? MS_OK : MS_ECUDA;
 }
 
@@ -1567,6 +1574,7 @@ ms_status ms_record_local_fields(ms_sim* s, const int64_t* mol_ids, int64_t m, f
       step_once(s, nullptr, q == nsteps - 1, &rec);
       rec.out += (size_t)m * 3;
     }
+    end_steps(s, s->slot, false);
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpyAsync(dst, d_out, nout, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess)

@@ -160,3 +160,39 @@ def test_steps_captured_by_the_caller_replay(B, captured):
     b.step(16)
     for x, y in zip(out(a), out(b)):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("captured", [1, 2])
+def test_replays_between_other_calls(B, captured):
+    """A caller's graph replayed after odd numbers of plain and of recorded
+    steps starts from the step that those have reached."""
+    import torch
+    wl = W.custom("between", 20, 12, 48, src_k=14, pulses=[[1e10, 1.5, 1e-15, 2e-16]], layer=(20, 24), n_per_sim=40,
+                  species=[W.species_config0(jmax=1)], seed=3, nsteps=60)
+
+    def out(sim):
+        r = sim.populations(), sim.dipoles(), sim.fields(B.MS_FIELD_E), sim.fields(B.MS_FIELD_H)
+        sim.close()
+        return r
+
+    a = B.Simulation(wl, step_graphs=B.MS_GRAPHS_OFF)
+    a.step(5 + 3 * captured + 1 + 3 + 17)
+    b = B.Simulation(wl)
+    b.step(5)
+    b.populations()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=b.stream):
+        b.step(captured)
+
+    def replay():
+        with torch.cuda.stream(b.stream):
+            g.replay()
+
+    replay()
+    b.step(1)
+    replay()
+    b.record_local_fields(np.arange(4), 3)
+    replay()
+    b.step(17)
+    for x, y in zip(out(a), out(b)):
+        assert np.array_equal(x, y)
