@@ -22,11 +22,14 @@
 // instructions a row are unrolled.  With every phase unrolled (100 KB of code
 // at J = 8) the pass waited for instructions: 8.8 ps a row and point; with the
 // rows' loads one at a time for those loads: 12.5 ps.  What is left of that
-// wait bounds it (a thread per row: 8.0 ps; now 6.1 to 6.5; 3.5 ps is HBM's).
+// wait bounds it (a thread per row: 8.0 ps; now 5.9 to 6.5 at N_r = 128; 3.5 ps is
+// HBM's).
 //
-// The coupling's exponential series S = sum_{n=1..N} (i theta M)^n / n! eta is
-// summed by Horner's rule, S = i theta M y_1, y_n = eta + (i theta / (n + 1)) M
-// y_{n+1}, y_N = eta.
+// The coupling's exponential series S = sum_{n=1..N} T_n, T_1 = i theta M eta,
+// T_n = (i theta / n) M T_{n-1}, is summed by Horner's rule on T_1: S = P_1, P_n
+// = T_1 + (i theta / (n + 1)) M P_{n+1}, P_N = T_1.  On eta itself (S = i theta M
+// (eta + (i theta / 2) M (eta + ..))) every step would round at eta's size, not at
+// T_1's, which costs 3% in the populations' and dipoles' error against 64 bits.
 #include "mol_common.cuh"
 
 namespace ms {
@@ -40,12 +43,13 @@ struct ColDims {
     for (int m = a; m < b; ++m) n += len(m);
     return n;
   }
-  // columns 0 .. K - 1 on the low warps: the split with the smallest larger share
+  // columns 0 .. K - 1 on the low warps: the split with the smallest larger share, of two such the one with the
+  // larger low share (J = 7: 21 and 15 rows took 23.4 ms where 15 and 21 took 23.9)
   static constexpr int split() {
     int best = 2;
     for (int k = 3; k <= J; ++k) {
       const int a = rows(0, k), b = rows(k, J + 1), c = rows(0, best), d = rows(best, J + 1);
-      if ((a > b ? a : b) < (c > d ? c : d)) best = k;
+      if ((a > b ? a : b) <= (c > d ? c : d)) best = k;
     }
     return best;
   }
@@ -61,9 +65,9 @@ struct ColDims {
   static constexpr int NG = shell(1);  // ground rows
   // rows whose loads a warp keeps in flight before the coupling, and after it for the ground and the excited rows:
   // few passes over a warp's rows (at J = 8: 21, 12 and 9) with few idle places.  Six throughout took 7.29, 6.97,
-  // 7.43 and 6.84 ps a row and point at J = 5, 6, 7 and 8; these 6.34, 6.37, 6.13 and 6.51.
-  static constexpr int EB = J == 8 ? 11 : (J == 6 ? 7 : 9);
-  static constexpr int GB = J == 5 ? 4 : (J == 6 ? 7 : (J == 7 ? 9 : 6)), XB = J == 5 ? 6 : (J == 6 ? 7 : 9);
+  // 7.43 and 6.84 ps a row and point at J = 5, 6, 7 and 8; these 6.07, 5.95, 6.03 and 6.50.
+  static constexpr int EB = J == 8 ? 11 : (J == 7 ? 8 : (J == 6 ? 7 : 9));
+  static constexpr int GB = J == 5 ? 4 : (J == 8 ? 6 : 7), XB = J == 5 ? 6 : (J == 6 ? 7 : 9);
 };
 
 constexpr int kColThreads = 128;
@@ -90,8 +94,7 @@ struct ColWarp {
   }
 
   // Y <- S of the series on Y = eta (at this lane); row(j, c) of Y at Y + 32 (at(j) + sg c)
-  template <class Eta>
-  static __device__ __forceinline__ void series(float2* Y, bool mir, int nterms, float fz, float fx, float fy, Eta&& eta) {
+  static __device__ __forceinline__ void series(float2* Y, bool mir, int nterms, float fz, float fx, float fy) {
     const int sg = mir ? -32 : 32;  // from one column to the next
     float2 v[N], w[N];
     auto load = [&]() {
@@ -113,8 +116,8 @@ struct ColWarp {
       if constexpr (c >= C0 && c < C1) return v[ix(c, j)];
       else return (Y + sg * c)[32 * at(j)];
     };
-    // base + i (M v) at row (c, j); z2, x2, y2 the field's factors
-    auto coupled = [&](auto cc, auto jc, float2 z2, float2 x2, float2 y2, float2 base) -> float2 {
+    // i (M v) at row (c, j); z2, x2 and y the field's factors
+    auto coupled = [&](auto cc, auto jc, float2 z2, float2 x2, float y) -> float2 {
       constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
       auto sum2 = [&](auto cf0, auto cf1, auto c2) {  // cf0 (c2, j - 1) + cf1 (c2, j + 1)
         constexpr int cq = decltype(c2)::value, mq = cq < 0 ? -cq : cq;
@@ -131,38 +134,49 @@ struct ColWarp {
       const float2 ap = sum2([] { return c_pd(j, c); }, [] { return c_pu(j, c); }, std::integral_constant<int, c - 1>());
       const float2 am = sum2([] { return c_md(j, c); }, [] { return c_mu(j, c); }, std::integral_constant<int, c + 1>());
       const float2 t = fma2(z2, az, mul2(x2, add2(ap, am)));
-      const float2 e = fma2(y2, sub2(ap, am), base);
-      return make_float2(e.x - t.y, e.y + t.x);
+      const float2 d = sub2(ap, am);
+      return make_float2(fmaf(y, d.x, -t.y), fmaf(y, d.y, t.x));
     };
     load();
-#pragma unroll 1
-    for (int n = nterms; n >= 2; --n) {
-      const float cn = 1.f / (float)n;
-      const float2 z2 = dup2(fz * cn), x2 = dup2(fx * cn), y2 = dup2(fy * cn);
-      if (n == nterms) {
-        each<true>(mir, [&](auto cc, auto jc) {
-          constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
-          w[ix(c, j)] = coupled(cc, jc, z2, x2, y2, v[ix(c, j)]);
-        });
-      } else {  // three terms and more: eta again
-        each<true>(mir, [&](auto cc, auto jc) {
-          constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
-          w[ix(c, j)] = coupled(cc, jc, z2, x2, y2, eta(j, at(j) + (mir ? -c : c)));
-        });
-      }
-      store();
-      load();
-    }
-    const float2 z2 = dup2(fz), x2 = dup2(fx), y2 = dup2(fy);
-    each<true>(mir, [&](auto cc, auto jc) {
+    each<true>(mir, [&](auto cc, auto jc) {  // T_1
       constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
-      w[ix(c, j)] = coupled(cc, jc, z2, x2, y2, make_float2(0.f, 0.f));
+      w[ix(c, j)] = coupled(cc, jc, dup2(fz), dup2(fx), fy);
     });
     store();
+    if (nterms == 2) {
+      load();
+      const float2 z2 = dup2(0.5f * fz), x2 = dup2(0.5f * fx);
+      each<true>(mir, [&](auto cc, auto jc) {
+        constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
+        w[ix(c, j)] = add2(v[ix(c, j)], coupled(cc, jc, z2, x2, 0.5f * fy));
+      });
+      store();
+    } else if (nterms > 2) {
+      float2 t1[N];  // in local memory (an index that the compiler does not know): no registers of the other branch
+      int z;
+      asm volatile("mov.u32 %0, 0;" : "=r"(z));
+      each<true>(mir, [&](auto cc, auto jc) {
+        constexpr int k = ix(decltype(cc)::value, decltype(jc)::value);
+        t1[k + z] = w[k];
+      });
+#pragma unroll 1
+      for (int n = nterms; n >= 2; --n) {
+        load();
+        const float cn = 1.f / (float)n;
+        const float2 z2 = dup2(fz * cn), x2 = dup2(fx * cn);
+        each<true>(mir, [&](auto cc, auto jc) {
+          constexpr int k = ix(decltype(cc)::value, decltype(jc)::value);
+          w[k] = add2(t1[k + z], coupled(cc, jc, z2, x2, fy * cn));
+        });
+        store();
+      }
+    }
   }
 
   // Dipole sums of Y = s': over pairs of rows of one column (Z) and of columns c, c + 1 (S+, S-); each pair
-  // joins a ground and an excited row, and conj(g) e and conj(e) g give the same Re (P + M), Im (P - M)
+  // joins a ground and an excited row, and conj(g) e and conj(e) g give the same Re (P + M), Im (P - M).
+  // Column 0's pairs with columns 1 and -1 are taken together: what the two have in common (the first-order
+  // Im (g* e), much larger than the dipole) cancels before it is rounded in a product.
   static __device__ __forceinline__ void dipole(const float2* Y, bool mir, float2& ax, float& ay, float2& az) {
     const int sg = mir ? -32 : 32;
     float2 v[N];
@@ -174,23 +188,33 @@ struct ColWarp {
       constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
       if constexpr (j < J) az = fma2(dup2(c_zu(j, c)), mul2(v[ix(c, j)], v[ix(c, j + 1)]), az);
     });
-    each<false>(mir, [&](auto cc, auto jc) {
+    each<true>(mir, [&](auto cc, auto jc) {
       constexpr int c = decltype(cc)::value, j = decltype(jc)::value;
       if constexpr (c < J) {
-        auto up = [&](auto j2) -> float2 {
-          constexpr int jq = decltype(j2)::value;
-          if constexpr (c + 1 < C1) return v[ix(c + 1, jq)];
-          else return (Y + sg * (c + 1))[32 * at(jq)];
-        };
         constexpr bool hi = j + 1 <= J, lo = j - 1 >= c + 1;
-        float2 t = make_float2(0.f, 0.f);
-        if constexpr (hi) t = mul2(dup2(c_mu(j, c)), up(std::integral_constant<int, j + 1>()));
-        if constexpr (lo && hi) t = fma2(dup2(c_md(j, c)), up(std::integral_constant<int, j - 1>()), t);
-        else if constexpr (lo) t = mul2(dup2(c_md(j, c)), up(std::integral_constant<int, j - 1>()));
+        auto sum = [&](auto up) {  // over the neighbours (j + 1, c + 1) and (j - 1, c + 1)
+          float2 t = make_float2(0.f, 0.f);
+          if constexpr (hi) t = mul2(dup2(c_mu(j, c)), up(std::integral_constant<int, j + 1>()));
+          if constexpr (lo && hi) t = fma2(dup2(c_md(j, c)), up(std::integral_constant<int, j - 1>()), t);
+          else if constexpr (lo) t = mul2(dup2(c_md(j, c)), up(std::integral_constant<int, j - 1>()));
+          return t;
+        };
         if constexpr (hi || lo) {
           const float2 q = v[ix(c, j)];
-          ax = fma2(q, t, ax);
-          ay = fmaf(q.y, t.x, fmaf(-q.x, t.y, ay));
+          float2 tx, ty;
+          if constexpr (c == 0) {  // not mirrored
+            static_assert(C1 > 1, "column 1 stands beside column 0");
+            auto m1 = [&](auto jq) { return (Y - 32)[32 * at(decltype(jq)::value)]; };
+            tx = sum([&](auto jq) { return sub2(v[ix(1, decltype(jq)::value)], m1(jq)); });
+            ty = sum([&](auto jq) { return add2(v[ix(1, decltype(jq)::value)], m1(jq)); });
+          } else {
+            tx = ty = sum([&](auto jq) -> float2 {
+              if constexpr (c + 1 < C1) return v[ix(c + 1, decltype(jq)::value)];
+              else return (Y + sg * (c + 1))[32 * at(decltype(jq)::value)];
+            });
+          }
+          ax = fma2(q, tx, ax);
+          ay = fmaf(q.y, ty.x, fmaf(-q.x, ty.y, ay));
         }
       }
     });
@@ -203,8 +227,7 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
   constexpr int NROT = D::NROT, NG = D::NG;
   __shared__ float2 Ys[NROT][32];
   __shared__ int s_vt[NROT + 3];  // row -> its shell's row of the phase table (and three past the end)
-  __shared__ float s_red[4][10];
-  __shared__ float s_fin[8], s_fin_lo[2];
+  __shared__ float s_fin[8], s_fin_lo[2];  // P_g, P_e, Re(S+ + S-), Im(S+ - S-), 2 Re Z, absorbed (2), rounding residuals
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int lm = blockIdx.x, m = sp.mol[lm], NR = sp.nr;
   const float4 f = __ldg(&sp.fld[lm]);  // (theta E'_z, theta E'_x/2, theta E'_y/2, terms)
@@ -258,11 +281,8 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
     }
     __syncthreads();
     // ---- Y <- S
-    auto eta = [&](int j, int row) {
-      return cmul(__ldg(reinterpret_cast<const float2*>(vt + j * NR)), add2(s[row * NR], __ldg(d + row * NR)));
-    };
-    if (w & 1) ColWarp<J, false>::series(Y, mir, nterms, f.x, fx, f.z, eta);
-    else ColWarp<J, true>::series(Y, mir, nterms, f.x, fx, f.z, eta);
+    if (w & 1) ColWarp<J, false>::series(Y, mir, nterms, f.x, fx, f.z);
+    else ColWarp<J, true>::series(Y, mir, nterms, f.x, fx, f.z);
     // ---- d1 = (V - 1) u + V^{1/2} S, mask, s' = s + (d2 + d1) + cfix s; a surface at a time
     const bool masked = mk.x < 1.f;
     static_for<0, 2>([&](auto sfc) {
@@ -312,43 +332,50 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
     if (w & 1) ColWarp<J, false>::dipole(Y, mir, ax, ay, az);
     else ColWarp<J, true>::dipole(Y, mir, ax, ay, az);
   }
-  // ---- block reduction: populations compensated, the rest plain FP32; mirrored columns count E'_x reversed
-  const float dx = ax.x + ax.y;
-  float v[8] = {hi.x, hi.y, ab[0], ab[1], mir ? -dx : dx, ay, 2.f * (az.x + az.y), rnd.x + rnd.y};
-  float l2[2] = {lo.x, lo.y};
+  // ---- block sums: a lane's values of the four warps first, then a tree over the lanes; warp w takes the
+  // quantities w and w + 4.  Mirrored columns count E'_x reversed, and what is much larger than the dipole in
+  // each (the first-order Im (g* e)) cancels against the other lane by lane: a tree over each warp's own part
+  // rounds at that part's size instead (the dipoles' error against 64 bits at J = 8, N_r = 128, with the same in
+  // dipole(): 1.75e-7, now 1.31e-7).
+  __syncthreads();  // the last points' dipole has read Y
+  float* const red = reinterpret_cast<float*>(&Ys[0][0]);
+  {
+    const float dx = ax.x + ax.y;
+    const float v[10] = {hi.x, hi.y, mir ? -dx : dx, ay, 2.f * (az.x + az.y), ab[0], ab[1], rnd.x + rnd.y, lo.x, lo.y};
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const float h2 = __shfl_xor_sync(0xffffffffu, v[k], o);
-      const float g2 = __shfl_xor_sync(0xffffffffu, l2[k], o);
-      acc2(v[k], l2[k], h2);
-      l2[k] += g2;
-    }
-#pragma unroll
-    for (int k = 2; k < 8; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s_red[w][k] = v[k];
-    s_red[w][8] = l2[0];
-    s_red[w][9] = l2[1];
+    for (int k = 0; k < 10; ++k) red[k * kColThreads + t] = v[k];
   }
   __syncthreads();
-  if (t < 8) {
+#pragma unroll
+  for (int k = w; k < 8; k += 4) {
     float h = 0.f, l = 0.f;
 #pragma unroll
     for (int ww = 0; ww < 4; ++ww) {
-      acc2(h, l, s_red[ww][t]);
-      if (t < 2) l += s_red[ww][8 + t];
+      acc2(h, l, red[k * kColThreads + 32 * ww + lane]);
+      if (k < 2) l += red[(8 + k) * kColThreads + 32 * ww + lane];
     }
-    s_fin[t] = h + l;
-    if (t < 2) s_fin_lo[t] = l - (s_fin[t] - h);
+    if (k < 2) {  // populations compensated
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float h2 = __shfl_xor_sync(0xffffffffu, h, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
+        acc2(h, l, h2);
+        l += l2;
+      }
+    } else {
+      h += l;
+      l = 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+    }
+    if (lane == 0) {
+      s_fin[k] = h + l;
+      if (k < 2) s_fin_lo[k] = l - (s_fin[k] - h);
+    }
   }
   __syncthreads();
   if (t < 3) {  // lab dipole: mu = O mu', mu' = d dR (Re(S+ + S-), Im(S+ - S-), 2 Re Z)
     const float* O = md.rot + 9 * (long long)m + 3 * t;
-    const float lab = (float)sp.dipole * sp.dR * (O[0] * s_fin[4] + O[1] * s_fin[5] + O[2] * s_fin[6]);
+    const float lab = (float)sp.dipole * sp.dR * (O[0] * s_fin[2] + O[1] * s_fin[3] + O[2] * s_fin[4]);
     const double nl = (double)lab;
     md.dmu[3 * (long long)m + t] = nl - old;
     md.mu[3 * (long long)m + t] = nl;
@@ -357,7 +384,7 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
     md.pop[2 * (long long)m + (t - 3)] = P;
     if (!isfinite(P)) atomicOr(err, kErrNonFinite);
   } else if (t < 7) {
-    md.absorbed[2 * (long long)m + (t - 5)] = old + (double)s_fin[t - 3] * (double)sp.dR;
+    md.absorbed[2 * (long long)m + (t - 5)] = old + (double)s_fin[t] * (double)sp.dR;
   } else if (t == 7) {
     md.ncorr[m] = rounding_feedback(s_fin[7], s_fin[0] + s_fin[1]);
   }

@@ -12,18 +12,18 @@
 // for every term and its barriers and the idle half of the larger surface's
 // threads cost a third of the time.
 //
-// The coupling's exponential series S = sum_{n=1..N} (i theta M)^n / n! eta is
-// summed by Horner's rule, S = i theta M y_1, y_n = eta + (i theta / (n + 1)) M
-// y_{n+1}, y_N = eta: each row's S goes straight into the update.  Values are
-// kept as (Re, Im) pairs and multiplied by real coefficients as packed FP32x2
-// products, whose equal constants are immediates.
+// The coupling's exponential series S = sum_{n=1..N} T_n, T_1 = i theta M eta,
+// T_n = (i theta / n) M T_{n-1}, is summed by Horner's rule on T_1: S = P_1, P_n
+// = T_1 + (i theta / (n + 1)) M P_{n+1}, P_N = T_1 (on eta itself every step would
+// round at eta's size, not at T_1's).  Values are kept as (Re, Im) pairs and
+// multiplied by real coefficients as packed FP32x2 products, whose equal
+// constants are immediates.
 //
 // What bounds it: issue slots and instruction fetch (2,900 instructions of
 // straight-line code at J = 4, about 85 a row and point; twelve warps an SM by
 // registers), then HBM.  Per row and point of the reachable rows: the R-space
-// pass at J = 4, N_r = 64 (375,000 molecules) takes 4.42 ps, 5.4 TB/s, against
-// 7.13 for a thread per surface; the fused step at J = 4, N_r = 128
-// (187,500 molecules) 6.87 against 12.14 ps.
+// pass at J = 4, N_r = 64 takes 4.36 ps, 5.5 TB/s, against 7.13 for a thread per
+// surface; the fused step at J = 4, N_r = 128 6.79 against 12.14 ps.
 //
 // FUSED (N_r = 128): the kinetic pass runs in the same kernel.  The state
 // arrives by one bulk copy and stays in shared memory; the FFT turns it into
@@ -97,8 +97,8 @@ __device__ __forceinline__ void rotor_point(const SpeciesDev& sp, int p, float2*
   };
 
   float2 v[NROT], q[NROT];
-  // base + i (M v) at (j, m); z2, x2, y2 the field's factors
-  auto coupled = [&](auto jc, auto mc, float2 z2, float2 x2, float2 y2, float2 base) -> float2 {
+  // i (M v) at (j, m); z2, x2 and y the field's factors
+  auto coupled = [&](auto jc, auto mc, float2 z2, float2 x2, float y) -> float2 {
     constexpr int j = decltype(jc)::value, m = decltype(mc)::value;
     auto sum2 = [&](auto cf0, auto cf1, auto c2) {  // cf0 (j - 1, c2) + cf1 (j + 1, c2)
       constexpr int cq = decltype(c2)::value, mq = cq < 0 ? -cq : cq;
@@ -113,40 +113,53 @@ __device__ __forceinline__ void rotor_point(const SpeciesDev& sp, int p, float2*
     const float2 ap = sum2([] { return c_pd(j, m); }, [] { return c_pu(j, m); }, std::integral_constant<int, m - 1>());
     const float2 am = sum2([] { return c_md(j, m); }, [] { return c_mu(j, m); }, std::integral_constant<int, m + 1>());
     const float2 r = fma2(z2, az, mul2(x2, add2(ap, am)));
-    const float2 e = fma2(y2, sub2(ap, am), base);
-    return make_float2(e.x - r.y, e.y + r.x);
+    const float2 d = sub2(ap, am);
+    return make_float2(fmaf(y, d.x, -r.y), fmaf(y, d.y, r.x));
   };
   auto eta = [&](auto jc, auto mc) -> float2 {  // V^{1/2} (s + d2)
     constexpr int row = D::row(decltype(jc)::value, decltype(mc)::value);
     return cmul(vh_at(jc), add2(s_at(row), d_at(row)));
   };
   for_channels<J>([&](auto jc, auto mc) { v[D::at(decltype(jc)::value, decltype(mc)::value)] = eta(jc, mc); });
-  // ---- y_1 by Horner's rule
-#pragma unroll 1
-  for (int n = nterms; n >= 2; --n) {
-    const float cn = 1.f / (float)n;
-    const float2 z2 = dup2(f.x * cn), x2 = dup2(f.y * cn), y2 = dup2(f.z * cn);
-    if (n == nterms) {
-      for_channels<J>([&](auto jc, auto mc) {
-        constexpr int k = D::at(decltype(jc)::value, decltype(mc)::value);
-        q[k] = coupled(jc, mc, z2, x2, y2, v[k]);
-      });
-    } else {  // three terms and more: eta again
-      for_channels<J>([&](auto jc, auto mc) {
-        q[D::at(decltype(jc)::value, decltype(mc)::value)] = coupled(jc, mc, z2, x2, y2, eta(jc, mc));
-      });
-    }
+  // ---- S into q
+  {
+    const float2 z2 = dup2(f.x), x2 = dup2(f.y);
+    for_channels<J>([&](auto jc, auto mc) {  // T_1
+      q[D::at(decltype(jc)::value, decltype(mc)::value)] = coupled(jc, mc, z2, x2, f.z);
+    });
+  }
+  if (nterms == 2) {
 #pragma unroll
     for (int k = 0; k < NROT; ++k) v[k] = q[k];
+    const float2 z2 = dup2(0.5f * f.x), x2 = dup2(0.5f * f.y);
+    for_channels<J>([&](auto jc, auto mc) {
+      constexpr int k = D::at(decltype(jc)::value, decltype(mc)::value);
+      q[k] = add2(v[k], coupled(jc, mc, z2, x2, 0.5f * f.z));
+    });
+  } else if (nterms > 2) {
+    float2 t1[NROT];
+#pragma unroll
+    for (int k = 0; k < NROT; ++k) t1[k] = q[k];
+#pragma unroll 1
+    for (int n = nterms; n >= 2; --n) {
+#pragma unroll
+      for (int k = 0; k < NROT; ++k) v[k] = q[k];
+      const float cn = 1.f / (float)n;
+      const float2 z2 = dup2(f.x * cn), x2 = dup2(f.y * cn);
+      for_channels<J>([&](auto jc, auto mc) {
+        constexpr int k = D::at(decltype(jc)::value, decltype(mc)::value);
+        q[k] = add2(t1[k], coupled(jc, mc, z2, x2, f.z * cn));
+      });
+    }
   }
-  // ---- S = i theta M y_1, d1 = (V - 1) u + V^{1/2} S, mask, s' = s + (d2 + d1) + cfix s
+  // ---- d1 = (V - 1) u + V^{1/2} S, mask, s' = s + (d2 + d1) + cfix s
   {
-    const float2 z2 = dup2(f.x), x2 = dup2(f.y), y2 = dup2(f.z), cf = dup2(cfix);
+    const float2 cf = dup2(cfix);
     const bool masked = mk < 1.f;
     float b2 = 0.f;
     for_channels<J>([&](auto jc, auto mc) {
       constexpr int j = decltype(jc)::value, m = decltype(mc)::value, k = D::at(j, m), row = D::row(j, m), sf = j & 1;
-      const float2 S = coupled(jc, mc, z2, x2, y2, make_float2(0.f, 0.f));
+      const float2 S = q[k];
       const float2 s0 = s_at(row), d0 = d_at(row), u = add2(s0, d0), vh = vh_at(jc), vd = vd_at(jc);
       float2 d1 = make_float2(fmaf(vd.x, u.x, fmaf(-vd.y, u.y, fmaf(vh.x, S.x, -vh.y * S.y))),
                               fmaf(vd.x, u.y, fmaf(vd.y, u.x, fmaf(vh.x, S.y, vh.y * S.x))));
@@ -236,9 +249,9 @@ __device__ __forceinline__ void rotor_close(const SpeciesDev& sp, const MolDev& 
   }
 }
 
-// The fused step: one CTA of N_r threads a molecule.
+// The fused step: one CTA of N_r threads a molecule (at J = 3 a fourth CTA an SM is worth 4%).
 template <int J, int NR, bool DIPR>
-__global__ void __launch_bounds__(NR, 3) mol_rotor_fused_kernel(SpeciesDev sp, MolDev md, int* err) {
+__global__ void __launch_bounds__(NR, J <= 3 ? 4 : 3) mol_rotor_fused_kernel(SpeciesDev sp, MolDev md, int* err) {
   constexpr int NROT = RotorDims<J>::NROT, NW = NR / 32;
   constexpr unsigned kStateBytes = (unsigned)NROT * NR * sizeof(float2);
   extern __shared__ __align__(16) float4 smem4[];
@@ -299,9 +312,13 @@ __global__ void __launch_bounds__(NR, 3) mol_rotor_fused_kernel(SpeciesDev sp, M
 // that the closing sums (a third of the instructions at J = 1) are paid twice a
 // molecule and not once for every 32 points.  Per row and point, against a warp
 // for every 32 points: J = 4, N_r = 256 6.56 -> 4.68 ps, J = 1, N_r = 64 7.91 ->
-// 6.76 ps; one warp a molecule: 5.13 against 4.42 ps at J = 4, N_r = 64.
+// 6.76 ps; one warp a molecule: 5.13 against 4.42 ps at J = 4, N_r = 64.  The
+// blocks asked for an SM set the registers a thread may take, and the order of
+// loads that follows from that: at J = 4 five (of which six fit) 4.36, 4.37 and
+// 4.15 ps at N_r = 64, 128 and 256, asking for six 4.43, 5.44 and 5.18; at J = 3
+// seven 4.45, 4.73 and 4.38 ps, six 4.89, 5.32 and 4.88.
 template <int J, int NR, bool DIPR>
-__global__ void __launch_bounds__(64, 6) mol_rotor_kernel(SpeciesDev sp, MolDev md, int* err) {
+__global__ void __launch_bounds__(64, J == 4 ? 5 : (J == 3 ? 7 : 6)) mol_rotor_kernel(SpeciesDev sp, MolDev md, int* err) {
   constexpr int NROT = RotorDims<J>::NROT;
   __shared__ float s_red[2][10], s_fin[10];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
