@@ -234,6 +234,8 @@ __device__ __forceinline__ float4 field_record(const SpeciesDev& sp, const MolDe
   if (!isfinite(x)) atomicOr(err, kErrNonFinite);  // a non-finite local field
   const int nt = coupling_terms(x);
   if (nt >= 24 || x > 4.f) atomicOr(err, kErrCouplingSeries);
+  // no field, or one that is not a number: no terms, and factors of zero for the kernels that always take one
+  if (nt == 0) return make_float4(0.f, 0.f, 0.f, __int_as_float(0));
   return make_float4(th * Ep[2], 0.5f * th * Ep[0], 0.5f * th * Ep[1], __int_as_float(nt));
 }
 
