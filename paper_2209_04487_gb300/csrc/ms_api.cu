@@ -1277,8 +1277,7 @@ static void end_steps(ms_sim* s, int begin, bool captured) {
 // of detector samples.
 static int cycle_steps(const ms_sim* s) {
   const int least = s->g.ndet > 0 ? ms::kDftBatch : 8;
-  const int L = s->nsub * std::max(1, (least + s->nsub - 1) / s->nsub);
-  return L % 2 ? 2 * L : L;  // even: a cycle ends on the counter slot it began with
+  return s->nsub * std::max(1, (least + s->nsub - 1) / s->nsub);
 }
 
 // Capture the launches of s->gsteps steps from phase 0 into a graph.  The
@@ -1291,6 +1290,7 @@ static ms_status capture_cycle(ms_sim* s) {
   s->gslot = s->slot;
   if (cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return MS_ECUDA;
   for (int q = 0; q < s->gsteps; ++q) step_once(s, nullptr, q == s->gsteps - 1);
+  keep_slot(s, s->gslot);  // an odd cycle: the next one starts where this one did
   s->steps = saved;
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(s->stream, &g);

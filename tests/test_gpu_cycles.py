@@ -1,0 +1,61 @@
+"""Which calls replay a captured cycle, and that the replays are the steps."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2209_04487_gb300 import build
+    build.build()
+    from paper_2209_04487_gb300 import binding
+    _graph_launches(lambda: torch.zeros(1, device="cuda"))  # the profiler's first session may miss calls
+    return binding
+
+
+def _graph_launches(fn):
+    """cudaGraphLaunch calls that fn makes, or None where the profiler records no runtime calls."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as p:
+        fn()
+        torch.cuda.synchronize()
+    names = [e.name for e in p.events()]
+    return names.count("cudaGraphLaunch") if any(n.startswith("cuda") for n in names) else None
+
+
+def _run(B, substeps, calls, graphs, planes=None):
+    wl = W.custom("cycles", 20, 12, 48, src_k=14, pulses=[[1e10, 1.5, 1e-15, 2e-16]], layer=(20, 24), n_per_sim=20,
+                  species=[W.species_config0(jmax=1)], seed=3, nsteps=200, mol_substeps=substeps)
+    sim = B.Simulation(wl, step_graphs=graphs)
+    if planes:
+        sim.set_detectors(planes, np.linspace(1.0, 3.0, 5) / 6.582119569e-16)
+    launches = []
+    for n in calls:
+        launches.append(_graph_launches(lambda: sim.step(n)))
+    out = [sim.populations(), sim.dipoles(), sim.fields(B.MS_FIELD_E), sim.fields(B.MS_FIELD_H)]
+    if planes:
+        out += [sim.dft(p, 0, c, f) for p in range(len(planes)) for c in range(4) for f in range(5)]
+    sim.close()
+    return launches, out
+
+
+@pytest.mark.parametrize("substeps,calls,want", [
+    (1, (7, 8, 17), (0, 1, 2)), (3, (9, 17, 1, 20), (1, 1, 0, 2)), (9, (9, 9, 4, 23), (1, 1, 0, 2)),
+    (11, (11, 22, 5, 17), (1, 2, 0, 1)), (40, (39, 1, 40, 80), (0, 0, 1, 2))])
+def test_whole_cycles_replay(B, substeps, calls, want):
+    """A cycle is the least number of whole molecular cycles with 8 field steps, odd ones too: every call that holds
+    one from the start of a molecular cycle on replays it."""
+    launches, got = _run(B, substeps, calls, B.MS_GRAPHS_AUTO)
+    _, ref = _run(B, substeps, calls, B.MS_GRAPHS_OFF)
+    for a, b in zip(got, ref):
+        assert np.array_equal(a, b)
+    if None in launches:
+        pytest.skip("the profiler records no runtime calls")
+    assert tuple(launches) == want
