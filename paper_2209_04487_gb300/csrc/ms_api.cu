@@ -1193,9 +1193,17 @@ static int pipelined_molecules(ms_sim* s, const ms::SpeciesDev* sp, int prescrib
   return launched;
 }
 
-// `last`: the last step of a call (or of a captured cycle), after which every
-// kept detector sample is added.
-static void step_once(ms_sim* s, float2* const* scratch, bool last, const FieldRecorder* rec = nullptr) {
+// Adds the kept detector samples; `done`: the counter slot that holds the step after the last of them.
+static int add_kept(ms_sim* s, const long long* done) {
+  if (s->dft_kept == 0) return 0;
+  ms::launch_dft_add(s->g, s->dft_kept, done, s->stream);
+  s->dft_kept = 0;
+  return 1;
+}
+
+// `left`: steps that the call (or a captured cycle that adds what it keeps) has left, this one included; after the
+// last every kept detector sample is added.
+static void step_once(ms_sim* s, float2* const* scratch, int64_t left, const FieldRecorder* rec = nullptr) {
   const bool fdtd = s->drive == MS_DRIVE_FDTD;
   // sub-stepping: the molecules advance (by nsub dt) on every nsub-th step only,
   // and only those steps' E updates take the molecular dipole change
@@ -1237,12 +1245,12 @@ static void step_once(ms_sim* s, float2* const* scratch, bool last, const FieldR
     ms::launch_yee_e(ge, s->stream);  // with the incident lines' E half step
     ++launched;
     if (s->g.ndet > 0) {
-      ms::launch_dft_keep(s->g, s->dft_kept++, s->stream);
       ++launched;
-      if (s->dft_kept == ms::kDftBatch || last) {
-        ms::launch_dft_add(s->g, s->dft_kept, s->stream);
-        s->dft_kept = 0;
-        ++launched;
+      if (s->dft_kept == 0 && left <= ms::kDftDirect) {
+        ms::launch_dft(s->g, s->stream);
+      } else {
+        ms::launch_dft_keep(s->g, s->stream);
+        if (++s->dft_kept == ms::kDftBatch || left == 1) launched += add_kept(s, s->g.step_next);
       }
     }
   }
@@ -1273,15 +1281,13 @@ static void end_steps(ms_sim* s, int begin, bool captured) {
   if (s->home >= 0) keep_slot(s, s->home);
 }
 
-// Steps of a captured cycle: whole molecular cycles, at least 8 steps, or a batch
-// of detector samples.
-static int cycle_steps(const ms_sim* s) {
-  const int least = s->g.ndet > 0 ? ms::kDftBatch : 8;
-  return s->nsub * std::max(1, (least + s->nsub - 1) / s->nsub);
-}
+// Steps of a captured cycle: whole molecular cycles, at least 8 steps.
+static int cycle_steps(const ms_sim* s) { return s->nsub * std::max(1, (8 + s->nsub - 1) / s->nsub); }
 
 // Capture the launches of s->gsteps steps from phase 0 into a graph.  The
-// host step count is restored: capturing runs nothing.
+// host step count is restored: capturing runs nothing.  A cycle shorter than a
+// batch of detector samples only keeps them (the batch is added between
+// cycles), a longer one adds all that it keeps.
 static ms_status capture_cycle(ms_sim* s) {
   if (s->gexec) cudaGraphExecDestroy(s->gexec);
   s->gexec = nullptr;
@@ -1289,7 +1295,8 @@ static ms_status capture_cycle(ms_sim* s) {
   const int64_t saved = s->steps;
   s->gslot = s->slot;
   if (cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return MS_ECUDA;
-  for (int q = 0; q < s->gsteps; ++q) step_once(s, nullptr, q == s->gsteps - 1);
+  for (int q = 0; q < s->gsteps; ++q) step_once(s, nullptr, s->gsteps < ms::kDftBatch ? ms::kDftBatch : s->gsteps - q);
+  s->dft_kept = 0;
   keep_slot(s, s->gslot);  // an odd cycle: the next one starts where this one did
   s->steps = saved;
   cudaGraph_t g = nullptr;
@@ -1317,20 +1324,22 @@ ms_status ms_step(ms_sim* s, int64_t n) {
   const int slot0 = s->slot;
   if (s->graphs && !s->timing && cs == cudaStreamCaptureStatusNone) {
     const int L = cycle_steps(s);
-    while (n > 0 && s->steps % s->nsub != 0) {  // to the start of a molecular cycle
-      step_once(s, nullptr, n == 1 || (s->steps + 1) % s->nsub == 0);
-      --n;
-    }
+    for (; n > 0 && s->steps % s->nsub != 0; --n) step_once(s, nullptr, n);  // to the start of a molecular cycle
     if (n >= L) {
+      add_kept(s, s->d_step + s->slot);
       if (!s->gexec || s->gdirty || s->gsteps != L) MS_TRY(capture_cycle(s));
       keep_slot(s, s->gslot);  // the captured cycle starts from this one
+      const int keeps = s->g.ndet > 0 && L < ms::kDftBatch ? L : 0;
       for (; n >= L; n -= L) {
+        if (s->dft_kept + keeps > ms::kDftBatch) add_kept(s, s->d_step + s->slot);
         if (cudaGraphLaunch(s->gexec, s->stream) != cudaSuccess) return MS_ECUDA;
         s->steps += L;
+        s->dft_kept += keeps;
       }
+      if (n == 0 || s->dft_kept == ms::kDftBatch) add_kept(s, s->d_step + s->slot);
     }
   }
-  for (int64_t q = 0; q < n; ++q) step_once(s, nullptr, q == n - 1);
+  for (; n > 0; --n) step_once(s, nullptr, n);
   end_steps(s, slot0, cs != cudaStreamCaptureStatusNone);
   return cudaGetLastError() == cudaSuccess ? MS_OK : MS_ECUDA;
 }
@@ -1354,7 +1363,7 @@ ms_status ms_step_noalloc(ms_sim* s, int64_t n) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess) return MS_ECUDA;
   const int slot0 = s->slot;
-  for (int64_t q = 0; q < n; ++q) step_once(s, scratch, q == n - 1);
+  for (; n > 0; --n) step_once(s, scratch, n);
   end_steps(s, slot0, cs != cudaStreamCaptureStatusNone);
   return cudaGetLastError() == cudaSuccess ? MS_OK : MS_ECUDA;
 }
@@ -1571,7 +1580,7 @@ ms_status ms_record_local_fields(ms_sim* s, const int64_t* mol_ids, int64_t m, f
   if (st == MS_OK) {
     FieldRecorder rec{static_cast<const long long*>(d_ids), (int)m, static_cast<float*>(d_out)};
     for (int64_t q = 0; q < nsteps; ++q) {
-      step_once(s, nullptr, q == nsteps - 1, &rec);
+      step_once(s, nullptr, nsteps - q, &rec);
       rec.out += (size_t)m * 3;
     }
     end_steps(s, s->slot, false);
@@ -1602,7 +1611,6 @@ ms_status ms_set_detectors(ms_sim* s, const int32_t* planes_z, int32_t nplanes, 
   double* dw = nullptr;
   double2* acc = nullptr;
   float* ring = nullptr;
-  long long* ring_n = nullptr;
   double* flux = nullptr;
   std::vector<int> k(planes_z, planes_z + nplanes);
   std::vector<double> w(omega, omega + nfreq);
@@ -1610,13 +1618,11 @@ ms_status ms_set_detectors(ms_sim* s, const int32_t* planes_z, int32_t nplanes, 
   MS_TRY(upload(s, &dw, w.data(), w.size()));
   MS_TRY(zeros(s, &acc, (size_t)s->g.nsim * nplanes * nfreq * 4 * s->g.nx * s->g.ny));
   MS_TRY(zeros(s, &ring, (size_t)ms::kDftBatch * s->g.nsim * nplanes * 6 * s->g.nx * s->g.ny));
-  MS_TRY(zeros(s, &ring_n, ms::kDftBatch));
   MS_TRY(zeros(s, &flux, (size_t)s->g.nsim * nfreq));
   s->g.det_k = dk;
   s->g.omega = dw;
   s->g.dft = acc;
   s->g.dft_ring = ring;
-  s->g.dft_n = ring_n;
   s->flux = flux;
   s->g.ndet = nplanes;
   s->g.nfreq = nfreq;

@@ -13,7 +13,8 @@ constexpr int kMaxSpecies = 8;
 constexpr int kMaxJ = 16;
 constexpr int kMaxRot = (kMaxJ + 1) * (kMaxJ + 1);  // 289 channels per surface
 constexpr int kMaxCoupl = 6;                          // nonzeros of R^hat per row
-constexpr int kDftBatch = 16;                         // steps whose detector samples one launch adds up
+constexpr int kDftBatch = 16;                         // steps whose detector samples one launch adds up (a power of two)
+constexpr int kDftDirect = 3;                         // up to so many last steps of a call are added one by one
 
 // error bits latched in the device error word
 enum : int {
@@ -100,9 +101,8 @@ struct Grid {
   const double* omega;   // [nfreq] angular frequencies (rad/s)
   double2* dft;          // [nsim][ndet][nfreq][4][ny][nx]: Ex, Ey on plane k at t_{n+1};
                          // Hx, Hy averaged over z = k -+ 1/2 at t_{n+1/2}
-  float* dft_ring;       // samples of the steps not yet added: [kDftBatch][nsim][ndet][6][ny][nx],
-                         // Ex, Ey, Hx below and above, Hy below and above
-  long long* dft_n;      // [kDftBatch]: their step indices
+  float* dft_ring;       // samples of the steps not yet added, step n's in slot n % kDftBatch:
+                         // [kDftBatch][nsim][ndet][6][ny][nx], Ex, Ey, Hx below and above, Hy below and above
 };
 
 // One species' device tables (all built on the host in FP64).
@@ -259,9 +259,10 @@ bool mol_mixed_supported(int nr);
 int mixed_strip_rows(int nr);
 int mixed_plane_offset(int row, int k, int nr);
 void launch_step_counter(const long long* from, long long* to, int add, cudaStream_t s);
-// spectral detection: keep this step's samples in slot `slot`; add the first `count` kept steps
-void launch_dft_keep(const Grid& g, int slot, cudaStream_t s);
-void launch_dft_add(const Grid& g, int count, cudaStream_t s);
+// spectral detection: add this step's samples; keep them; add those of the `count` steps before step *done
+void launch_dft(const Grid& g, cudaStream_t s);
+void launch_dft_keep(const Grid& g, cudaStream_t s);
+void launch_dft_add(const Grid& g, int count, const long long* done, cudaStream_t s);
 // Poynting flux spectra of one plane: out[nsim][nfreq]
 void launch_flux(const Grid& g, int plane, double dx2, double* out, cudaStream_t s);
 // E^n at the cells of the listed molecules: out[k][3] for k < m

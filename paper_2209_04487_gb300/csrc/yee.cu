@@ -594,12 +594,51 @@ void launch_record_fields(const Grid& g, const int* cell, const long long* ids, 
 // planes of 128 x 128 cells, 48 frequencies: 201 MB); the FP64 products alone
 // need 22 us (two a clock and SM).  So a step only keeps its samples, and one
 // launch adds up to kDftBatch kept steps, in their order: every accumulator is
-// read and written once a batch and takes the same sums as step by step.
-__global__ void dft_keep_kernel(Grid g, int slot) {
+// read and written once a batch and takes the same sums as step by step.  Where a
+// call has kDftDirect steps or fewer left, each is added straight from the
+// fields: calls of 1, 2 and 3 steps of that workload, half steps included, take
+// 90, 180 and 270 us so and 153, 226 and 287 with kept samples (a step more: 90 and
+// 63).
+constexpr int kDftF = 8;  // frequencies a block
+
+// One step: a block covers 256 cells of one plane and kDftF frequencies.
+__global__ void dft_kernel(Grid g, int nfc) {
+  __shared__ double2 ph[2][kDftF];  // dt e^{i omega t} at the E and at the H times
+  const long long n = *g.step;
+  const int d = blockIdx.y / nfc, f0 = (blockIdx.y % nfc) * kDftF, sim = blockIdx.z;
+  const int nf = min(kDftF, g.nfreq - f0);
+  if (threadIdx.x < 2 * nf) {
+    const int f = threadIdx.x % nf, h = threadIdx.x / nf;
+    double sn, cs;
+    sincos(g.omega[f0 + f] * (h ? (double)n + 0.5 : (double)(n + 1)) * g.dt, &sn, &cs);
+    ph[h][f] = make_double2(cs * g.dt, sn * g.dt);
+  }
+  __syncthreads();
+  const long long plane = (long long)g.ny * g.nx;
+  const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (q >= plane) return;
+  const long long ck = sim * g.ncell_sim + (long long)g.det_k[d] * plane + q, cm = ck - plane;
+  const double v[4] = {g.E[0][ck], g.E[1][ck], 0.5 * ((double)g.H[0][cm] + (double)g.H[0][ck]),
+                       0.5 * ((double)g.H[1][cm] + (double)g.H[1][ck])};
+  double2* acc = g.dft + (((long long)sim * g.ndet + d) * g.nfreq + f0) * 4 * plane + q;
+  for (int f = 0; f < nf; ++f) {  // four independent sums at a time
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const double2 w = ph[c < 2 ? 0 : 1][f];
+      double2* a = acc + ((long long)f * 4 + c) * plane;
+      double2 x = *a;
+      x.x = fma(v[c], w.x, x.x);
+      x.y = fma(v[c], w.y, x.y);
+      *a = x;
+    }
+  }
+}
+
+__global__ void dft_keep_kernel(Grid g) {
   const long long plane = (long long)g.ny * g.nx, q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (q == 0 && blockIdx.y == 0 && blockIdx.z == 0) g.dft_n[slot] = *g.step;
   if (q >= plane) return;
   const long long ck = blockIdx.z * g.ncell_sim + (long long)g.det_k[blockIdx.y] * plane + q, cm = ck - plane;
+  const int slot = (int)(*g.step & (kDftBatch - 1));
   float* o = g.dft_ring + (((long long)slot * g.nsim + blockIdx.z) * g.ndet + blockIdx.y) * 6 * plane + q;
   o[0] = g.E[0][ck];
   o[plane] = g.E[1][ck];
@@ -609,16 +648,15 @@ __global__ void dft_keep_kernel(Grid g, int slot) {
   o[5 * plane] = g.H[1][ck];
 }
 
-constexpr int kDftF = 8;  // frequencies a block
-
-// A block: 256 cells of one plane, kDftF frequencies, every component, `count` kept steps.
-__global__ void __launch_bounds__(256) dft_add_kernel(Grid g, int nfc, int count) {
+// A block: 256 cells of one plane, kDftF frequencies, every component, the `count` steps before step *done.
+__global__ void __launch_bounds__(256) dft_add_kernel(Grid g, int nfc, int count, const long long* done) {
   __shared__ double2 ph[2][kDftF][kDftBatch];  // dt e^{i omega t} at the E and at the H times
+  const long long n0 = *done - count;
   const int d = blockIdx.y / nfc, f0 = (blockIdx.y % nfc) * kDftF, sim = blockIdx.z;
   const int nf = min(kDftF, g.nfreq - f0);
   for (int q = threadIdx.x; q < 2 * nf * count; q += blockDim.x) {
     const int b = q % count, f = (q / count) % nf, h = q / (count * nf);
-    const long long n = g.dft_n[b];
+    const long long n = n0 + b;
     double sn, cs;
     sincos(g.omega[f0 + f] * (h ? (double)n + 0.5 : (double)(n + 1)) * g.dt, &sn, &cs);
     ph[h][f][b] = make_double2(cs * g.dt, sn * g.dt);
@@ -636,9 +674,10 @@ __global__ void __launch_bounds__(256) dft_add_kernel(Grid g, int nfc, int count
 #pragma unroll
     for (int b = 0; b < kDftBatch; ++b) {
       v[b] = 0.0;
-      if (b < count)
-        v[b] = c < 2 ? (double)ring[b * slot + c * plane]
-                     : 0.5 * ((double)ring[b * slot + (2 * c - 2) * plane] + (double)ring[b * slot + (2 * c - 1) * plane]);
+      if (b < count) {
+        const float* r = ring + ((n0 + b) & (kDftBatch - 1)) * slot;
+        v[b] = c < 2 ? (double)r[c * plane] : 0.5 * ((double)r[(2 * c - 2) * plane] + (double)r[(2 * c - 1) * plane]);
+      }
     }
 #pragma unroll 1
     for (int f = 0; f < nf; f += 2) {  // two frequencies at a time: four independent chains
@@ -689,15 +728,18 @@ __global__ void __launch_bounds__(512) flux_kernel(Grid g, int plane, double dx2
 void launch_flux(const Grid& g, int plane, double dx2, double* out, cudaStream_t s) {
   flux_kernel<<<dim3((unsigned)g.nfreq, (unsigned)g.nsim), 512, 0, s>>>(g, plane, dx2, out);
 }
-void launch_dft_keep(const Grid& g, int slot, cudaStream_t s) {
+static dim3 dft_grid(const Grid& g, int nfc) {
   const long long plane = (long long)g.ny * g.nx;
-  dft_keep_kernel<<<dim3((unsigned)((plane + 255) / 256), (unsigned)g.ndet, (unsigned)g.nsim), 256, 0, s>>>(g, slot);
+  return dim3((unsigned)((plane + 255) / 256), (unsigned)(g.ndet * nfc), (unsigned)g.nsim);
 }
-void launch_dft_add(const Grid& g, int count, cudaStream_t s) {
-  const long long plane = (long long)g.ny * g.nx;
+void launch_dft(const Grid& g, cudaStream_t s) {
   const int nfc = (g.nfreq + kDftF - 1) / kDftF;
-  const dim3 grid((unsigned)((plane + 255) / 256), (unsigned)(g.ndet * nfc), (unsigned)g.nsim);
-  dft_add_kernel<<<grid, 256, 0, s>>>(g, nfc, count);
+  dft_kernel<<<dft_grid(g, nfc), 256, 0, s>>>(g, nfc);
+}
+void launch_dft_keep(const Grid& g, cudaStream_t s) { dft_keep_kernel<<<dft_grid(g, 1), 256, 0, s>>>(g); }
+void launch_dft_add(const Grid& g, int count, const long long* done, cudaStream_t s) {
+  const int nfc = (g.nfreq + kDftF - 1) / kDftF;
+  dft_add_kernel<<<dft_grid(g, nfc), 256, 0, s>>>(g, nfc, count, done);
 }
 void launch_step_counter(const long long* from, long long* to, int add, cudaStream_t s) {
   step_counter_kernel<<<1, 1, 0, s>>>(from, to, add);

@@ -38,7 +38,10 @@ def _run(B, substeps, calls, graphs, planes=None):
         sim.set_detectors(planes, np.linspace(1.0, 3.0, 5) / 6.582119569e-16)
     launches = []
     for n in calls:
-        launches.append(_graph_launches(lambda: sim.step(n)))
+        if graphs == B.MS_GRAPHS_OFF:
+            sim.step(n)
+        else:
+            launches.append(_graph_launches(lambda: sim.step(n)))
     out = [sim.populations(), sim.dipoles(), sim.fields(B.MS_FIELD_E), sim.fields(B.MS_FIELD_H)]
     if planes:
         out += [sim.dft(p, 0, c, f) for p in range(len(planes)) for c in range(4) for f in range(5)]
@@ -59,3 +62,30 @@ def test_whole_cycles_replay(B, substeps, calls, want):
     if None in launches:
         pytest.skip("the profiler records no runtime calls")
     assert tuple(launches) == want
+
+
+@pytest.mark.parametrize("substeps,calls,want", [
+    (1, (7, 8, 15, 16, 17, 1, 40, 25), (0, 1, 1, 2, 2, 0, 5, 3)), (3, (9, 17, 1, 20, 31), (1, 1, 0, 2, 3)),
+    (20, (20, 5, 55, 40), (1, 0, 2, 2))])
+def test_cycles_with_detectors(B, substeps, calls, want):
+    """Detectors leave the cycle's length as it is, and the accumulators are those of single steps: cycles shorter
+    than a batch of kept samples, longer ones, and steps before, between and after them."""
+    launches, got = _run(B, substeps, calls, B.MS_GRAPHS_AUTO, planes=[12, 40])
+    _, ref = _run(B, substeps, (1,) * sum(calls), B.MS_GRAPHS_OFF, planes=[12, 40])
+    for a, b in zip(got, ref):
+        assert np.array_equal(a, b)
+    if None in launches:
+        pytest.skip("the profiler records no runtime calls")
+    assert tuple(launches) == want
+
+
+def test_short_calls_keep_no_samples(B):
+    """Calls of up to three steps add their samples from the fields: two half steps and one launch a step."""
+    wl = W.custom("single", 20, 18, 48, src_k=14, pulses=[[1e9, 1.5, 1e-15, 1e-16]], n_per_sim=0, nsteps=10)
+    sim = B.Simulation(wl)
+    sim.set_detectors([12, 40], np.array([2.0, 3.0]) / 6.582119569e-16)
+    for n, most in ((1, 3), (2, 6), (3, 9), (4, 13)):
+        sim.timing_begin()
+        sim.step(n)
+        assert sim.timing_end()[2] <= most
+    sim.close()
