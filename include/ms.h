@@ -378,8 +378,10 @@ ms_status ms_record_local_fields(ms_sim* sim, const int64_t* mol_ids, int64_t m,
  *   - omega: nfreq (1..512) angular frequencies in rad/s.
  * A call replaces the detectors set before and zeroes the accumulators;
  * each call allocates their device memory (nsim * nplanes * nfreq * 4 * nx
- * * ny * 16 bytes, and 384 bytes a cell of every plane for the samples of the
- * steps of a call that are added together, at most 16) until ms_destroy.  FDTD-driven handles only.  Errors:
+ * * ny * 16 bytes, and where it can be had 384 bytes a cell of every plane
+ * for the samples of the steps of a call that are added together, at most
+ * 16; without them every step is added by itself, with the same results)
+ * until ms_destroy.  FDTD-driven handles only.  Errors:
  * MS_EINVAL, MS_ENOMEM. */
 ms_status ms_set_detectors(ms_sim* sim, const int32_t* planes_z, int32_t nplanes, const double* omega,
                            int32_t nfreq);

@@ -1246,7 +1246,7 @@ static void step_once(ms_sim* s, float2* const* scratch, int64_t left, const Fie
     ++launched;
     if (s->g.ndet > 0) {
       ++launched;
-      if (s->dft_kept == 0 && left <= ms::kDftDirect) {
+      if (!s->g.dft_ring || (s->dft_kept == 0 && left <= ms::kDftDirect)) {
         ms::launch_dft(s->g, s->stream);
       } else {
         ms::launch_dft_keep(s->g, s->stream);
@@ -1329,7 +1329,7 @@ ms_status ms_step(ms_sim* s, int64_t n) {
       add_kept(s, s->d_step + s->slot);
       if (!s->gexec || s->gdirty || s->gsteps != L) MS_TRY(capture_cycle(s));
       keep_slot(s, s->gslot);  // the captured cycle starts from this one
-      const int keeps = s->g.ndet > 0 && L < ms::kDftBatch ? L : 0;
+      const int keeps = s->g.ndet > 0 && s->g.dft_ring && L < ms::kDftBatch ? L : 0;
       for (; n >= L; n -= L) {
         if (s->dft_kept + keeps > ms::kDftBatch) add_kept(s, s->d_step + s->slot);
         if (cudaGraphLaunch(s->gexec, s->stream) != cudaSuccess) return MS_ECUDA;
@@ -1617,8 +1617,10 @@ ms_status ms_set_detectors(ms_sim* s, const int32_t* planes_z, int32_t nplanes, 
   MS_TRY(upload(s, &dk, k.data(), k.size()));
   MS_TRY(upload(s, &dw, w.data(), w.size()));
   MS_TRY(zeros(s, &acc, (size_t)s->g.nsim * nplanes * nfreq * 4 * s->g.nx * s->g.ny));
-  MS_TRY(zeros(s, &ring, (size_t)ms::kDftBatch * s->g.nsim * nplanes * 6 * s->g.nx * s->g.ny));
   MS_TRY(zeros(s, &flux, (size_t)s->g.nsim * nfreq));
+  // where no memory is left for kept samples every step is added from the fields
+  const ms_status rs = zeros(s, &ring, (size_t)ms::kDftBatch * s->g.nsim * nplanes * 6 * s->g.nx * s->g.ny);
+  if (rs != MS_OK && rs != MS_ENOMEM) return rs;
   s->g.det_k = dk;
   s->g.omega = dw;
   s->g.dft = acc;

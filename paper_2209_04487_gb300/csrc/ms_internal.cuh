@@ -102,7 +102,8 @@ struct Grid {
   double2* dft;          // [nsim][ndet][nfreq][4][ny][nx]: Ex, Ey on plane k at t_{n+1};
                          // Hx, Hy averaged over z = k -+ 1/2 at t_{n+1/2}
   float* dft_ring;       // samples of the steps not yet added, step n's in slot n % kDftBatch:
-                         // [kDftBatch][nsim][ndet][6][ny][nx], Ex, Ey, Hx below and above, Hy below and above
+                         // [kDftBatch][nsim][ndet][6][ny][nx], Ex, Ey, Hx below and above, Hy below and above;
+                         // null: none are kept
 };
 
 // One species' device tables (all built on the host in FP64).

@@ -89,3 +89,36 @@ def test_short_calls_keep_no_samples(B):
         sim.step(n)
         assert sim.timing_end()[2] <= most
     sim.close()
+
+
+class _NoBlocksOf:
+    """An allocator that refuses blocks of one size."""
+
+    def __init__(self, B, size):
+        inner = B._TorchAllocator()
+        self.inner, self.refused = inner, 0
+
+        def alloc(n, ctx):
+            if n == size:
+                self.refused += 1
+                return None
+            return inner._alloc(n, ctx)
+        self.c_alloc, self.c_free = B._ALLOC(alloc), B._FREE(inner._free)
+
+
+def test_detectors_without_memory_for_kept_samples(B):
+    """Detectors are set where only the kept samples find no memory, with the same accumulators."""
+    nx, ny, planes, om = 20, 18, [12, 40], np.linspace(1.0, 3.0, 2) / 6.582119569e-16
+    wl = W.custom("no ring", nx, ny, 48, src_k=14, pulses=[[1e9, 1.5, 1e-15, 1e-16]], n_per_sim=0, nsteps=100)
+    got = []
+    for al in (None, _NoBlocksOf(B, 384 * len(planes) * nx * ny)):
+        sim = B.Simulation(wl, allocator=al) if al else B.Simulation(wl)
+        sim.set_detectors(planes, om)
+        for n in (1, 5, 24, 13):
+            sim.step(n)
+        got.append([sim.dft(p, 0, c, f) for p in range(2) for c in range(4) for f in range(2)])
+        sim.close()
+    assert al.refused == 1
+    assert max(np.abs(a).max() for a in got[0]) > 0
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
