@@ -266,9 +266,8 @@ ms_status ms_create(const ms_grid_desc* grid, const ms_materials_desc* materials
  * captured on first use (and again after ms_set_prescribed_field,
  * ms_set_replay_field or ms_set_detectors change what the kernels read).
  * Steps that the caller captures into a graph of its own replay from whatever
- * step the handle has reached, also between other calls; capture them again
- * after ms_set_species_plan, or after ms_load of a state that populates rows
- * the j = 0 start cannot reach: both can change the order of the stored rows. */
+ * step the handle has reached, also between other calls, after ms_load of any
+ * state and after ms_set_species_plan (with the plans of the capture). */
 ms_status ms_step(ms_sim* sim, int64_t n);
 
 /* Allocation-free stepping.  The paper has no counterpart: this is a library

@@ -118,6 +118,7 @@ constexpr int kChunk = 32;            // widest R-space chunk (one radial point 
 template <int NR, bool FUSED, int MAXR>
 __global__ void __launch_bounds__(FFTShape<NR>::THREADS, FUSED ? 2 : (MAXR <= 4 ? 4 : (MAXR <= 12 ? 2 : 1)))
     mol_step_kernel(SpeciesDev sp, MolDev md, Grid g, int prescribed, int CH, int* err) {
+  if (idle_launch(sp)) return;
   // CH radial points per chunk (32 down to 4): a warp covers 32/CH rows of CH points
   constexpr int NT = FFTShape<NR>::THREADS, NRP = NR + kPad, NW = NT / 32;
   extern __shared__ float4 smem4[];
@@ -472,6 +473,7 @@ constexpr int ch_of(int j, int m, int J) { return (j < 0 || j > J || m < -j || m
 // record waits for three dependent loads, and its CTA with it: 9.99 against 9.30
 // ms for eight steps of 50,000 molecules).
 __global__ void mol_field_kernel(SpeciesDev sp, MolDev md, Grid g, int prescribed, int* err) {
+  if (idle_launch(sp)) return;
   const int lm = blockIdx.x * blockDim.x + threadIdx.x;
   if (lm < sp.nmol) sp.fld[lm] = field_record(sp, md, g, prescribed, sp.mol[lm], err);
 }
@@ -598,6 +600,7 @@ __device__ __forceinline__ void dipole_rows(const V& gv, const W& ev, float2& ac
 template <int J, int NR, bool FUSED, bool DIPR = false>
 __global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? 2 : 1))
     mol_rpoint_kernel(SpeciesDev sp, MolDev md, int* err) {
+  if (idle_launch(sp)) return;
   using L = Rows<J, false>;
   constexpr int ROWS = L::ROWS, NG = L::NG, NT = 2 * NR, NW = NT / 32;
   constexpr int RMAX = L::NG > L::NE ? L::NG : L::NE;
@@ -863,6 +866,7 @@ static void launch_rpoint_n(const SpeciesDev& sp, const MolDev& md, int* err, cu
 // radial point each), then writes mu and the change over the step.
 template <int J, int NR, bool PAR>
 __global__ void __launch_bounds__(FFTShape<NR>::THREADS) mol_dipole_r_kernel(SpeciesDev sp, MolDev md, int* err) {
+  if (idle_launch(sp)) return;
   using L = Rows<J, PAR>;
   constexpr int ROWS = L::ROWS, NG = L::NG, NE = L::NE, NT = FFTShape<NR>::THREADS, NW = NT / 32;
   constexpr unsigned kStateBytes = (unsigned)ROWS * NR * sizeof(float2);
@@ -1118,6 +1122,7 @@ template <int NR>
 __global__ void __launch_bounds__(FFTShape<NR>::THREADS)
     mol_kinetic_kernel(SpeciesDev sp, MolDev md, Grid g, int prescribed, int nfld, long long rows_total, int RB,
                        int* err) {
+  if (idle_launch(sp)) return;
   if ((int)blockIdx.x < nfld) {
     const int lm = blockIdx.x * FFTShape<NR>::THREADS + threadIdx.x;
     if (lm < sp.nmol) sp.fld[lm] = field_record(sp, md, g, prescribed, sp.mol[lm], err);
@@ -1365,7 +1370,7 @@ bool mol_tensor_maps_available() { return tensor_map_encoder() != nullptr; }
 // (streaming), 2.70 and 1.16 ms with 50,000 at J = 4, N_r = 128 (fused).
 bool mol_reachable_rows(const SpeciesDev& sp) {
   if (sp.par_form) return true;
-  if (sp.all_rows) return false;
+  if (sp.all_rows || sp.keep_all) return false;
   return use_point(sp) ||
          (sp.path == MS_MOL_STREAMING && sp.kern == MS_KERN_DEFAULT && sp.jmax >= 5 &&
           (sp.jmax <= 8 || mol_tensor_maps_available()));
@@ -1379,6 +1384,20 @@ void mol_set_rows(SpeciesDev& sp, bool reachable) {
     sp.rows_g = 0;
     for (int j = 0; j <= sp.jmax; j += 2) sp.rows_g += 2 * j + 1;
   }
+}
+
+bool mol_both_orders(const SpeciesDev& sp, SpeciesDev v[2]) {
+  v[0] = v[1] = sp;
+  mol_set_rows(v[0], false);
+  v[1].all_rows = 0;
+  if (!mol_reachable_rows(v[1])) {  // a plan that names a kernel for every row: the rule's kernel for the reachable ones
+    v[1].kern = MS_KERN_DEFAULT;
+    v[1].ch = v[1].cps = 0;
+  }
+  if (!mol_reachable_rows(v[1])) return false;
+  mol_set_rows(v[1], true);
+  v[0].guard = v[1].guard = 1;
+  return true;
 }
 
 namespace {
@@ -1512,6 +1531,7 @@ struct TcShape {
 
 template <int NR>
 __global__ void __launch_bounds__(256, 1) mol_kinetic_tc_kernel(SpeciesDev sp, long long rows, int* err) {
+  if (idle_launch(sp)) return;
   using S = TcShape<NR>;
   constexpr int TR = S::TR, KS = S::KS, APL = S::APL, BPL = S::BPL, LOADS = S::LOADS;
   constexpr unsigned SBO_A = 2 * 128, SBO_B = (NR / 8) * 128;

@@ -225,6 +225,7 @@ template <int J>
 __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesDev sp, MolDev md, int* err) {
   using D = ColDims<J>;
   constexpr int NROT = D::NROT, NG = D::NG;
+  if (idle_launch(sp)) return;
   __shared__ float2 Ys[NROT][32];
   __shared__ int s_vt[NROT + 3];  // row -> its shell's row of the phase table (and three past the end)
   __shared__ float s_fin[8], s_fin_lo[2];  // P_g, P_e, Re(S+ + S-), Im(S+ - S-), 2 Re Z, absorbed (2), rounding residuals

@@ -121,6 +121,7 @@ __device__ __forceinline__ int shell_row(int jp) {
 template <int J, int TILE, bool PAR>
 __global__ void __launch_bounds__(Rs2Dims<J, TILE, PAR>::NT, Rs2Dims<J, TILE, PAR>::MINB)
     mol_rspace_pair_kernel(SpeciesDev sp, MolDev md, int* err, const __grid_constant__ RspaceMaps maps) {
+  if (idle_launch(sp)) return;
   using D = Rs2Dims<J, TILE, PAR>;
   constexpr int NROT = D::NGR, ROWS = D::ROWS, NV = D::NV, NW = D::NW, RPW = D::RPW, NT = D::NT;
   constexpr int RPL = D::RPL, SEG = D::SEG, SLOT = D::SLOT, TBB = D::TBB, G0 = kTriGuard * SEG;

@@ -255,6 +255,7 @@ template <int J, int NR, bool DIPR>
 __global__ void __launch_bounds__(NR, J <= 3 ? 4 : 3) mol_rotor_fused_kernel(SpeciesDev sp, MolDev md, int* err) {
   constexpr int NROT = RotorDims<J>::NROT, NW = NR / 32;
   constexpr unsigned kStateBytes = (unsigned)NROT * NR * sizeof(float2);
+  if (idle_launch(sp)) return;
   extern __shared__ __align__(16) float4 smem4[];
   float2* Sb = reinterpret_cast<float2*>(smem4);  // [NROT][NR] s
   float2* Db = Sb + NROT * NR;                    // [NROT][NR] d2
@@ -321,6 +322,7 @@ __global__ void __launch_bounds__(NR, J <= 3 ? 4 : 3) mol_rotor_fused_kernel(Spe
 template <int J, int NR, bool DIPR>
 __global__ void __launch_bounds__(64, J == 4 ? 5 : (J == 3 ? 7 : 6)) mol_rotor_kernel(SpeciesDev sp, MolDev md, int* err) {
   constexpr int NROT = RotorDims<J>::NROT;
+  if (idle_launch(sp)) return;
   __shared__ float s_red[2][10], s_fin[10];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int lm = blockIdx.x, m = sp.mol[lm];

@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(RsDims<J, TILE>::NT, RsDims<J, TILE>::MINB)
   constexpr int NROT = D::NROT, ROWS = D::ROWS, NV = D::NV, NW = D::NW, RPW = D::RPW, NT = D::NT;
   constexpr int RPL = D::RPL, SEG = D::SEG, TBB = D::TBB, G0 = kTriGuard * SEG;
   constexpr int SLOT = RPL * SEG;                 // bytes of one warp's rows in a tile buffer
+  if (idle_launch(sp)) return;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long s_bar[1];
   __shared__ float s_rot[9];

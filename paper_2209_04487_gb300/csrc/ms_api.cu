@@ -85,6 +85,8 @@ struct ms_sim {
   int slot = 0;                 // the one that holds the current step
   int gslot = 0;                // the one the captured cycle starts from
   int home = -1;                // the one every call ends on once the caller has captured steps; -1 before
+  bool caller = false;          // the steps being queued go into a graph of the caller's
+  int* d_order = nullptr;       // per species: the order of its rows (SpeciesDev::order)
   // device address of the library's fixed scratch array (ms_step_noalloc),
   // looked up at create with the handle's device current; null if that failed
   float2* noalloc_base = nullptr;
@@ -414,7 +416,13 @@ ms_status build_species(ms_sim* s, int si, const ms_species& d, double dt, const
     sp.theta = dmax * dtau;
     MS_TRY(upload(s, (float**)&sp.dipw, w.data(), w.size()));
   }
+  sp.keep_all = sp.guard = 0;
+  sp.order = nullptr;
   ms::mol_set_rows(sp, ms::mol_reachable_rows(sp));
+  if (!par) {
+    sp.order = s->d_order + si;
+    if (cudaMemsetAsync(sp.order, sp.par, 1, s->stream) != cudaSuccess) return MS_ECUDA;
+  }
   std::vector<double> r(nr), Ug(nr), Ue(nr);
   for (int i = 0; i < nr; ++i) {
     r[i] = d.rmin + i * dR;
@@ -535,16 +543,22 @@ ms_status ensure_scratch(ms_sim* s, ms::SpeciesDev& sp) {
   return zeros(s, &sp.d2, (size_t)sp.nmol * sp.mrows * sp.nr);
 }
 
-// Brings a full-form species' rows into the order that its plan's kernels
-// process (on the handle's stream).
+// Brings a full-form species' rows, which stand in the other order, into an order (on the handle's stream); the device
+// word that callers' graphs read follows.
+ms_status put_rows(ms_sim* s, ms::SpeciesDev& sp, bool reachable_first) {
+  if (ms::launch_order_rows(sp, reachable_first, s->stream) != cudaSuccess) return MS_ECUDA;
+  ms::mol_set_rows(sp, reachable_first);
+  if (sp.order && cudaMemsetAsync(sp.order, reachable_first, 1, s->stream) != cudaSuccess) return MS_ECUDA;
+  return MS_OK;
+}
+
+// Into the order that the species' plan processes.
 ms_status order_rows(ms_sim* s, ms::SpeciesDev& sp) {
   if (sp.bloch || sp.par_form) return MS_OK;
   const bool want = ms::mol_reachable_rows(sp);
   if (want == (sp.par != 0)) return MS_OK;
-  if (ms::launch_order_rows(sp, want, s->stream) != cudaSuccess) return MS_ECUDA;
-  ms::mol_set_rows(sp, want);
   s->gdirty = true;
-  return MS_OK;
+  return put_rows(s, sp, want);
 }
 
 // While it lives, every full-form species' rows are in channel order, the order
@@ -559,8 +573,7 @@ struct ChannelOrder {
       ms::SpeciesDev& sp = s->sp[si];
       par[si] = sp.par;
       if (sp.bloch || sp.par_form || !sp.par || st != MS_OK) continue;
-      if (ms::launch_order_rows(sp, false, s->stream) != cudaSuccess) st = MS_ECUDA;
-      else ms::mol_set_rows(sp, false);
+      st = put_rows(s, sp, false);
     }
   }
   ms_status end() {
@@ -612,6 +625,7 @@ ms_status tune_species(ms_sim* s, int si) {
   const size_t per = (size_t)sp.mrows * sp.nr;
   Scratch sc{s, {}};
   ms::SpeciesDev t = sp;
+  t.order = nullptr;
   ms::MolDev m = s->md;
   t.nmol = nt;
   t.psi = (float2*)sc.get(per * nt * sizeof(float2));
@@ -757,6 +771,7 @@ ms_status create_impl(const ms_grid_desc* G, const ms_materials_desc* M, const m
   MS_TRY(zeros(s, &s->d_step, 2));
   g.step = g.step_next = s->d_step;  // a step's launches take them from s->slot
   MS_TRY(zeros(s, &s->d_err, 1));
+  MS_TRY(zeros(s, &s->d_order, ms::kMaxSpecies));
   if (cudaMallocHost((void**)&s->h_read, kReadStage + 64) != cudaSuccess) {  // reads then go without
     cudaGetLastError();
     s->h_read = nullptr;
@@ -1162,10 +1177,10 @@ struct FieldRecorder {  // ms_record_local_fields: E^n of listed molecules, one 
 // the previous one; the handle's stream then waits for the last stage 2.
 // Every molecule gets the same kernels on the same data: results do not
 // depend on the batching.
-static int pipelined_molecules(ms_sim* s, const ms::SpeciesDev* sp, int prescribed) {
-  ms::SpeciesDev runs[ms::kMaxSpecies * kMaxMolBatches];
+static int pipelined_molecules(ms_sim* s, const ms::SpeciesDev* sp, int nsp, int prescribed) {
+  ms::SpeciesDev runs[2 * ms::kMaxSpecies * kMaxMolBatches];
   int nrun = 0;
-  for (int si = 0; si < s->nspecies; ++si) {
+  for (int si = 0; si < nsp; ++si) {
     const ms::SpeciesDev& a = sp[si];
     const int nb = a.path == MS_MOL_STREAMING && !a.bloch ? std::min(s->batches, std::max(a.nmol, 1)) : 1;
     const size_t per = (size_t)a.mrows * a.nr, per_d2 = (size_t)a.rows * a.nr;
@@ -1221,21 +1236,24 @@ static void step_once(ms_sim* s, float2* const* scratch, int64_t left, const Fie
     ++launched;
   }
   if (s->timing) mark(s);
-  ms::SpeciesDev sp[ms::kMaxSpecies];
+  ms::SpeciesDev sp[2 * ms::kMaxSpecies];
+  int nsp = 0;
   for (int si = 0; si < s->nspecies; ++si) {
-    sp[si] = s->sp[si];
-    if (scratch && sp[si].path == MS_MOL_STREAMING) sp[si].d2 = scratch[si];  // rewritten before it is read
+    ms::SpeciesDev a = s->sp[si];
+    if (scratch && a.path == MS_MOL_STREAMING) a.d2 = scratch[si];  // rewritten before it is read
+    if (s->caller && a.order && !a.keep_all && ms::mol_both_orders(a, sp + nsp)) nsp += 2;
+    else sp[nsp++] = a;
   }
   if (molecular && s->batches > 0) {
-    launched += pipelined_molecules(s, sp, fdtd ? 0 : 1);
+    launched += pipelined_molecules(s, sp, nsp, fdtd ? 0 : 1);
     if (s->timing) mark(s);  // stages overlap: only the molecular phase as a whole is timed
   } else {
     if (molecular)
-      for (int si = 0; si < s->nspecies; ++si)
+      for (int si = 0; si < nsp; ++si)
         launched += ms::launch_mol_stage1(sp[si], s->md, s->g, fdtd ? 0 : 1, s->d_err, s->stream);
     if (s->timing) mark(s);
     if (molecular)
-      for (int si = 0; si < s->nspecies; ++si)
+      for (int si = 0; si < nsp; ++si)
         launched += ms::launch_mol_stage2(sp[si], s->md, s->g, fdtd ? 0 : 1, s->d_err, s->stream);
   }
   if (s->timing) mark(s);
@@ -1276,7 +1294,16 @@ static void keep_slot(ms_sim* s, int slot) {
 // The end of a call's steps.  A call that the caller captures ends on the counter
 // slot it began with, and so does every call after it: the caller's graph can be
 // replayed, by itself and between other calls.
+static void begin_steps(ms_sim* s, bool captured) {
+  s->caller = captured;
+  if (!captured) return;
+  for (int si = 0; si < s->nspecies; ++si) {  // no kernel for the reachable rows in this layout: always every row
+    ms::SpeciesDev& sp = s->sp[si], v[2];
+    if (sp.order && !ms::mol_both_orders(sp, v)) sp.keep_all = 1;
+  }
+}
 static void end_steps(ms_sim* s, int begin, bool captured) {
+  s->caller = false;
   if (captured && s->home < 0) s->home = begin;
   if (s->home >= 0) keep_slot(s, s->home);
 }
@@ -1322,6 +1349,7 @@ ms_status ms_step(ms_sim* s, int64_t n) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess) return MS_ECUDA;
   const int slot0 = s->slot;
+  begin_steps(s, cs != cudaStreamCaptureStatusNone);
   if (s->graphs && !s->timing && cs == cudaStreamCaptureStatusNone) {
     const int L = cycle_steps(s);
     for (; n > 0 && s->steps % s->nsub != 0; --n) step_once(s, nullptr, n);  // to the start of a molecular cycle
@@ -1363,6 +1391,7 @@ ms_status ms_step_noalloc(ms_sim* s, int64_t n) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess) return MS_ECUDA;
   const int slot0 = s->slot;
+  begin_steps(s, cs != cudaStreamCaptureStatusNone);
   for (; n > 0; --n) step_once(s, scratch, n);
   end_steps(s, slot0, cs != cudaStreamCaptureStatusNone);
   return cudaGetLastError() == cudaSuccess ? MS_OK : MS_ECUDA;
@@ -2028,7 +2057,7 @@ ms_status ms_set_mol_batches(ms_sim* s, int32_t batches) {
       s->stream2 = nullptr;
       return MS_ECUDA;
     }
-    const size_t nev = (size_t)ms::kMaxSpecies * kMaxMolBatches + 1;  // one per run, one for the join
+    const size_t nev = (size_t)2 * ms::kMaxSpecies * kMaxMolBatches + 1;  // one per run, one for the join
     while (s->bev.size() < nev) {
       cudaEvent_t e = nullptr;
       if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {

@@ -121,6 +121,9 @@ struct SpeciesDev {
   int mrows;                // rows stored per molecule
   int par_form;             // MS_STATE_PARITY
   int all_rows;             // a loaded state populates the other rows too: process every row
+  int keep_all;             // a caller's graph can only process every row: so does every later step
+  int* order;               // full-form wavepackets: device word, the order in which the rows stand (a value of par)
+  int guard;                // a launch in a caller's graph: it runs only while the rows stand in its order
   int nmol;                 // molecules of this species
   const int* mol;           // their global ids (sorted by species, then by id)
   float2* psi;              // state [nmol][mrows][nr], s = T^{-1/2} psi
@@ -194,6 +197,10 @@ struct MolDev {
   const float* replay;      // replay drive [nwave][n][3] (lab V/m), else null
 };
 
+// A launch in a caller's graph, which outlives changes of the rows' order (a plan, a loaded state): such a graph holds
+// the kernels of both orders, and those of the other one do nothing.
+__device__ __forceinline__ bool idle_launch(const SpeciesDev& sp) { return sp.guard && *sp.order != sp.par; }
+
 // Lab-frame field (V/m) driving molecule m during the current step: the
 // replay samples, the prescribed amp x wave, or the components its cell owns
 // on the grid (E^n, before this step's E update).
@@ -240,6 +247,9 @@ void launch_bloch_observe(const SpeciesDev& sp, const MolDev& md, cudaStream_t s
 bool mol_step_supported(int nr, int nrot, int path);
 // whether the kernels of the species' plan process only the reachable rows
 bool mol_reachable_rows(const SpeciesDev& sp);
+// a species' two forms for a caller's graph, v[par], each guarded; false where its layout has no kernel for the
+// reachable rows alone, v[0] is then unguarded
+bool mol_both_orders(const SpeciesDev& sp, SpeciesDev v[2]);
 // sets par, rows and rows_g for processing the reachable rows (or every row)
 void mol_set_rows(SpeciesDev& sp, bool reachable);
 // full-form molecules: channel order -> reachable rows first (or back), in place
