@@ -267,7 +267,12 @@ ms_status ms_create(const ms_grid_desc* grid, const ms_materials_desc* materials
  * ms_set_replay_field or ms_set_detectors change what the kernels read).
  * Steps that the caller captures into a graph of its own replay from whatever
  * step the handle has reached, also between other calls, after ms_load of any
- * state and after ms_set_species_plan (with the plans of the capture). */
+ * state and after ms_set_species_plan (with the plans of the capture).  With
+ * mol_substeps > 1 capture whole molecular cycles from the start of one: which
+ * steps move the molecules is fixed in the graph.  Replays are counted on the
+ * device; ms_step_count, ms_save and the calls that read results wait for them
+ * and take up the count (ms_step's check against the prescribed samples uses
+ * the count last taken up; a step beyond them latches MS_EINVAL). */
 ms_status ms_step(ms_sim* sim, int64_t n);
 
 /* Allocation-free stepping.  The paper has no counterpart: this is a library
@@ -297,7 +302,8 @@ ms_status ms_step(ms_sim* sim, int64_t n);
  * Errors as for ms_step. */
 ms_status ms_step_noalloc(ms_sim* sim, int64_t n);
 
-/* Number of steps taken so far. */
+/* Number of steps taken so far (waits for the stream once the caller has
+ * captured steps: replays are counted on the device). */
 int64_t ms_step_count(const ms_sim* sim);
 
 /* Copy the E (which = MS_FIELD_E) or H field of one sim to host_dst,

@@ -122,3 +122,45 @@ def test_replays_after_loads(B, tmp_path, nr, jmax, nmol, path, prec, dip, plan,
         (replay or second)(n // 4)
         _close(sim, o)
     sim.close()
+
+
+@pytest.mark.parametrize("substeps,captured", [(1, 1), (1, 4), (3, 3), (3, 6)])
+def test_replays_count(B, tmp_path, substeps, captured):
+    """Capture, replay, save, load, step: the steps, the cadence, the source and the detectors' phases are those of
+    plain stepping, bit for bit, in the handle and in one that loads its checkpoint."""
+    wl = W.custom("count", 20, 12, 48, src_k=14, pulses=[[1e10, 1.5, 1e-15, 2e-16]], layer=(20, 24), n_per_sim=40,
+                  species=[W.species_config0(jmax=1)], seed=3, nsteps=100, mol_substeps=substeps)
+    planes, om = [12, 40], np.linspace(1.0, 3.0, 2) / 6.582119569e-16
+    lead, reps, tail = 2 * substeps, 5, 7
+
+    def make(graphs):
+        s = B.Simulation(wl, step_graphs=graphs)
+        s.set_detectors(planes, om)
+        return s
+
+    def out(s):
+        r = [s.populations(), s.dipoles(), s.fields(B.MS_FIELD_E), s.fields(B.MS_FIELD_H)]
+        r += [s.dft(p, 0, c, f) for p in range(2) for c in range(4) for f in range(2)]
+        s.close()
+        return r
+
+    a = make(B.MS_GRAPHS_OFF)
+    a.step(lead + reps * captured + tail)
+    b = make(B.MS_GRAPHS_AUTO)
+    b.step(lead)
+    replay = _capture(b, captured)
+    assert b.steps == lead                 # capturing takes no step
+    replay(reps)
+    p = str(tmp_path / "c.ck")
+    b.save(p)
+    assert b.steps == lead + reps * captured
+    c = make(B.MS_GRAPHS_AUTO)
+    c.load(p)
+    assert c.steps == lead + reps * captured
+    b.step(tail)
+    c.step(tail)
+    assert a.steps == b.steps == c.steps
+    ref = out(a)
+    for s in (b, c):
+        for x, y in zip(ref, out(s)):
+            assert np.array_equal(x, y)
