@@ -424,12 +424,10 @@ __global__ void __launch_bounds__(FFTShape<NR>::THREADS, FUSED ? 2 : (MAXR <= 4 
 // outside the basis are zero and their reads land on finite data: kTriGuard
 // zero rows precede each buffer, and a missing run points at them.
 // ----------------------------------------------------------------------------
-// The angular tables of every translation unit's copy.
+// Fills the copies of the angular tables of the kernels that read them.
 cudaError_t upload_triplet_tables(const CouplEntry* dip) {
-  cudaError_t e = upload_triplet_tables_local(dip);
-  if (e == cudaSuccess) e = upload_triplet_tables_tile(dip);
-  if (e != cudaSuccess) return e;
-  return upload_triplet_tables_pair(dip);
+  const cudaError_t e = upload_triplet_tables_tile(dip);
+  return e == cudaSuccess ? upload_triplet_tables_pair(dip) : e;
 }
 
 // Diagnostic of the bounded wait: one CTA waits on a barrier that nothing

@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
   constexpr int NROT = D::NROT, NG = D::NG;
   if (idle_launch(sp)) return;
   __shared__ float2 Ys[NROT][32];
-  __shared__ int s_vt[NROT + 3];  // row -> its shell's row of the phase table (and three past the end)
+  __shared__ int s_vt[NROT];  // row -> its shell's row of the phase table
   __shared__ float s_fin[8], s_fin_lo[2];  // P_g, P_e, Re(S+ + S-), Im(S+ - S-), 2 Re Z, absorbed (2), rounding residuals
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int lm = blockIdx.x, m = sp.mol[lm], NR = sp.nr;
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kColThreads, 4) mol_rspace_col_kernel(SpeciesD
   // what the closing threads add to: the previous dipole, the absorbed norm so far
   const double old = t < 3 ? md.mu[3 * (long long)m + t]
                            : (t == 5 || t == 6 ? md.absorbed[2 * (long long)m + (t - 5)] : 0.0);
-  for (int q = t; q < NROT + 3; q += kColThreads) {
+  for (int q = t; q < NROT; q += kColThreads) {
     int j = q >= NG, r = q - (j ? NG : 0);
     while (r >= 2 * j + 1 && j + 2 <= J) {
       r -= 2 * j + 1;

@@ -10,7 +10,7 @@
 #include <cstddef>
 #include <type_traits>
 
-#include "mol_common.cuh"
+#include "mol_tri.cuh"
 
 namespace ms {
 namespace {
