@@ -21,6 +21,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -79,17 +80,33 @@ def _peaks():
     return 6800.0, "recipe fallback 6.8 TB/s (of fallback)"
 
 
+def _source_digest(path: str) -> str:
+    """sha256 over a kernel's source file and every file of the repository that it includes, in the order met."""
+    seen, todo = [], [path]
+    while todo:
+        f = os.path.normpath(todo.pop(0))
+        if f in seen:
+            continue
+        seen.append(f)
+        for name in re.findall(r'^\s*#include\s+"([^"]+)"', open(f).read(), re.M):
+            near = [os.path.join(d, name) for d in (os.path.dirname(f), os.path.join(ROOT, "include"))]
+            todo += [p for p in near if os.path.exists(p)][:1]
+    h = hashlib.sha256()
+    for f in seen:
+        h.update(open(f, "rb").read())
+    return h.hexdigest()
+
+
 def _kernel_traffic(kernel: str):
     """DRAM bytes per molecule from the committed ncu summary, valid only while
-    the kernel's source is unchanged (sha256 of the .cu file)."""
+    the kernel's source and what it includes are unchanged (_source_digest)."""
     path = os.path.join(ROOT, "profiles", "traffic.txt")
     if not os.path.exists(path):
         return None
     for line in open(path):
         f = line.split()
         if len(f) >= 4 and not line.startswith("#") and f[0] == kernel:
-            src = os.path.join(ROOT, "paper_2209_04487_gb300", "csrc", f[1])
-            sha = hashlib.sha256(open(src, "rb").read()).hexdigest()
+            sha = _source_digest(os.path.join(ROOT, "paper_2209_04487_gb300", "csrc", f[1]))
             return float(f[3]) if sha == f[2] else None
     return None
 
