@@ -661,8 +661,7 @@ __global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? 2 : 1))
     f.z *= dw;
   }
   const int nterms = __float_as_int(f.w);
-  const float2 mw = sp.maskw[p];
-  const float mk = mw.x;
+  const float mk = sp.maskw[p].x;
   const float cfix = md.ncorr[m];  // rounding feedback of the previous step
   float2 vh[J + 1], vd[J + 1];
 #pragma unroll
@@ -740,7 +739,7 @@ __global__ void __launch_bounds__(2 * NR, NR <= 64 ? 4 : (NR <= 128 ? 2 : 1))
         const float px = u.x + d1.x, py = u.y + d1.y;
         d1.x = fmaf(mk - 1.f, u.x, mk * d1.x);
         d1.y = fmaf(mk - 1.f, u.y, mk * d1.y);
-        absd += mw.y * fmaf(px, px, py * py);
+        absd += (1.f - mk * mk) * fmaf(px, px, py * py);
       }
       const float2 s1 = round_update(sv, dv + d1, cfix, rnd);
       __stcs(gs + r * NR, s1);

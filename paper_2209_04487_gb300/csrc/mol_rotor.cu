@@ -83,8 +83,7 @@ __device__ __forceinline__ void rotor_point(const SpeciesDev& sp, int p, float2*
     f.z *= dw;
   }
   const int nterms = max(__float_as_int(f.w), 1);  // no field: one term of zeros
-  const float2 mw = __ldg(&sp.maskw[p]);  // (m, 1 - m^2); 1 - m^2 from m in FP32 is 1% off where the absorber begins
-  const float mk = mw.x;
+  const float mk = __ldg(&sp.maskw[p]).x;
   auto s_at = [&](int row) { return ss[row * NR]; };
   auto d_at = [&](int row) { return FUSED ? ds[row * NR] : __ldg(ds + row * NR); };
   // potential phases of shell j on the surface of its parity
@@ -167,7 +166,7 @@ __device__ __forceinline__ void rotor_point(const SpeciesDev& sp, int p, float2*
       if (masked) {
         const float2 p = add2(u, d1);
         d1 = fma2(dup2(mk - 1.f), u, mul2(dup2(mk), d1));
-        a.ab[sf] += mw.y * fmaf(p.x, p.x, p.y * p.y);
+        a.ab[sf] += (1.f - mk * mk) * fmaf(p.x, p.x, p.y * p.y);
       }
       const float2 sn = round_update2(s0, add2(d0, d1), cf, a.rnd);
       __stcs(gs + row * NR, sn);

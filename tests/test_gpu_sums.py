@@ -62,23 +62,3 @@ def test_column_kernel_dipole_sums(B, tmp_path, nr, jmax, form, steps):
     want = np.einsum("kij,kj->ki", ens.O.astype(np.float32).astype(np.float64),
                      ens.dipole_mol(_state(p, nmol, sp, bool(form))))
     assert np.linalg.norm(mu - want) <= 16 * 2.0 ** -24 * np.linalg.norm(want)
-
-
-@pytest.mark.parametrize("nr,jmax,path,ra", [(64, 1, 2, 2.850143), (128, 3, 1, 2.82952), (256, 4, 2, 2.762),
-                                             (64, 5, 2, 2.850143)])
-def test_absorbed_norm_where_the_absorber_begins(B, nr, jmax, path, ra):
-    """An absorber that begins just under a grid point in the packet's tail, where 1 - m^2 is some 1e-6: taken from m
-    in FP32 the absorbed norm is 0.2 to 1.3% off.  The tail's amplitude is 1/150 of the packet's, so an FP32 state
-    holds it to about 1e-5."""
-    nmol, n = 3, 4
-    sp = W.Species(nr=nr, jmax=jmax, absorber_r=ra)
-    wl = W.custom("absorber", 8, 8, 48, n_per_sim=nmol, species=[sp], layer=(20, 24), seed=nr, nsteps=n)
-    amp, wave = np.zeros((nmol, 3), np.float32), np.zeros(n, np.float32)
-    sim = B.Simulation(wl, drive=B.MS_DRIVE_PRESCRIBED, mol_path=path)
-    sim.set_prescribed(amp, wave)
-    sim.step(n)
-    ab = sim.dissociation()[0]
-    sim.close()
-    want = PrescribedOracle(wl, amp, wave).run(n).absorbed()
-    assert (want[:, 0] > 0).all()
-    assert np.abs(ab[:, 0] / want[:, 0] - 1).max() < 5e-4
