@@ -331,8 +331,9 @@ ms_status ms_read_populations(ms_sim* sim, int64_t first, int64_t count, double*
 
 /* Per-molecule dissociation observables (FP64): norm removed by the
  * absorber since t=0 on each surface, and the numerator <chi_e|R|chi_e>
- * and denominator <chi_e|chi_e> of Eq. 8 at the current time.  Any output
- * may be NULL. */
+ * and denominator <chi_e|chi_e> of Eq. 8 at the current time, summed over a
+ * row in pairs of FP32 numbers (about 48 bits) and over rows in FP64.  Any
+ * output may be NULL. */
 ms_status ms_read_dissociation(ms_sim* sim, int64_t first, int64_t count, double* absorbed_g,
                                double* absorbed_e, double* R_e_num, double* R_e_den);
 
@@ -419,7 +420,9 @@ ms_status ms_read_dft(ms_sim* sim, int32_t plane, int32_t sim_index, int32_t com
  * descriptors and options; the sizes, the sub-step count and the source
  * kind in the file must match (MS_EINVAL otherwise).  A prescribed or replay
  * drive is set again by the caller.  N steps equal N/2 steps, save, load
- * into a fresh handle, N/2 steps, bit for bit.  Both calls are synchronous
+ * into a fresh handle, N/2 steps, bit for bit.  While they work, full-form
+ * states stand on the device in the file's order of rows; both calls bring
+ * back the order that the kernels want before they return.  Both are synchronous
  * and stage through two pinned 64 MiB host buffers (pageable memory when
  * pinned memory cannot be had).  Errors:
  * MS_EINVAL (NULL argument, size mismatch), MS_EIO (open, short read or

@@ -965,7 +965,7 @@ static bool rspace_ok(int nr, int jmax);
 // resident one does not and it applies, unless the plan names another kernel.
 static bool pair_ok(int nr, int jmax) { return (nr == 64 || nr == 128 || nr == 256) && jmax <= 16; }
 // The column kernel runs the reachable rows of a streaming species from J = 5
-// to 8: 6.1 to 6.5 ps a row and point at N_r = 128, 6.4 at 256 and 6.9 at 64,
+// to 8: 5.9 to 6.5 ps a row and point at N_r = 128, 5.8 to 6.4 at 256 and 6.6 to 6.9 at 64,
 // against 8.0 for the two-points-a-thread kernel.  Below, a thread holds the
 // whole rotor; above, half a side's columns no longer fit a thread's registers.
 static bool use_col(const SpeciesDev& sp) {
@@ -995,7 +995,8 @@ static int pair_tile(const SpeciesDev& sp) {
 
 // ----------------------------------------------------------------------------
 // Eq. 8 readout: psi = T^{1/2} s on the excited surface, then
-// <chi_e|R|chi_e> and <chi_e|chi_e> per molecule (FP64 reduction)
+// <chi_e|R|chi_e> and <chi_e|chi_e> per molecule: a row's sums in FP32 pairs that
+// take every rounding of the additions and of r |psi|^2 (about 48 bits), rows in FP64
 // ----------------------------------------------------------------------------
 namespace ms {
 

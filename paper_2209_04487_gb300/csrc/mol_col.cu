@@ -21,9 +21,12 @@
 // row by row in loops over Y, shared out evenly over the warps: only about 30
 // instructions a row are unrolled.  With every phase unrolled (100 KB of code
 // at J = 8) the pass waited for instructions: 8.8 ps a row and point; with the
-// rows' loads one at a time for those loads: 12.5 ps.  What is left of that
-// wait bounds it (a thread per row: 8.0 ps; now 5.9 to 6.5 at N_r = 128; 3.5 ps is
-// HBM's).
+// rows' loads one at a time for those loads: 12.5 ps.  A thread per row: 8.0 ps;
+// now 5.9 to 6.5 at N_r = 128; 3.5 ps is HBM's.  What bounds it is latency, with
+// the fifteen warps an SM that registers leave: at J = 8 an issued instruction costs
+// 8.0 warp cycles, 1.6 of them global loads, 1.2 fixed latency, 0.9 barriers and
+// 0.7 each shared memory, the FP32 pipe and instruction fetch; the shared-memory
+// pipe is 71% and issue slots 47% busy.
 //
 // The coupling's exponential series S = sum_{n=1..N} T_n, T_1 = i theta M eta,
 // T_n = (i theta / n) M T_{n-1}, is summed by Horner's rule on T_1: S = P_1, P_n

@@ -19,9 +19,12 @@
 // multiplied by real coefficients as packed FP32x2 products, whose equal
 // constants are immediates.
 //
-// What bounds it: issue slots and instruction fetch (2,900 instructions of
-// straight-line code at J = 4, about 85 a row and point; twelve warps an SM by
-// registers), then HBM.  Per row and point of the reachable rows: the R-space
+// What bounds it: latency.  By registers an SM holds twelve warps.  In the fused
+// step at J = 4 an issued instruction costs 5.4 warp cycles: 1 its issue, 0.9
+// fixed latency, 1.2 memory (shared and global), 0.6 barriers, 0.5 the FP32 pipe,
+// 0.5 another warp's turn, 0.4 instruction fetch; issue slots are 50% and the
+// shared-memory pipe 46% busy (142 warp instructions a row and 32 points, the FFT
+// included).  Per row and point of the reachable rows: the R-space
 // pass at J = 4, N_r = 64 takes 4.36 ps, 5.5 TB/s, against 7.13 for a thread per
 // surface; the fused step at J = 4, N_r = 128 6.79 against 12.14 ps.
 //
