@@ -1302,9 +1302,7 @@ static void keep_slot(ms_sim* s, int slot) {
   s->slot = slot;
 }
 
-// The end of a call's steps.  A call that the caller captures ends on the counter
-// slot it began with, and so does every call after it: the caller's graph can be
-// replayed, by itself and between other calls.
+// The start of a call's steps, which may go into a graph of the caller's.
 static void begin_steps(ms_sim* s, bool captured) {
   s->caller = captured;
   if (!captured) return;
@@ -1313,6 +1311,10 @@ static void begin_steps(ms_sim* s, bool captured) {
     if (sp.order && !ms::mol_both_orders(sp, v)) sp.keep_all = 1;
   }
 }
+
+// The end of a call's steps.  A call that the caller captures ends on the counter
+// slot it began with, and so does every call after it: the caller's graph can be
+// replayed, by itself and between other calls.
 static void end_steps(ms_sim* s, int begin, bool captured) {
   s->caller = false;
   if (captured && s->home < 0) s->home = begin;
